@@ -53,7 +53,10 @@ typedef enum { MELT_WIN_HANN_PERIODIC = 0, MELT_WIN_HANN_SYMMETRIC = 1 } melt_wi
 /*
  * GEMM operand formats (the paper runs FP32/TF32 only; the reduced forms are
  * this library's).  All accumulate in FP32 and take FP32 waveforms.
- *   MELT_FP32    FP32 samples x FP32 basis on CUDA cores (FFMA).
+ *   MELT_FP32    FP32 samples x FP32 basis, each split exactly into three BF16
+ *                parts, the six leading products on tcgen05 tensor cores, sums
+ *                of at most four K-steps added in FP32 (CUDA cores, FFMA, for
+ *                hops too short for that layout).
  *   MELT_BF16    BF16 samples x BF16 basis on tcgen05 tensor cores.
  *   MELT_BF16X3  two-term BF16 splits of both operands, three products
  *                (hi*hi + hi*lo + lo*hi) on tcgen05 tensor cores.
@@ -163,7 +166,7 @@ typedef struct {
 } melt_plan;
 
 /* melt_plan_get - the layout the next forward will use (host struct out).
- * MELT_ERR_UNSUPPORTED for an FP32 (CUDA-core) basis, which has no layout. */
+ * MELT_ERR_UNSUPPORTED for an FP32 basis, which has no layout to choose. */
 melt_status melt_plan_get(const melt_basis* basis, melt_plan* plan);
 
 /* melt_plan_set - force a layout (plan NULL = back to the default choice).

@@ -17,6 +17,7 @@
 
 #include "melt_diag.h"
 #include "melt_internal.h"
+#include "melt_slab.h"
 #include "melt_tc.h"
 #include "sm100_ptx.cuh"
 
@@ -59,6 +60,7 @@ struct melt_basis {
   float* d_dct = nullptr;      // [K][M]
   int* d_err = nullptr;        // latched kernel errors
   TcBasis tc;                  // tensor-core operand images (BF16/FP8 forms)
+  SlabBasis slab;              // FP32 form: three-part split operands (no image: the CUDA-core kernel runs)
   Staging staging[kStagingSlots];
   int next_slot = 0;
   std::vector<TileDesc> plan;  // host scratch for planning
@@ -93,6 +95,7 @@ void free_basis(melt_basis* b) {
   cudaFree(b->d_err);
   cudaFree(b->d_fb);
   tc_free(&b->tc);
+  slab_free(&b->slab);
   for (auto& s : b->staging) {
     if (s.done) cudaEventSynchronize(s.done), cudaEventDestroy(s.done);
     cudaFreeHost(s.host);
@@ -193,6 +196,8 @@ melt_status create_common(double sr, int n_fft, int hop, const double* freqs, in
     TcConfig c{n_fft, hop, n_freqs, precision, n_mfcc, stft_bands};
     st = tc_build(&b->tc, c, b->w64.data());
   }
+  if (st == MELT_OK && precision == MELT_FP32)
+    st = slab_build(&b->slab, n_fft, hop, n_freqs, n_mfcc, 3, b->w64.data());
   if (st == MELT_OK) {
     cudaError_t e = melt::dev_alloc(&b->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, sizeof(int));
@@ -220,6 +225,30 @@ int64_t frames_of(const melt_basis* b, int64_t len) {
 // own rows), so the order changes no result.
 void order_longest_first(TileDesc* t, long long n) {
   std::stable_sort(t, t + n, [](const TileDesc& a, const TileDesc& b) { return a.n_frames > b.n_frames; });
+}
+
+// The FP32 form over n_tiles device descriptors.  The tensor-core kernel with
+// three-part split operands runs wherever its rings fit shared memory (64 x 30 s,
+// N 400, 80 bins: 99 us against 508 us on the CUDA cores; 8 x 1 s: 13.5 against
+// 52 us; one 160 s clip, N 1200, 128 bins, 40 MFCCs: 59 against 421 us).  Hops
+// so short that a slab of all Z rows does not fit twice, and the raw
+// projections (mode 1), run on the CUDA cores.
+cudaError_t launch_fp32(melt_basis* b, const float* wave, const TileDesc* tiles, int n_tiles, float* out, int mode,
+                        cudaStream_t stream) {
+  if (mode == 0 && b->slab.d_img) {
+    SlabLaunch L;
+    L.wave = wave; L.tiles = tiles; L.n_tiles = n_tiles; L.out = out;
+    L.dct = b->d_dct; L.w32 = b->d_w32; L.mp = b->mp;
+    L.n_mfcc = b->n_mfcc; L.eps = (float)b->eps; L.err = b->d_err; L.sm_count = b->sm_count;
+    return slab_launch(&b->slab, L, stream);
+  }
+  SimtParams p;
+  p.wave = wave; p.tiles = tiles; p.n_tiles = n_tiles;
+  p.w32 = b->d_w32; p.dct = b->d_dct; p.out = out;
+  p.n_fft = b->n_fft; p.hop = b->hop; p.n_mels = b->n_mels; p.mp = b->mp;
+  p.n_mfcc = b->n_mfcc; p.n_out = b->n_mfcc ? b->n_mfcc : b->n_mels;
+  p.eps = (float)b->eps; p.mode = mode;
+  return launch_simt(p, b->mj, b->sm_count, stream);
 }
 
 // Build the tile list of a batch; returns MELT_ERR_ARG on bad offsets/lengths.
@@ -313,13 +342,7 @@ melt_status forward_impl(melt_basis* b, const float* wave, const int64_t* offset
   cudaError_t e;
   bool fused = false;  // the kernel applied the correction itself
   if (b->precision == MELT_FP32 || mode == 1) {
-    SimtParams p;
-    p.wave = wave; p.tiles = slot->dev; p.n_tiles = n_tiles;
-    p.w32 = b->d_w32; p.dct = b->d_dct; p.out = out;
-    p.n_fft = b->n_fft; p.hop = b->hop; p.n_mels = b->n_mels; p.mp = b->mp;
-    p.n_mfcc = b->n_mfcc; p.n_out = b->n_mfcc ? b->n_mfcc : b->n_mels;
-    p.eps = (float)b->eps; p.mode = mode;
-    e = launch_simt(p, b->mj, b->sm_count, stream);
+    e = launch_fp32(b, wave, slot->dev, n_tiles, out, mode, stream);
   } else {
     TcLaunch L;
     L.wave = wave; L.tiles = slot->dev; L.n_tiles = n_tiles; L.out = out;
@@ -400,13 +423,7 @@ melt_status launch_forward_tiles(melt_basis* b, const float* wave, const TileDes
   cudaError_t e;
   bool fused = false;
   if (b->precision == MELT_FP32) {
-    SimtParams p;
-    p.wave = wave; p.tiles = d_tiles; p.n_tiles = n_tiles;
-    p.w32 = b->d_w32; p.dct = b->d_dct; p.out = out;
-    p.n_fft = b->n_fft; p.hop = b->hop; p.n_mels = b->n_mels; p.mp = b->mp;
-    p.n_mfcc = b->n_mfcc; p.n_out = b->n_mfcc ? b->n_mfcc : b->n_mels;
-    p.eps = (float)b->eps; p.mode = 0;
-    e = launch_simt(p, b->mj, b->sm_count, stream);
+    e = launch_fp32(b, wave, d_tiles, n_tiles, out, 0, stream);
   } else {
     TcLaunch L;
     L.wave = wave; L.tiles = d_tiles; L.n_tiles = n_tiles; L.out = out;

@@ -1,4 +1,6 @@
-// Plain FP32 MelT on CUDA cores (FFMA, FP32 accumulate).
+// Plain FP32 MelT on CUDA cores (FFMA, FP32 accumulate): the raw projections
+// (melt_forward_components), and the FP32 form at hops so short that the
+// tensor-core kernel's slabs do not fit shared memory.
 //
 // Computes the projection of Sec. III-A, Eq. 6 ([R | I] = X [W_r; W_i]^T)
 // with implicit framing: frame f of a tile is read straight from the packed

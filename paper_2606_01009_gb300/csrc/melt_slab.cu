@@ -1,0 +1,205 @@
+// Host side of the slab kernel: the operand image, the shared-memory plan and
+// the launch (device code in melt_slab_kernel.cuh).
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
+#include "melt_slab_kernel.cuh"
+
+namespace melt {
+
+using namespace slab;
+
+namespace {
+
+constexpr uint32_t kSmemMax = 227 * 1024;
+
+uint32_t up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
+
+// BF16 (round to nearest even) nearest to v; *v becomes the exact remainder.
+uint16_t take_bf16(double* v) {
+  const float f = (float)*v;
+  uint32_t bits;
+  std::memcpy(&bits, &f, 4);
+  bits = (bits + 0x7fffu + ((bits >> 16) & 1u)) & 0xffff0000u;
+  float h;
+  std::memcpy(&h, &bits, 4);
+  *v -= h;
+  return (uint16_t)(bits >> 16);
+}
+
+// MFCC: the DCT matrix and two buffers of eight coefficients of every row.
+uint32_t mfcc_bytes(const SlabParams& p, int n_mfcc) {
+  return n_mfcc > 0 ? up(4u * n_mfcc * 8u * p.groups, 128) + 2u * 8u * kF * 4u : 0u;
+}
+
+// Geometry and shared-memory plan; false where two slots of either ring do not fit.
+bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
+  const int P = sb->parts;
+  p.N = sb->n_fft;
+  p.H = sb->hop;
+  p.M = sb->n_mels;
+  p.J = sb->J;
+  p.n_slab = sb->n_slab;
+  p.ksteps = sb->ksteps;
+  p.groups = sb->groups;
+  p.zrows = kF + p.J - 1;
+  p.n_last = p.N - (p.J - 1) * p.H;
+  // a chunk's truncations grow with its K-steps, its drains with their number:
+  // at most 4 K-steps, and all slices of a slab where there are fewer
+  p.kps = std::min(p.J, 4);
+  p.step_bytes = (uint32_t)p.groups * P * 256u;
+  int zr = p.zrows;
+  while ((zr & 7) != 4) ++zr;  // rows = 4 mod 8: the two core columns of a converter store fall on other banks
+  p.lbo_a = (uint32_t)zr * 16u;
+  p.a_part = 2 * p.lbo_a;
+  p.a_slot = P * p.a_part;
+  const int least = (p.groups + kBlockBins / 8 - 1) / (kBlockBins / 8);  // blocks, and groups of the widest one
+  const int wbg = 2 * ((p.groups / 2 + least - 1) / least);
+  p.b_slot = (uint32_t)wbg * P * 256u * p.kps;
+  const uint32_t fixed = up(8u * SlabBars(kMaxSlots, kMaxSlots).total, 128) + 128u +
+                         mfcc_bytes(p, n_mfcc) + kCvtWarps * kStageBytes + 128u;
+  if (fixed > kSmemMax) return false;
+  const uint32_t room = kSmemMax - fixed;
+  // six A slots (one per converter warp) where four basis slots fit beside them
+  for (int need = 4; need >= 2; need -= 2)
+    for (int na = 6; na >= 2; --na) {
+      const uint32_t a = up(p.a_slot, 128) * na;
+      if (a >= room) continue;
+      const int nb = std::min<int>(kMaxSlots, (int)((room - a) / up(p.b_slot, 128)));
+      if (nb < need || (need == 4 && na < 3)) continue;
+      p.NA = na;
+      p.NB = nb;
+      p.ncv = std::min(na, kCvtWarps);
+      p.a_slot = up(p.a_slot, 128);
+      p.b_slot = up(p.b_slot, 128);
+      p.off_a = 0;
+      p.off_b = p.a_slot * na;
+      p.off_st = p.off_b + p.b_slot * nb;
+      p.off_bar = p.off_st + kCvtWarps * kStageBytes;
+      p.off_misc = p.off_bar + up(8u * SlabBars(na, nb).total, 128);
+      p.off_dct = p.off_misc + 128u;
+      p.off_part = p.off_dct + up(4u * n_mfcc * 8u * p.groups, 128);
+      return true;
+    }
+  return false;
+}
+
+uint32_t smem_bytes(const SlabParams& p, int n_mfcc) { return p.off_dct + mfcc_bytes(p, n_mfcc) + 128u; }
+
+}  // namespace
+
+melt_status slab_build(SlabBasis* sb, int n_fft, int hop, int n_mels, int n_mfcc, int parts, const double* w64) {
+  sb->parts = parts;
+  sb->n_fft = n_fft;
+  sb->hop = hop;
+  sb->n_mels = n_mels;
+  sb->J = (n_fft + hop - 1) / hop;
+  sb->n_slab = (hop + 15) / 16;
+  sb->groups = (n_mels + 15) / 16 * 2;
+  const int n_last = n_fft - (sb->J - 1) * hop;
+  sb->ksteps = sb->n_slab * (sb->J - 1) + (n_last + 15) / 16;
+  SlabParams p;
+  std::memset(&p, 0, sizeof(p));
+  if (!plan(sb, n_mfcc, p)) return MELT_OK;
+  const size_t half = (size_t)sb->ksteps * p.step_bytes;
+  std::vector<uint16_t> img(half);  // two halves of half / 2 values each
+  for (int h = 0; h < 2; ++h) {
+    uint16_t* step = img.data() + (size_t)h * (half / 2);
+    for (int kk = 0; kk < sb->n_slab; ++kk) {
+      const int js = 16 * kk < n_last ? sb->J : sb->J - 1;
+      for (int j = 0; j < js; ++j, step += p.step_bytes / 2)
+        for (int m = 0; m < n_mels; ++m) {
+          const double* w = w64 + ((size_t)h * n_mels + m) * n_fft;
+          uint16_t* grp = step + (size_t)(m >> 3) * parts * 128 + (m & 7) * 8;
+          for (int e = 0; e < 16; ++e) {
+            const int r = 16 * kk + e, n = j * hop + r;
+            double v = r < hop && n < n_fft ? w[n] : 0.0;
+            for (int t = 0; t < parts; ++t) grp[t * 128 + (e >> 3) * 64 + (e & 7)] = take_bf16(&v);
+          }
+        }
+    }
+  }
+  if (melt::dev_alloc(&sb->d_img, 2 * half) != cudaSuccess) return MELT_ERR_OOM;
+  if (cudaMemcpy(sb->d_img, img.data(), 2 * half, cudaMemcpyHostToDevice) != cudaSuccess) return MELT_ERR_CUDA;
+  return MELT_OK;
+}
+
+void slab_free(SlabBasis* sb) {
+  cudaFree(sb->d_img);
+  sb->d_img = nullptr;
+}
+
+cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream) {
+  SlabParams p;
+  std::memset(&p, 0, sizeof(p));
+  if (!sb->d_img || !plan(sb, L.n_mfcc, p)) return cudaErrorInvalidConfiguration;
+  p.wave = L.wave;
+  p.tiles = L.tiles;
+  p.img = static_cast<const uint8_t*>(sb->d_img);
+  p.dct = L.dct;
+  p.w32 = L.w32;
+  p.mp = L.mp;
+  p.out = L.out;
+  p.err = L.err;
+  p.eps = L.eps;
+  p.n_tiles = L.n_tiles;
+  p.n_pairs = (L.n_tiles + 1) / 2;
+  p.n_mfcc = L.n_mfcc;
+  p.n_out = L.n_mfcc ? L.n_mfcc : sb->n_mels;
+  void (*fn)(SlabParams) = L.n_mfcc ? melt_slab_kernel<3, true> : melt_slab_kernel<3, false>;
+  const int smem = (int)smem_bytes(p, L.n_mfcc);
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  if (sb->clusters < 0 || sb->clusters_smem != smem) {
+    // (always the same limit, so that bases of different sizes do not lower each other's)
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = dim3(2 * (L.sm_count / 2), 1, 1);
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
+    if (e != cudaSuccess) return e;
+    sb->clusters = n;
+    sb->clusters_smem = smem;
+  }
+  const int C = sb->clusters;
+  if (C < 1) return cudaErrorInvalidConfiguration;
+  // Blocks of Mel bins: as few as fit the epilogue's registers, or more where
+  // the pairs leave clusters idle (a block below about 44 bins takes no less
+  // time: reading A from shared memory bounds its MMAs).  MFCC sums over all
+  // bins, so its blocks stay in one cluster.
+  const int pairs16 = p.groups / 2;
+  int best = (pairs16 + kBlockBins / 16 - 1) / (kBlockBins / 16);
+  if (L.n_mfcc == 0) {
+    long long cost = -1;
+    for (int nb = best, first = best; nb <= std::max(first, (pairs16 + 1) / 2); ++nb) {
+      const int w = (pairs16 + nb - 1) / nb, n = (pairs16 + w - 1) / w;
+      const long long rounds = ((long long)p.n_pairs * n + C - 1) / C;
+      const long long t = rounds * (std::max(16 * w, 44) + 6);
+      if (cost < 0 || t < cost) {
+        cost = t;
+        best = nb;
+      }
+    }
+  }
+  p.wbg = 2 * ((pairs16 + best - 1) / best);
+  p.nblk = (p.groups + p.wbg - 1) / p.wbg;
+  p.inner = L.n_mfcc ? p.nblk : 1;
+  p.n_units = L.n_mfcc ? p.n_pairs : p.n_pairs * p.nblk;
+  cfg.gridDim = dim3(2 * std::min(p.n_units, C), 1, 1);
+  return cudaLaunchKernelEx(&cfg, fn, p);
+}
+
+}  // namespace melt

@@ -1,0 +1,39 @@
+// Host interface of the slab kernel (melt_slab_kernel.cuh): the projection in
+// CTA pairs with both operands streamed through shared memory in K slabs.
+#pragma once
+
+#include "melt_internal.h"
+
+namespace melt {
+
+// Device-resident operands of one basis for the slab kernel.
+struct SlabBasis {
+  int parts = 0;                       // BF16 parts per operand: 3 for the FP32 form
+  int n_fft = 0, hop = 0, n_mels = 0;
+  int J = 0, n_slab = 0, ksteps = 0;   // polyphase slices, 16-sample slabs, MMA K-steps
+  int groups = 0;                      // groups of 8 Mel bins
+  void* d_img = nullptr;               // two halves (W_r rows, W_i rows) of K-step blocks
+  int clusters = -1, clusters_smem = 0;  // co-resident clusters of the kernel at that shared-memory size
+};
+
+struct SlabLaunch {
+  const float* wave;
+  const TileDesc* tiles;
+  int n_tiles;
+  float* out;
+  const float* dct;    // [n_mfcc][n_mels] or nullptr
+  const float* w32;    // [n_fft][2 mp] FP32 basis (the tiles the split operands cannot hold)
+  int mp;
+  int n_mfcc;
+  float eps;
+  int* err;
+  int sm_count;
+};
+
+// Builds the operand image for `parts` BF16 parts; leaves d_img null (MELT_OK)
+// where the kernel's shared-memory layout does not fit the geometry.
+melt_status slab_build(SlabBasis* sb, int n_fft, int hop, int n_mels, int n_mfcc, int parts, const double* w64);
+void slab_free(SlabBasis* sb);
+cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream);
+
+}  // namespace melt
