@@ -14,19 +14,21 @@
 // small to be worth tensor-core tiles, and FP32 keeps the gradients close
 // enough to the FP64 definition to check them element by element.
 //
-// Kernels of one step (B = batch rows gathered through `rows`):
-//   1. H = Xh W1^T + b1, A = GELU(H)                  [B x Hd]
-//   2. Y = X + A W2^T + b2, dY = 2 (Y - T) / (B M), loss partial sums
-//   3. dH = (dY W2) * GELU'(H)                        [B x Hd]
-//   4. dW2 = dY^T A, dW1 = dH^T Xh                    (sums over the batch)
-//   5. db1, db2 = column sums of dH, dY
-//   6. AdamW over the packed parameter vector
+// Kernels of one step (B = batch rows gathered through `rows`), three launches:
+//   rows_kernel   8 rows per block: Xh, H = Xh W1^T + b1, A = GELU(H),
+//                 Y = X + A W2^T + b2, dY = 2 (Y - T) / (B M), the loss, and
+//                 dH = (dY W2) * GELU'(H); Xh, A, dY and dH go to memory
+//   wgrad_kernel  dW1 = dH^T Xh, dW2 = dY^T A and the column sums db1, db2 over
+//                 a slice of the batch, partial sums to memory
+//   reduce_kernel sums the slices in order; in a training step also AdamW
+// Each may start while the one before drains (programmatic dependent launch).
+//
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
-#include <type_traits>
 #include <vector>
 
 #include <cuda_bf16.h>
@@ -35,7 +37,7 @@
 
 namespace {
 
-constexpr int kBM = 64, kBN = 64, kBK = 16, kGemmThreads = 256;
+constexpr int kMaxSmem = 227 * 1024;
 constexpr int kMaxIn = 128;       // M (bands) limit of the fused apply kernel
 constexpr int kApplyFrames = 64;  // frames per CTA of the fused apply kernel
 constexpr int kApplyChunk = 64;   // hidden units per chunk of the fused apply kernel
@@ -49,168 +51,477 @@ __device__ __forceinline__ float gelu_grad_f(float h) {
          h * 0.39894228040143268f * expf(-0.5f * h * h);
 }
 
-// ---- operand loaders: (i, k) -> element of op(A) [rows i, inner k]
-struct LoadRowK {            // p[i * ld + k]
-  const float* p;
-  long long ld;
-  static constexpr bool kMajorK = true;
-  __device__ float operator()(long long i, long long k) const { return p[i * ld + k]; }
-};
-struct LoadColK {            // p[k * ld + i]
-  const float* p;
-  long long ld;
-  static constexpr bool kMajorK = false;
-  __device__ float operator()(long long i, long long k) const { return p[k * ld + i]; }
-};
-struct LoadStdX {            // standardised x of gathered row i, band k
-  const float* x;
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+__device__ __forceinline__ void copy16(float* dst, const float* src, int bytes) {  // zeros past `bytes`
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void copy4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+// ---- rows_kernel: forward and backward of 8 rows per block.
+//
+// Bound: a step of 1024 rows at 80 -> 256 -> 80 is 0.1 GFMA of FP32, about 3 us
+// of the chip's FFMAs, so what counts is to have every SM at work and few
+// launches.  8 rows per block make 128 blocks; the block holds UC hidden units
+// of both weight matrices in shared memory (all of them up to 256 at 80 bands:
+// one copy of 160 KB from L2, kept for the block's further rows), and its
+// three products read shared memory about as long as they multiply:
+//   H   thread = unit, its rows: one 16-byte read of W1 and one broadcast per
+//       row for 4 FFMAs a row (W1 rows an odd number of 16-byte steps apart)
+//   Y   warp = a run of units, lanes = bands: per four units one 16-byte read
+//       per band and 8 broadcasts; the 8 warps' sums meet in shared memory
+//   dH  thread = unit: one read of W2 and broadcasts of dY per band
+// With more hidden units than UC, the block walks chunks of UC (weights copied
+// per chunk, GELU' and A through memory).
+// It replaces three 64 x 64-tile GEMM launches; with wgrad_kernel and
+// reduce_kernel a gradient of 1024 rows went from 478 to 22 us on the GPU (4096
+// rows: 1430 to 57), of which the serial column sums over the batch and the
+// weight gradients on 8 blocks had taken most.
+constexpr int kRows = 8, kRowThreads = 256, kRowWarps = kRowThreads / 32;
+
+__host__ __device__ constexpr int rows_ld1(int M) { return 4 * (((M + 3) / 4) | 1); }
+int rows_smem_bytes(int M, int UC) {
+  const int M4 = (M + 3) / 4 * 4;
+  return 4 * (UC * rows_ld1(M) + M * (UC + 4) + kRows * M4 + kRows * UC + kRows * M + kRowWarps * kRows * M);
+}
+
+struct RowsParams {
+  const float *x, *t;
   const int64_t* rows;
-  const float* mu;
-  const float* sd;
-  int M;
-  static constexpr bool kMajorK = true;
-  __device__ float operator()(long long i, long long k) const {
-    const long long r = rows ? rows[i] : i;
-    return (x[r * M + k] - mu[k]) / sd[k];
-  }
-};
-struct LoadStdXT {           // transposed: (band i, row k)
-  LoadStdX s;
-  static constexpr bool kMajorK = false;
-  __device__ float operator()(long long i, long long k) const { return s(k, i); }
+  const float *W1, *b1, *W2, *b2, *mu, *sd;
+  float *xh, *A, *dY, *dH, *loss;
+  int B, M, Hd;
+  float scale;  // 2 / (B M)
 };
 
-// ---- epilogues: called once per output element (i, j) with the dot product
-struct EpiHidden {           // H = acc + b1, A = GELU(H)
-  const float* b1;
-  float* H;
-  float* A;
-  int Hd;
-  __device__ void operator()(long long i, long long j, float acc) const {
-    const float h = acc + b1[j];
-    H[i * Hd + j] = h;
-    A[i * Hd + j] = gelu_f(h);
-  }
-};
-struct EpiOutGrad {          // Y = X + acc + b2; dY = 2 (Y - T) / (B M); loss partial
-  const float* x;
-  const float* t;
-  const int64_t* rows;
-  const float* b2;
-  float* dY;
-  float* loss_acc;           // per-thread partial, summed by the caller
-  int M;
-  float scale;               // 2 / (B M)
-  __device__ void operator()(long long i, long long j, float acc) const {
-    const long long r = rows ? rows[i] : i;
-    const float y = x[r * M + j] + acc + b2[j];
-    const float d = y - t[r * M + j];
-    dY[i * M + j] = scale * d;
-    *loss_acc += d * d;
-  }
-};
-struct EpiBackHidden {       // dH = acc * GELU'(H)
-  const float* H;
-  float* dH;
-  int Hd;
-  __device__ void operator()(long long i, long long j, float acc) const {
-    dH[i * Hd + j] = acc * gelu_grad_f(H[i * Hd + j]);
-  }
-};
-struct EpiStore {            // G[i * ld + j] = acc
-  float* g;
-  long long ld;
-  __device__ void operator()(long long i, long long j, float acc) const { g[i * ld + j] = acc; }
-};
-
-// C[i, j] = sum_k opA(i, k) opB(j, k), 64 x 64 tiles, 4 x 4 outputs per thread.
-template <class LA, class LB, class EPI>
-__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(long long nr, long long nc, long long K,
-                                                            LA la, LB lb, EPI epi, float* loss) {
-  __shared__ float As[kBK][kBM + 4];
-  __shared__ float Bs[kBK][kBN + 4];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const long long i0 = (long long)blockIdx.y * kBM, j0 = (long long)blockIdx.x * kBN;
-  float acc[4][4];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-  for (long long k0 = 0; k0 < K; k0 += kBK) {
-    for (int e = threadIdx.x; e < kBM * kBK; e += kGemmThreads) {
-      const int ii = LA::kMajorK ? e / kBK : e % kBM;
-      const int kk = LA::kMajorK ? e % kBK : e / kBM;
-      As[kk][ii] = (i0 + ii < nr && k0 + kk < K) ? la(i0 + ii, k0 + kk) : 0.f;
+template <int UC, int MQ>
+__global__ void __launch_bounds__(kRowThreads, 1) rows_kernel(RowsParams p) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int RPT = kRows * UC / kRowThreads;  // rows per thread in the H and dH products
+  constexpr int ld2 = UC + 4;
+  const int M = p.M, M4 = (M + 3) / 4 * 4, ld1 = rows_ld1(M), Hd = p.Hd;
+  float* w1s = sm;                   // [UC][ld1]
+  float* w2s = w1s + UC * ld1;       // [M][ld2]
+  float* xs = w2s + M * ld2;         // [kRows][M4]
+  float* as = xs + kRows * M4;       // [kRows][UC]
+  float* dys = as + kRows * UC;      // [M][kRows]
+  float* red = dys + kRows * M;      // [kRowWarps][kRows][M]
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int unit = t % UC, r0 = t / UC * RPT;  // H and dH products: this thread's unit and rows
+  const int chunks = Hd / UC;
+  pdl_next();
+  pdl_wait();
+  auto load_w1 = [&](int h0) {
+    if ((M & 3) == 0) {
+      const int q = M >> 2;
+      for (int e = t; e < UC * q; e += kRowThreads) copy16(w1s + e / q * ld1 + e % q * 4, p.W1 + (size_t)h0 * M + 4 * e, 16);
+    } else {
+      for (int e = t; e < UC * M; e += kRowThreads) copy4(w1s + e / M * ld1 + e % M, p.W1 + (size_t)h0 * M + e);
     }
-    for (int e = threadIdx.x; e < kBN * kBK; e += kGemmThreads) {
-      const int jj = LB::kMajorK ? e / kBK : e % kBN;
-      const int kk = LB::kMajorK ? e % kBK : e / kBN;
-      Bs[kk][jj] = (j0 + jj < nc && k0 + kk < K) ? lb(j0 + jj, k0 + kk) : 0.f;
+    copies_commit();
+  };
+  auto load_w2 = [&](int h0) {
+    for (int e = t; e < M * (UC / 4); e += kRowThreads)
+      copy16(w2s + e / (UC / 4) * ld2 + e % (UC / 4) * 4, p.W2 + (size_t)(e / (UC / 4)) * Hd + h0 + e % (UC / 4) * 4, 16);
+    copies_commit();
+  };
+  if (M4 != M) {  // the columns that pad a row to 16 bytes
+    for (int e = t; e < UC * (M4 - M); e += kRowThreads) w1s[e / (M4 - M) * ld1 + M + e % (M4 - M)] = 0.f;
+    for (int e = t; e < kRows * (M4 - M); e += kRowThreads) xs[e / (M4 - M) * M4 + M + e % (M4 - M)] = 0.f;
+  }
+  if (chunks == 1) {
+    load_w1(0);
+    load_w2(0);
+  }
+  // this thread's elements (t, t + 256, ...) of the rows' bands: x and target are
+  // fetched one block of rows ahead, so that the gathers' latency hides
+  // behind the products of the rows before
+  constexpr int kOwn = (kRows * kMaxIn + kRowThreads - 1) / kRowThreads;
+  float xv[kOwn], tv[kOwn];
+  auto gather = [&](int b0) {
+#pragma unroll
+    for (int k = 0; k < kOwn; ++k) {
+      const int e = t + k * kRowThreads, r = e / M, m = e - r * M;
+      xv[k] = tv[k] = 0.f;
+      if (e < kRows * M && b0 + r < p.B) {
+        const long long src = p.rows ? p.rows[b0 + r] : b0 + r;
+        xv[k] = p.x[src * M + m];
+        tv[k] = p.t[src * M + m];
+      }
     }
+  };
+  gather(blockIdx.x * kRows);
+  float loss = 0.f;
+  bool first = true;
+  for (int b0 = blockIdx.x * kRows; b0 < p.B; b0 += gridDim.x * kRows) {
+    if (!first) __syncthreads();  // the previous rows' readers of xs, as, dys are done
+    float xc[kOwn], tc[kOwn];
+#pragma unroll
+    for (int k = 0; k < kOwn; ++k) {
+      const int e = t + k * kRowThreads, r = e / M, m = e - r * M;
+      xc[k] = xv[k];
+      tc[k] = tv[k];
+      if (e < kRows * M) {
+        float v = 0.f;
+        if (b0 + r < p.B) {
+          v = (xc[k] - p.mu[m]) / p.sd[m];
+          p.xh[(size_t)(b0 + r) * M + m] = v;
+        }
+        xs[r * M4 + m] = v;
+      }
+    }
+    if (b0 + (int)gridDim.x * kRows < p.B) gather(b0 + gridDim.x * kRows);
+    float y[kRows][MQ];
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+#pragma unroll
+      for (int q = 0; q < MQ; ++q) y[r][q] = 0.f;
+    float gp[RPT];  // GELU'(H) of this thread's unit and rows (one chunk)
+    for (int c = 0; c < chunks; ++c) {
+      const int h0 = c * UC;
+      if (chunks > 1) {
+        __syncthreads();  // the previous chunk's readers of w1s, w2s and as are done
+        load_w1(h0);
+        load_w2(h0);
+      }
+      if (chunks > 1 || first) copies_wait<1>();
+      __syncthreads();  // W1 and xs are in
+      float h[RPT];
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) h[r] = 0.f;
+#pragma unroll 4
+      for (int m = 0; m < M4; m += 4) {
+        const float4 w = *reinterpret_cast<const float4*>(w1s + unit * ld1 + m);
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) {
+          const float4 v = *reinterpret_cast<const float4*>(xs + (r0 + r) * M4 + m);
+          h[r] = fmaf(v.x, w.x, h[r]);
+          h[r] = fmaf(v.y, w.y, h[r]);
+          h[r] = fmaf(v.z, w.z, h[r]);
+          h[r] = fmaf(v.w, w.w, h[r]);
+        }
+      }
+      const float bias = p.b1[h0 + unit];
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) {
+        const float v = h[r] + bias, a = gelu_f(v);
+        gp[r] = gelu_grad_f(v);
+        as[(r0 + r) * UC + unit] = a;
+        if (b0 + r0 + r < p.B) {
+          p.A[(size_t)(b0 + r0 + r) * Hd + h0 + unit] = a;
+          if (chunks > 1) p.dH[(size_t)(b0 + r0 + r) * Hd + h0 + unit] = gp[r];
+        }
+      }
+      if (chunks > 1 || first) copies_wait<0>();
+      __syncthreads();  // W2 and this chunk's A are in
+      const int j0 = warp * (UC / kRowWarps);
+#pragma unroll 2
+      for (int j = j0; j < j0 + UC / kRowWarps; j += 4) {
+        float4 w[MQ];
+#pragma unroll
+        for (int q = 0; q < MQ; ++q) w[q] = *reinterpret_cast<const float4*>(w2s + min(lane + 32 * q, M - 1) * ld2 + j);
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+          const float4 a = *reinterpret_cast<const float4*>(as + r * UC + j);
+#pragma unroll
+          for (int q = 0; q < MQ; ++q) {
+            y[r][q] = fmaf(a.x, w[q].x, y[r][q]);
+            y[r][q] = fmaf(a.y, w[q].y, y[r][q]);
+            y[r][q] = fmaf(a.z, w[q].z, y[r][q]);
+            y[r][q] = fmaf(a.w, w[q].w, y[r][q]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; ++r)
+#pragma unroll
+      for (int q = 0; q < MQ; ++q)
+        if (lane + 32 * q < M) red[(warp * kRows + r) * M + lane + 32 * q] = y[r][q];
     __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < kBK; ++kk) {
-      float a[4], b[4];
+    for (int k = 0; k < kOwn; ++k) {
+      const int e = t + k * kRowThreads, r = e / M, m = e - r * M;
+      if (e >= kRows * M) continue;
+      float d = 0.f;
+      if (b0 + r < p.B) {
+        float s = 0.f;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty * 4 + r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx * 4 + c];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
+        for (int w = 0; w < kRowWarps; ++w) s += red[w * kRows * M + e];
+        d = xc[k] + s + p.b2[m] - tc[k];
+        loss = fmaf(d, d, loss);
+        d *= p.scale;
+        p.dY[(size_t)(b0 + r) * M + m] = d;
+      }
+      dys[m * kRows + r] = d;
     }
-    __syncthreads();
+    for (int c = 0; c < chunks; ++c) {
+      const int h0 = c * UC;
+      if (chunks > 1) {
+        __syncthreads();  // the readers of w2s are done
+        load_w2(h0);
+        copies_wait<0>();
+      }
+      __syncthreads();  // dys (and W2) are in
+      float g[RPT];
+#pragma unroll
+      for (int r = 0; r < RPT; ++r) g[r] = 0.f;
+#pragma unroll 8
+      for (int m = 0; m < M; ++m) {
+        const float w = w2s[m * ld2 + unit];
+        float d[RPT];
+        if constexpr (RPT == 1) {
+          d[0] = dys[m * kRows + r0];
+        } else if constexpr (RPT == 2) {
+          const float2 v = *reinterpret_cast<const float2*>(dys + m * kRows + r0);
+          d[0] = v.x;
+          d[1] = v.y;
+        } else {
+#pragma unroll
+          for (int r = 0; r < RPT; r += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(dys + m * kRows + r0 + r);
+            d[r] = v.x;
+            d[r + 1] = v.y;
+            d[r + 2] = v.z;
+            d[r + 3] = v.w;
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < RPT; ++r) g[r] = fmaf(d[r], w, g[r]);
+      }
+#pragma unroll
+      for (int r = 0; r < RPT; ++r)
+        if (b0 + r0 + r < p.B) {
+          float* d = p.dH + (size_t)(b0 + r0 + r) * Hd + h0 + unit;
+          *d = g[r] * (chunks > 1 ? *d : gp[r]);
+        }
+    }
+    first = false;
   }
-  float part = 0.f;
-  EPI e = epi;
-  if constexpr (std::is_same<EPI, EpiOutGrad>::value) e.loss_acc = &part;
+  if (first) copies_wait<0>();
+  if (p.loss) {
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const long long i = i0 + ty * 4 + r, j = j0 + tx * 4 + c;
-      if (i < nr && j < nc) e(i, j, acc[r][c]);
+    for (int o = 16; o; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+    __syncthreads();
+    if (lane == 0) red[warp] = loss;
+    __syncthreads();
+    if (t == 0) {
+      float s = 0.f;
+      for (int w = 0; w < kRowWarps; ++w) s += red[w];
+      atomicAdd(p.loss, s);
     }
-  if constexpr (std::is_same<EPI, EpiOutGrad>::value) {
-    if (loss) atomicAdd(loss, part);
   }
 }
 
-template <class LA, class LB, class EPI>
-cudaError_t gemm(long long nr, long long nc, long long K, LA la, LB lb, EPI epi, float* loss,
-                 cudaStream_t s) {
-  const dim3 grid((unsigned)((nc + kBN - 1) / kBN), (unsigned)((nr + kBM - 1) / kBM));
-  gemm_kernel<LA, LB, EPI><<<grid, kGemmThreads, 0, s>>>(nr, nc, K, la, lb, epi, loss);
-  return cudaGetLastError();
-}
+// ---- wgrad_kernel: a 64-unit tile of dW1 (blockIdx.y 0: dH^T Xh, and db1) or
+// dW2 (1: A^T dY, and db2 by tile 0) over one slice of the batch (blockIdx.z).
+// Stages of 32 rows of both operands arrive by asynchronous copies while the
+// previous stage multiplies; thread (ty, tx) owns units 4 ty .. 4 ty + 3 and
+// bands tx + 16 q.  The batch is cut into enough slices to fill the chip (the
+// 64 x 64 tiles over the whole batch before ran on 8 blocks); their partial
+// sums are added in order by reduce_kernel.
+constexpr int kStage = 32;
 
-// db1[j] = sum_b dH[b, j] (j < Hd), db2[m] = sum_b dY[b, m]
-__global__ void colsum_kernel(const float* dH, const float* dY, int B, int Hd, int M, float* db1,
-                              float* db2) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= Hd + M) return;
-  float s = 0.f;
-  if (c < Hd) {
-    for (int b = 0; b < B; ++b) s += dH[(long long)b * Hd + c];
-    db1[c] = s;
+struct WgradParams {
+  const float *xh, *A, *dY, *dH;
+  float* part;        // [slices][n_params], packed like the parameters
+  long long n_params;
+  int B, M, Hd, slice;  // rows per slice
+};
+
+// Asks for more than half of an SM's shared memory, so that an SM takes one
+// block: the blocks are scheduled while rows_kernel's still fill most SMs, and
+// four or five of them would gather on the few free ones (1024 rows: 38.7 us
+// a gradient that way, 22.1 with one to an SM).
+int wgrad_smem_bytes(int M) { return std::max(4 * (2 * kStage * 64 + 2 * (kStage * M + 128)), 116 * 1024); }
+
+template <int NQ>
+__global__ void __launch_bounds__(256) wgrad_kernel(WgradParams p) {
+  extern __shared__ __align__(16) float sm[];
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  const int M = p.M, Hd = p.Hd, j0 = blockIdx.x * 64;
+  const bool second = blockIdx.y != 0;
+  const float* P = second ? p.A : p.dH;   // [B][Hd]
+  const float* Q = second ? p.dY : p.xh;  // [B][M]
+  const int qs = kStage * M + 128;        // (a band lane past M reads on past its row)
+  float* Ps = sm;                         // [2][kStage][64]
+  float* Qs = sm + 2 * kStage * 64;       // [2][kStage][M]
+  const int first = blockIdx.z * p.slice, end = min(first + p.slice, p.B);
+  pdl_next();
+  pdl_wait();
+  auto load = [&](int k0, int s) {
+    for (int e = t; e < kStage * 16; e += 256) {
+      const int k = e >> 4, c = e & 15;
+      const bool ok = k0 + k < end;
+      copy16(Ps + (s * kStage + k) * 64 + 4 * c, P + (size_t)(ok ? k0 + k : first) * Hd + j0 + 4 * c, ok ? 16 : 0);
+    }
+    const long long from = (long long)k0 * M, left = (long long)(end - k0) * M;  // floats of this slice
+    for (int e = 4 * t; e < kStage * M; e += 1024) {
+      const int n = (int)min(4ll, max(0ll, left - e));
+      copy16(Qs + s * qs + e, Q + (n ? from + e : 0), 4 * n);
+    }
+    copies_commit();
+  };
+  float acc[4][NQ];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) acc[i][q] = 0.f;
+  float col = 0.f;  // column sum: unit j0 + t of dH, or band t of dY
+  const bool sums = second ? blockIdx.x == 0 && t < M : t < 64;
+  load(first, 0);
+  int s = 0;
+  for (int k0 = first; k0 < end; k0 += kStage, s ^= 1) {
+    if (k0 + kStage < end) {
+      load(k0 + kStage, s ^ 1);
+      copies_wait<1>();
+    } else {
+      copies_wait<0>();
+    }
+    __syncthreads();
+    const float* a = Ps + s * kStage * 64 + 4 * ty;
+    const float* b = Qs + s * qs + tx;
+#pragma unroll 8
+    for (int k = 0; k < kStage; ++k) {
+      const float4 v = *reinterpret_cast<const float4*>(a + k * 64);
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        const float w = b[k * M + 16 * q];
+        acc[0][q] = fmaf(v.x, w, acc[0][q]);
+        acc[1][q] = fmaf(v.y, w, acc[1][q]);
+        acc[2][q] = fmaf(v.z, w, acc[2][q]);
+        acc[3][q] = fmaf(v.w, w, acc[3][q]);
+      }
+    }
+    if (sums) {
+      const float* cs = second ? Qs + s * qs + t : Ps + s * kStage * 64 + t;
+      const int ld = second ? M : 64;
+      float s0 = 0.f, s1 = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < kStage; k += 2) {
+        s0 += cs[k * ld];
+        s1 += cs[(k + 1) * ld];
+      }
+      col += s0 + s1;
+    }
+    __syncthreads();  // this stage's readers are done before it is refilled
+  }
+  float* g = p.part + (size_t)blockIdx.z * p.n_params;
+  const size_t w1 = (size_t)Hd * M;
+  if (!second) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int q = 0; q < NQ; ++q)
+        if (tx + 16 * q < M) g[(size_t)(j0 + 4 * ty + i) * M + tx + 16 * q] = acc[i][q];
+    if (sums) g[w1 + j0 + t] = col;
   } else {
-    const int m = c - Hd;
-    for (int b = 0; b < B; ++b) s += dY[(long long)b * M + m];
-    db2[m] = s;
+    g += w1 + Hd;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+      if (tx + 16 * q < M) {
+        float* row = g + (size_t)(tx + 16 * q) * Hd + j0 + 4 * ty;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) row[i] = acc[i][q];
+      }
+    if (sums) g[w1 + t] = col;
   }
 }
 
-__global__ void adamw_kernel(float* p, const float* g, float* m, float* v, long long n, float lr,
-                             float b1, float b2, float eps, float wd, float c1, float c2) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+struct AdamW {
+  float lr, b1, b2, eps, wd, c1, c2;
+};
+
+__device__ __forceinline__ void adamw_update(float* p, float* m, float* v, long long i, float gi, const AdamW& a) {
+  const float mi = a.b1 * m[i] + (1.f - a.b1) * gi;
+  const float vi = a.b2 * v[i] + (1.f - a.b2) * gi * gi;
   m[i] = mi;
   v[i] = vi;
-  p[i] = p[i] * (1.f - lr * wd) - lr * (mi * c1) / (sqrtf(vi * c2) + eps);
+  p[i] = p[i] * (1.f - a.lr * a.wd) - a.lr * (mi * a.c1) / (sqrtf(vi * a.c2) + a.eps);
+}
+
+// Gradients from the slices' partial sums, added in order: to `grads`, or
+// (grads null) straight into the AdamW update.
+__global__ void reduce_kernel(const float* part, int slices, long long n, float* grads, float* prm, float* m, float* v,
+                              AdamW a) {
+  pdl_next();
+  pdl_wait();
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  float g = 0.f;
+#pragma unroll 8
+  for (int s = 0; s < slices; ++s) g += part[s * n + i];
+  if (grads) grads[i] = g;
+  else adamw_update(prm, m, v, i, g, a);
+}
+
+__global__ void adamw_kernel(float* p, const float* g, float* m, float* v, long long n, AdamW a) {
+  pdl_next();
+  pdl_wait();
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) adamw_update(p, m, v, i, g[i], a);
+}
+
+// Launch that may start while the stream's previous kernel drains (the kernels
+// above touch memory only after griddepcontrol.wait).
+template <class... A>
+cudaError_t launch_pdl(void (*fn)(A...), dim3 grid, int threads, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
+using RowsFn = void (*)(RowsParams);
+template <int UC>
+RowsFn rows_fn(int M) {
+  switch ((M + 31) / 32) {
+    case 1: return rows_kernel<UC, 1>;
+    case 2: return rows_kernel<UC, 2>;
+    case 3: return rows_kernel<UC, 3>;
+    default: return rows_kernel<UC, 4>;
+  }
+}
+
+RowsFn rows_fn(int M, int uc) { return uc == 256 ? rows_fn<256>(M) : uc == 128 ? rows_fn<128>(M) : rows_fn<64>(M); }
+
+using WgradFn = void (*)(WgradParams);
+WgradFn wgrad_fn(int M) {
+  switch ((M + 15) / 16) {
+    case 1: return wgrad_kernel<1>;
+    case 2: return wgrad_kernel<2>;
+    case 3: return wgrad_kernel<3>;
+    case 4: return wgrad_kernel<4>;
+    case 5: return wgrad_kernel<5>;
+    case 6: return wgrad_kernel<6>;
+    case 7: return wgrad_kernel<7>;
+    default: return wgrad_kernel<8>;
+  }
+}
+
+// Batch slices of the weight gradients: about 152 blocks over the tiles, at
+// least 32 rows each (a stage), at most 32 slices.
+int wgrad_slices(int Hd, int B) {
+  const int want = std::max(1, 152 / (2 * (Hd / 64)));
+  return std::max(1, std::min(std::min(want, 32), (B + kStage - 1) / kStage));
 }
 
 // Per-band population mean and standard deviation (two passes, one thread per band).
@@ -342,10 +653,13 @@ struct melt_mlp {
   long long t = 0;            // AdamW steps taken
   double lr = 1e-3, beta1 = 0.9, beta2 = 0.999, eps = 1e-8, wd = 0.01;
   int cap = 0;                // batch rows the workspace holds
-  float* d_H = nullptr;
+  float* d_xh = nullptr;
   float* d_A = nullptr;
   float* d_dY = nullptr;
   float* d_dH = nullptr;
+  float* d_part = nullptr;    // partial weight gradients, one packed vector per batch slice
+  int uc = 0;                 // hidden units a block of rows_kernel holds
+  int sms = 0;
 };
 
 namespace {
@@ -353,11 +667,12 @@ namespace {
 long long param_count(int M, int Hd) { return 2LL * M * Hd + Hd + M; }
 
 void free_ws(melt_mlp* p) {
-  cudaFree(p->d_H);
+  cudaFree(p->d_xh);
   cudaFree(p->d_A);
   cudaFree(p->d_dY);
   cudaFree(p->d_dH);
-  p->d_H = p->d_A = p->d_dY = p->d_dH = nullptr;
+  cudaFree(p->d_part);
+  p->d_xh = p->d_A = p->d_dY = p->d_dH = p->d_part = nullptr;
   p->cap = 0;
 }
 
@@ -365,8 +680,10 @@ melt_status ensure_ws(melt_mlp* p, int batch) {
   if (batch <= p->cap) return MELT_OK;
   free_ws(p);
   const size_t h = (size_t)batch * p->Hd * sizeof(float), o = (size_t)batch * p->M * sizeof(float);
-  if (melt::dev_alloc(&p->d_H, h) != cudaSuccess || melt::dev_alloc(&p->d_A, h) != cudaSuccess ||
-      melt::dev_alloc(&p->d_dY, o) != cudaSuccess || melt::dev_alloc(&p->d_dH, h) != cudaSuccess) {
+  const size_t g = (size_t)wgrad_slices(p->Hd, batch) * p->n_params * sizeof(float);
+  if (melt::dev_alloc(&p->d_xh, o) != cudaSuccess || melt::dev_alloc(&p->d_A, h) != cudaSuccess ||
+      melt::dev_alloc(&p->d_dY, o) != cudaSuccess || melt::dev_alloc(&p->d_dH, h) != cudaSuccess ||
+      melt::dev_alloc(&p->d_part, g) != cudaSuccess) {
     free_ws(p);
     return MELT_ERR_OOM;
   }
@@ -374,38 +691,63 @@ melt_status ensure_ws(melt_mlp* p, int batch) {
   return MELT_OK;
 }
 
+AdamW adamw_of(const melt_mlp* p) {  // of step p->t
+  AdamW a;
+  a.lr = (float)p->lr;
+  a.b1 = (float)p->beta1;
+  a.b2 = (float)p->beta2;
+  a.eps = (float)p->eps;
+  a.wd = (float)p->wd;
+  a.c1 = (float)(1.0 / (1.0 - std::pow(p->beta1, (double)p->t)));
+  a.c2 = (float)(1.0 / (1.0 - std::pow(p->beta2, (double)p->t)));
+  return a;
+}
+
+// Gradient of one batch to `grads`, or (null) an AdamW update from it.
 melt_status grad_impl(melt_mlp* p, const float* X, const float* T, const int64_t* rows, int B,
                       float* grads, float* loss, cudaStream_t s) {
   const int M = p->M, Hd = p->Hd;
-  const float* W1 = p->d_params;
-  const float* b1 = W1 + (long long)Hd * M;
-  const float* W2 = b1 + Hd;
-  const float* b2 = W2 + (long long)M * Hd;
-  float* gW1 = grads;
-  float* gb1 = gW1 + (long long)Hd * M;
-  float* gW2 = gb1 + Hd;
-  float* gb2 = gW2 + (long long)M * Hd;
-  const LoadStdX sx{X, rows, p->d_mu, p->d_sd, M};
-  cudaError_t e;
-  // 1. H = Xh W1^T + b1, A = GELU(H)
-  e = gemm(B, Hd, M, sx, LoadRowK{W1, M}, EpiHidden{b1, p->d_H, p->d_A, Hd}, nullptr, s);
-  if (e != cudaSuccess) return MELT_ERR_CUDA;
-  // 2. Y = X + A W2^T + b2 -> dY, loss
-  e = gemm(B, M, Hd, LoadRowK{p->d_A, Hd}, LoadRowK{W2, Hd},
-           EpiOutGrad{X, T, rows, b2, p->d_dY, nullptr, M, 2.f / ((float)B * (float)M)}, loss, s);
-  if (e != cudaSuccess) return MELT_ERR_CUDA;
-  // 3. dH = (dY W2) * GELU'(H):  op(B)(j, m) = W2[m, j]
-  e = gemm(B, Hd, M, LoadRowK{p->d_dY, M}, LoadColK{W2, Hd}, EpiBackHidden{p->d_H, p->d_dH, Hd},
-           nullptr, s);
-  if (e != cudaSuccess) return MELT_ERR_CUDA;
-  // 4. dW2[m, j] = sum_b dY[b, m] A[b, j];  dW1[j, m] = sum_b dH[b, j] Xh[b, m]
-  e = gemm(M, Hd, B, LoadColK{p->d_dY, M}, LoadColK{p->d_A, Hd}, EpiStore{gW2, Hd}, nullptr, s);
-  if (e != cudaSuccess) return MELT_ERR_CUDA;
-  e = gemm(Hd, M, B, LoadColK{p->d_dH, Hd}, LoadStdXT{sx}, EpiStore{gW1, M}, nullptr, s);
-  if (e != cudaSuccess) return MELT_ERR_CUDA;
-  // 5. bias gradients
-  colsum_kernel<<<(Hd + M + 127) / 128, 128, 0, s>>>(p->d_dH, p->d_dY, B, Hd, M, gb1, gb2);
-  if (cudaGetLastError() != cudaSuccess) return MELT_ERR_CUDA;
+  RowsParams r;
+  r.x = X;
+  r.t = T;
+  r.rows = rows;
+  r.W1 = p->d_params;
+  r.b1 = r.W1 + (long long)Hd * M;
+  r.W2 = r.b1 + Hd;
+  r.b2 = r.W2 + (long long)M * Hd;
+  r.mu = p->d_mu;
+  r.sd = p->d_sd;
+  r.xh = p->d_xh;
+  r.A = p->d_A;
+  r.dY = p->d_dY;
+  r.dH = p->d_dH;
+  r.loss = loss;
+  r.B = B;
+  r.M = M;
+  r.Hd = Hd;
+  r.scale = 2.f / ((float)B * (float)M);
+  const int blocks = std::min((B + kRows - 1) / kRows, p->sms);
+  if (launch_pdl(rows_fn(M, p->uc), dim3(blocks), kRowThreads, rows_smem_bytes(M, p->uc), s, r) != cudaSuccess)
+    return MELT_ERR_CUDA;
+  WgradParams w;
+  w.xh = p->d_xh;
+  w.A = p->d_A;
+  w.dY = p->d_dY;
+  w.dH = p->d_dH;
+  w.part = p->d_part;
+  w.n_params = p->n_params;
+  w.B = B;
+  w.M = M;
+  w.Hd = Hd;
+  const int want = wgrad_slices(Hd, B);
+  w.slice = ((B + want - 1) / want + kStage - 1) / kStage * kStage;
+  const int slices = (B + w.slice - 1) / w.slice;
+  if (launch_pdl(wgrad_fn(M), dim3(Hd / 64, 2, slices), 256, wgrad_smem_bytes(M), s, w) != cudaSuccess)
+    return MELT_ERR_CUDA;
+  const long long n = p->n_params;
+  if (launch_pdl(reduce_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, s, (const float*)p->d_part, slices, n, grads,
+                 p->d_params, p->d_m, p->d_v, grads ? AdamW{} : adamw_of(p)) != cudaSuccess)
+    return MELT_ERR_CUDA;
   return MELT_OK;
 }
 
@@ -549,6 +891,16 @@ melt_status melt_mlp_create(int n_in, int n_hidden, const float* params, const f
   p->M = n_in;
   p->Hd = n_hidden;
   p->n_params = param_count(n_in, n_hidden);
+  // the most hidden units (256, 128 or 64, dividing Hd) whose weights fit a block's shared memory
+  p->uc = 256;
+  while (p->uc > 64 && (n_hidden % p->uc != 0 || rows_smem_bytes(n_in, p->uc) > kMaxSmem)) p->uc /= 2;
+  // (the limit is set to the same value whatever the sizes, for every MLP of the process)
+  if (cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaFuncSetAttribute(rows_fn(n_in, p->uc), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess ||
+      cudaFuncSetAttribute(wgrad_fn(n_in), cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
+    delete p;
+    return MELT_ERR_NO_DEVICE;
+  }
   const size_t pb = (size_t)p->n_params * sizeof(float);
   bool ok = melt::dev_alloc(&p->d_params, pb) == cudaSuccess && melt::dev_alloc(&p->d_grads, pb) == cudaSuccess &&
             melt::dev_alloc(&p->d_m, pb) == cudaSuccess && melt::dev_alloc(&p->d_v, pb) == cudaSuccess &&
@@ -605,33 +957,19 @@ melt_status melt_mlp_train_step(melt_mlp* p, const float* X, const float* target
   if (st != MELT_OK) return st;
   if ((st = ensure_ws(p, batch)) != MELT_OK) return st;
   cudaStream_t s = (cudaStream_t)stream;
-  if ((st = grad_impl(p, X, target, rows, batch, p->d_grads, loss, s)) != MELT_OK) return st;
   p->t += 1;
-  const float c1 = (float)(1.0 / (1.0 - std::pow(p->beta1, (double)p->t)));
-  const float c2 = (float)(1.0 / (1.0 - std::pow(p->beta2, (double)p->t)));
-  const long long n = p->n_params;
-  adamw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p->d_params, p->d_grads, p->d_m, p->d_v, n,
-                                                          (float)p->lr, (float)p->beta1,
-                                                          (float)p->beta2, (float)p->eps,
-                                                          (float)p->wd, c1, c2);
-  return cudaGetLastError() == cudaSuccess ? MELT_OK : MELT_ERR_CUDA;
+  if ((st = grad_impl(p, X, target, rows, batch, nullptr, loss, s)) != MELT_OK) p->t -= 1;
+  return st;
 }
 
 melt_status melt_mlp_adamw_apply(melt_mlp* p, const float* grads, void* stream) {
   if (!p || !grads) return MELT_ERR_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (cudaMemcpyAsync(p->d_grads, grads, (size_t)p->n_params * sizeof(float),
-                      cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-    return MELT_ERR_CUDA;
   p->t += 1;
-  const float c1 = (float)(1.0 / (1.0 - std::pow(p->beta1, (double)p->t)));
-  const float c2 = (float)(1.0 / (1.0 - std::pow(p->beta2, (double)p->t)));
   const long long n = p->n_params;
-  adamw_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p->d_params, p->d_grads, p->d_m, p->d_v, n,
-                                                          (float)p->lr, (float)p->beta1,
-                                                          (float)p->beta2, (float)p->eps,
-                                                          (float)p->wd, c1, c2);
-  return cudaGetLastError() == cudaSuccess ? MELT_OK : MELT_ERR_CUDA;
+  return launch_pdl(adamw_kernel, dim3((unsigned)((n + 255) / 256)), 256, 0, (cudaStream_t)stream, p->d_params, grads,
+                    p->d_m, p->d_v, n, adamw_of(p)) == cudaSuccess
+             ? MELT_OK
+             : MELT_ERR_CUDA;
 }
 
 melt_status melt_mlp_forward(const melt_mlp* p, const float* X, float* Y, int64_t n, void* stream) {
