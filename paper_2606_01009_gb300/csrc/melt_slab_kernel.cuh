@@ -33,10 +33,10 @@
 // into more blocks to use more SMs.
 //
 // Warps: 0-7 epilogue (two per TMEM lane quarter, each half of the block's
-// bins), 8-10, 12 and 13 converters (each takes whole slabs by itself: its samples
+// bins), 8-10 and 12-14 converters (each takes whole slabs by itself: its samples
 // arrive by asynchronous copies in a staging area of its own, one arrival per
-// slab), 11 and 15 MMA issue, even and odd slabs (odd CTA: forwards its basis
-// fills to the even one), 14 basis producer and L2 prefetch.
+// slab), 11 MMA issue (odd CTA: forwards its basis fills to the even one), 15
+// basis producer and L2 prefetch.
 //
 // Code size counts here: the issue thread's few hundred instructions per chunk
 // run once per 1200 clocks between three other warps on its scheduler, and it
@@ -60,9 +60,9 @@ namespace slab {
 using namespace ptx;
 
 constexpr int kF = kTileFrames;
-// Warps 0-7 epilogue; 8-10, 12 and 13 converters; 14 basis producer; 11 and 15,
-// on the scheduler that no converter shares, MMA issue.
-constexpr int kEpiWarps = 8, kCvtWarps = 5, kCvtWarp0 = 8, kMmaWarp = 11, kMmaWarp2 = 15, kBWarp = 14;
+// Warps 0-7 epilogue; 8-10 and 12-14 converters; 11 and 15, on the scheduler
+// that no converter shares, MMA issue and basis producer.
+constexpr int kEpiWarps = 8, kCvtWarps = 6, kCvtWarp0 = 8, kMmaWarp = 11, kBWarp = 15;
 constexpr int kThreads = 512;  // 128 registers a thread
 constexpr int kBlockBins = 80;  // Mel bins of a block: 2 x 40 accumulators per epilogue thread
 constexpr int kGroupsPerWarp = kBlockBins / 16;  // groups of 8 bins per epilogue warp
@@ -317,13 +317,15 @@ static __device__ __forceinline__ void chunk_mmas(uint32_t d, uint32_t a, uint32
   for (int k = 0; k < NK; ++k) mma_pair<true>(d, a + k, ah, w + k * step, wh, idesc);
 }
 
+static __device__ __forceinline__ bool bar_done(uint32_t bar, uint32_t parity) { return mbar_test_wait(bar, parity); }
+
 // ---- even CTA: every MMA of the pair.
-// A chunk's 15 to 24 MMAs take 1200 to 1900 clocks at 80 bins.  One thread
-// took about 1650 clocks a chunk for its waits, ring arithmetic, MMAs and
-// commits, and so bounded the kernel; two threads take the slabs in turn
-// (chunks have accumulators of their own, so their MMAs need no order).
+// A chunk's 15 to 24 MMAs take 1200 to 1900 clocks at 80 bins.  With its waits,
+// ring arithmetic, MMAs and commits one after another this thread took about
+// 1650 clocks a chunk and so bounded the kernel; it now looks at the next
+// chunk's barriers (all at once) before it issues the MMAs of this one.
 template <int P>
-static __device__ void mma_issue(const SlabParams& p, const Ctx& c, const SlabBars& B, uint32_t tmem, int mine) {
+static __device__ void mma_issue(const SlabParams& p, const Ctx& c, const SlabBars& B, uint32_t tmem) {
   constexpr uint32_t ah = (128u >> 4) | (1u << 14);         // SBO 128 B
   constexpr uint32_t wh = ((P * 256u) >> 4) | (1u << 14);   // SBO: the next group of 8 bins
   const uint32_t a0 = ((c.sbase + p.off_a) >> 4) | ((p.lbo_a >> 4) << 16);
@@ -337,44 +339,52 @@ static __device__ void mma_issue(const SlabParams& p, const Ctx& c, const SlabBa
   int* err = p.err;
   Ring ra, rb, rt;
   uint32_t al = a0, bl = b0, d = tmem;
-  int q, b;
-  uint32_t turn = (uint32_t)mine;  // this thread's slabs: those it is zero at
-  bool ok = true;
-  for (int i = 0; ok && unit_at(p, c, i, q, b); ++i) {
-    const int ng = blk_groups(p, b);
-    const uint32_t idesc = idesc_f32acc(1u, 2 * kF, 16u * ng);
-    const uint32_t step = (uint32_t)ng * ((P * 256u) >> 4);
-    for (int kk = 0; ok && kk < n_slab; ++kk, turn ^= 1) {
-      const int js = 16 * kk < n_last ? J : J - 1;
-      if (turn == 0) ok = bar_wait(a_full + 8 * ra.slot, ra.phase, abort, err);
-      for (int j0 = 0; ok && j0 < js; j0 += kps) {
-        if (turn == 0) {
-          ok = bar_wait(b_full + 8 * rb.slot, rb.phase, abort, err) &&
-               bar_wait(t_empty + 8 * rt.slot, rt.phase ^ 1, abort, err);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t a = al + (uint32_t)j0;
-          switch (min(kps, js - j0)) {
-            case 1: chunk_mmas<1>(d, a, ah, bl, wh, ap, step, idesc); break;
-            case 2: chunk_mmas<2>(d, a, ah, bl, wh, ap, step, idesc); break;
-            case 3: chunk_mmas<3>(d, a, ah, bl, wh, ap, step, idesc); break;
-            default: chunk_mmas<4>(d, a, ah, bl, wh, ap, step, idesc); break;
-          }
-          mma_commit_pair_mc(b_empty + 8 * rb.slot, 3);
-          mma_commit_pair_mc(t_full + 8 * rt.slot, 3);
-        }
-        bl += bs;
-        rb.next(NB);
-        if (rb.slot == 0) bl = b0;
-        d += 2 * kBlockBins;
-        rt.next(kNacc);
-        if (rt.slot == 0) d = tmem;
-      }
-      if (ok && turn == 0) mma_commit_pair_mc(a_empty + 8 * ra.slot, 3);
+  int i = 0, q, b, kk = 0, j0 = 0, js = slab_steps(p, 0);
+  bool more = unit_at(p, c, 0, q, b), ready = false;
+  uint32_t ng = more ? (uint32_t)blk_groups(p, b) : 0u;
+  while (more) {
+    const uint32_t bar_a = a_full + 8 * ra.slot, bar_b = b_full + 8 * rb.slot, bar_t = t_empty + 8 * rt.slot;
+    if (!ready && !(bar_wait(bar_a, ra.phase, abort, err) && bar_wait(bar_b, rb.phase, abort, err) &&
+                    bar_wait(bar_t, rt.phase ^ 1, abort, err)))
+      break;
+    tc_fence_after();
+    // this chunk, and the step to the next one
+    const uint32_t a = al + (uint32_t)j0, w = bl, acc = d, idesc = idesc_f32acc(1u, 2 * kF, 16u * ng);
+    const uint32_t step = ng * ((P * 256u) >> 4);
+    const uint32_t done_a = a_empty + 8 * ra.slot, done_b = b_empty + 8 * rb.slot, done_t = t_full + 8 * rt.slot;
+    const int n = min(kps, js - j0);
+    bl += bs;
+    rb.next(NB);
+    if (rb.slot == 0) bl = b0;
+    d += 2 * kBlockBins;
+    rt.next(kNacc);
+    if (rt.slot == 0) d = tmem;
+    j0 += kps;
+    const bool slab_end = j0 >= js;
+    if (slab_end) {
+      j0 = 0;
       al += as;
       ra.next(NA);
       if (ra.slot == 0) al = a0;
+      if (++kk == n_slab) {
+        kk = 0;
+        more = unit_at(p, c, ++i, q, b);
+        if (more) ng = (uint32_t)blk_groups(p, b);
+      }
+      js = 16 * kk < n_last ? J : J - 1;
     }
+    const bool ok_a = bar_done(a_full + 8 * ra.slot, ra.phase), ok_b = bar_done(b_full + 8 * rb.slot, rb.phase),
+               ok_t = bar_done(t_empty + 8 * rt.slot, rt.phase ^ 1);
+    switch (n) {
+      case 1: chunk_mmas<1>(acc, a, ah, w, wh, ap, step, idesc); break;
+      case 2: chunk_mmas<2>(acc, a, ah, w, wh, ap, step, idesc); break;
+      case 3: chunk_mmas<3>(acc, a, ah, w, wh, ap, step, idesc); break;
+      default: chunk_mmas<4>(acc, a, ah, w, wh, ap, step, idesc); break;
+    }
+    mma_commit_pair_mc(done_b, 3);
+    mma_commit_pair_mc(done_t, 3);
+    if (slab_end) mma_commit_pair_mc(done_a, 3);
+    ready = ok_a && ok_b && ok_t;
   }
   // no pair MMA may still be running when either CTA releases TMEM
   mma_commit_pair_mc(bar_at(p, c, B.drain), 3);
@@ -724,7 +734,7 @@ __global__ void __launch_bounds__(kThreads, 1) melt_slab_kernel(const __grid_con
       mbar_init(bar(B.t_empty + i), 2 * kEpiWarps);
     }
     for (int i = 0; i < 16; ++i) mbar_init(bar(B.half + i), 1);
-    mbar_init(bar(B.drain), 2);
+    mbar_init(bar(B.drain), 1);
     *c.abort = 0;
     fence_mbar_init();
   }
@@ -749,10 +759,10 @@ __global__ void __launch_bounds__(kThreads, 1) melt_slab_kernel(const __grid_con
   if (threadIdx.x == 0) pdl_launch_dependents();
   // the basis and the MMAs touch the library's own data only; what reads
   // tiles or samples or writes features waits for the stream's previous kernel
-  if (warp == kMmaWarp || warp == kMmaWarp2) {
+  if (warp == kMmaWarp) {
     if (elect_one()) {
-      if (c.rank == 0) mma_issue<P>(p, c, B, tmem, warp == kMmaWarp ? 0 : 1);
-      else if (warp == kMmaWarp) basis_signal(p, c, B);
+      if (c.rank == 0) mma_issue<P>(p, c, B, tmem);
+      else basis_signal(p, c, B);
       volatile int never = 0;
       mbar_wait(bar_at(p, c, B.drain), 0, &never, p.err, kErrTimeout);
     }
