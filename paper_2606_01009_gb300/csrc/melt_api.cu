@@ -60,7 +60,7 @@ struct melt_basis {
   float* d_dct = nullptr;      // [K][M]
   int* d_err = nullptr;        // latched kernel errors
   TcBasis tc;                  // tensor-core operand images (BF16/FP8 forms)
-  SlabBasis slab;              // FP32 form: three-part split operands (no image: the CUDA-core kernel runs)
+  SlabBasis slab;              // operands of the slab kernel (no image: it does not run for this basis)
   Staging staging[kStagingSlots];
   int next_slot = 0;
   std::vector<TileDesc> plan;  // host scratch for planning
@@ -196,8 +196,16 @@ melt_status create_common(double sr, int n_fft, int hop, const double* freqs, in
     TcConfig c{n_fft, hop, n_freqs, precision, n_mfcc, stft_bands};
     st = tc_build(&b->tc, c, b->w64.data());
   }
+  // operands of the slab kernel: the FP32 form, and log-Mel of split BF16, and
+  // of BF16 where no layout keeps the basis in shared memory
   if (st == MELT_OK && precision == MELT_FP32)
     st = slab_build(&b->slab, n_fft, hop, n_freqs, n_mfcc, 3, b->w64.data());
+  melt_plan first;
+  if (st == MELT_OK && (precision == MELT_BF16 || precision == MELT_BF16X3) && n_freqs <= 128 && n_mfcc == 0 &&
+      stft_bands == 0 && tc_current_plan(&b->tc, &first) && (precision == MELT_BF16X3 || !first.basis_resident)) {
+    st = slab_build(&b->slab, n_fft, hop, n_freqs, 0, precision == MELT_BF16X3 ? 2 : 1, b->w64.data());
+    if (b->slab.d_img) b->tc.slab = &b->slab;
+  }
   if (st == MELT_OK) {
     cudaError_t e = melt::dev_alloc(&b->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(b->d_err, 0, sizeof(int));
@@ -234,12 +242,13 @@ void order_longest_first(TileDesc* t, long long n) {
 // so short that a slab of all Z rows does not fit twice, and the raw
 // projections (mode 1), run on the CUDA cores.
 cudaError_t launch_fp32(melt_basis* b, const float* wave, const TileDesc* tiles, int n_tiles, float* out, int mode,
-                        cudaStream_t stream) {
+                        unsigned flags, cudaStream_t stream) {
   if (mode == 0 && b->slab.d_img) {
     SlabLaunch L;
     L.wave = wave; L.tiles = tiles; L.n_tiles = n_tiles; L.out = out;
     L.dct = b->d_dct; L.w32 = b->d_w32; L.mp = b->mp;
     L.n_mfcc = b->n_mfcc; L.eps = (float)b->eps; L.err = b->d_err; L.sm_count = b->sm_count;
+    L.early_inputs = (flags & MELT_FWD_INPUT_READY) != 0;
     return slab_launch(&b->slab, L, stream);
   }
   SimtParams p;
@@ -342,7 +351,7 @@ melt_status forward_impl(melt_basis* b, const float* wave, const int64_t* offset
   cudaError_t e;
   bool fused = false;  // the kernel applied the correction itself
   if (b->precision == MELT_FP32 || mode == 1) {
-    e = launch_fp32(b, wave, slot->dev, n_tiles, out, mode, stream);
+    e = launch_fp32(b, wave, slot->dev, n_tiles, out, mode, flags, stream);
   } else {
     TcLaunch L;
     L.wave = wave; L.tiles = slot->dev; L.n_tiles = n_tiles; L.out = out;
@@ -423,7 +432,7 @@ melt_status launch_forward_tiles(melt_basis* b, const float* wave, const TileDes
   cudaError_t e;
   bool fused = false;
   if (b->precision == MELT_FP32) {
-    e = launch_fp32(b, wave, d_tiles, n_tiles, out, 0, stream);
+    e = launch_fp32(b, wave, d_tiles, n_tiles, out, 0, 0, stream);
   } else {
     TcLaunch L;
     L.wave = wave; L.tiles = d_tiles; L.n_tiles = n_tiles; L.out = out;

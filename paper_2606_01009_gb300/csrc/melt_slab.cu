@@ -1,6 +1,7 @@
 // Host side of the slab kernel: the operand image, the shared-memory plan and
 // the launch (device code in melt_slab_kernel.cuh).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <vector>
 
@@ -16,15 +17,19 @@ constexpr uint32_t kSmemMax = 227 * 1024;
 
 uint32_t up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 
-// BF16 (round to nearest even) nearest to v; *v becomes the exact remainder.
+// BF16 (round to nearest even; zero below 2^-126) nearest to v, which becomes
+// the exact remainder.
 uint16_t take_bf16(double* v) {
-  const float f = (float)*v;
+  uint64_t d;
+  std::memcpy(&d, v, 8);
+  d = (d + ((uint64_t)1 << 44) - 1 + ((d >> 45) & 1)) & ~(((uint64_t)1 << 45) - 1);  // 8 significant bits
+  double r;
+  std::memcpy(&r, &d, 8);
+  if (!(std::fabs(r) >= 1.1754943508222875e-38)) r = 0.0;
+  const float f = (float)r;  // exact
   uint32_t bits;
   std::memcpy(&bits, &f, 4);
-  bits = (bits + 0x7fffu + ((bits >> 16) & 1u)) & 0xffff0000u;
-  float h;
-  std::memcpy(&h, &bits, 4);
-  *v -= h;
+  *v -= r;
   return (uint16_t)(bits >> 16);
 }
 
@@ -33,7 +38,8 @@ uint32_t mfcc_bytes(const SlabParams& p, int n_mfcc) {
   return n_mfcc > 0 ? up(4u * n_mfcc * 8u * p.groups, 128) + 2u * 8u * kF * 4u : 0u;
 }
 
-// Geometry and shared-memory plan; false where two slots of either ring do not fit.
+// Geometry and shared-memory plan; false where two stages do not fit (never for
+// log-Mel; MFCC with a large DCT matrix).
 bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
   const int P = sb->parts;
   p.N = sb->n_fft;
@@ -43,45 +49,31 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
   p.n_slab = sb->n_slab;
   p.ksteps = sb->ksteps;
   p.groups = sb->groups;
-  p.zrows = kF + p.J - 1;
   p.n_last = p.N - (p.J - 1) * p.H;
-  // a chunk's truncations grow with its K-steps, its drains with their number:
-  // at most 4 K-steps, and all slices of a slab where there are fewer
-  p.kps = std::min(p.J, 4);
+  // a slab's slices in equal stages
+  const int per_slab = (p.J + max_kps(P) - 1) / max_kps(P);
+  p.kps = (p.J + per_slab - 1) / per_slab;
   p.step_bytes = (uint32_t)p.groups * P * 256u;
-  int zr = p.zrows;
-  while ((zr & 7) != 4) ++zr;  // rows = 4 mod 8: the two core columns of a converter store fall on other banks
-  p.lbo_a = (uint32_t)zr * 16u;
+  p.lbo_a = (uint32_t)(p.kps <= 5 ? kRowsA : kRowsA + 8) * 16u;
   p.a_part = 2 * p.lbo_a;
-  p.a_slot = P * p.a_part;
+  p.a_bytes = up(P * p.a_part, 128);
   const int least = (p.groups + kBlockBins / 8 - 1) / (kBlockBins / 8);  // blocks, and groups of the widest one
   const int wbg = 2 * ((p.groups / 2 + least - 1) / least);
-  p.b_slot = (uint32_t)wbg * P * 256u * p.kps;
-  const uint32_t fixed = up(8u * SlabBars(kMaxSlots, kMaxSlots).total, 128) + 128u +
-                         mfcc_bytes(p, n_mfcc) + kCvtWarps * kStageBytes + 128u;
-  if (fixed > kSmemMax) return false;
-  const uint32_t room = kSmemMax - fixed;
-  // six A slots (one per converter warp) where four basis slots fit beside them
-  for (int need = 4; need >= 2; need -= 2)
-    for (int na = 6; na >= 2; --na) {
-      const uint32_t a = up(p.a_slot, 128) * na;
-      if (a >= room) continue;
-      const int nb = std::min<int>(kMaxSlots, (int)((room - a) / up(p.b_slot, 128)));
-      if (nb < need || (need == 4 && na < 3)) continue;
-      p.NA = na;
-      p.NB = nb;
-      p.ncv = std::min(na, kCvtWarps);
-      p.a_slot = up(p.a_slot, 128);
-      p.b_slot = up(p.b_slot, 128);
-      p.off_a = 0;
-      p.off_b = p.a_slot * na;
-      p.off_st = p.off_b + p.b_slot * nb;
-      p.off_bar = p.off_st + kCvtWarps * kStageBytes;
-      p.off_misc = p.off_bar + up(8u * SlabBars(na, nb).total, 128);
-      p.off_dct = p.off_misc + 128u;
-      p.off_part = p.off_dct + up(4u * n_mfcc * 8u * p.groups, 128);
-      return true;
-    }
+  p.stage = p.a_bytes + up((uint32_t)wbg * P * 256u * p.kps, 128);
+  const uint32_t fixed = up(8u * SlabBars(kMaxStages).total, 128) + 128u + mfcc_bytes(p, n_mfcc) + 128u;
+  // as many stages as fit, each of the first kCvtTeams with a converter team's raw samples
+  for (int ns = kMaxStages; ns >= 2; --ns) {
+    const uint32_t raw = std::min(ns, kCvtTeams) * kRawBytes;
+    if (fixed + raw + ns * p.stage > kSmemMax) continue;
+    p.NS = ns;
+    p.ncv = std::min(ns, kCvtTeams);
+    p.off_raw = p.stage * ns;
+    p.off_bar = p.off_raw + raw;
+    p.off_misc = p.off_bar + up(8u * SlabBars(ns).total, 128);
+    p.off_dct = p.off_misc + 128u;
+    p.off_part = p.off_dct + up(4u * n_mfcc * 8u * p.groups, 128);
+    return true;
+  }
   return false;
 }
 
@@ -147,7 +139,11 @@ cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream)
   p.n_pairs = (L.n_tiles + 1) / 2;
   p.n_mfcc = L.n_mfcc;
   p.n_out = L.n_mfcc ? L.n_mfcc : sb->n_mels;
-  void (*fn)(SlabParams) = L.n_mfcc ? melt_slab_kernel<3, true> : melt_slab_kernel<3, false>;
+  p.early_inputs = L.early_inputs ? 1 : 0;
+  void (*fn)(SlabParams) = sb->parts == 1   ? melt_slab_kernel<1, false>
+                           : sb->parts == 2 ? melt_slab_kernel<2, false>
+                           : L.n_mfcc       ? melt_slab_kernel<3, true>
+                                            : melt_slab_kernel<3, false>;
   const int smem = (int)smem_bytes(p, L.n_mfcc);
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
@@ -162,7 +158,7 @@ cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream)
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.blockDim = dim3(slab_threads(sb->parts), 1, 1);
   if (sb->clusters < 0 || sb->clusters_smem != smem) {
     // (always the same limit, so that bases of different sizes do not lower each other's)
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);

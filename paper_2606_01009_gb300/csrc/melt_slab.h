@@ -8,7 +8,7 @@ namespace melt {
 
 // Device-resident operands of one basis for the slab kernel.
 struct SlabBasis {
-  int parts = 0;                       // BF16 parts per operand: 3 for the FP32 form
+  int parts = 0;                       // BF16 parts per operand: 3 for the FP32 form, 2 for split BF16, 1 for BF16
   int n_fft = 0, hop = 0, n_mels = 0;
   int J = 0, n_slab = 0, ksteps = 0;   // polyphase slices, 16-sample slabs, MMA K-steps
   int groups = 0;                      // groups of 8 Mel bins
@@ -28,6 +28,7 @@ struct SlabLaunch {
   float eps;
   int* err;
   int sm_count;
+  bool early_inputs;   // MELT_FWD_INPUT_READY: the waveform readers need not wait for the kernel before
 };
 
 // Builds the operand image for `parts` BF16 parts; leaves d_img null (MELT_OK)

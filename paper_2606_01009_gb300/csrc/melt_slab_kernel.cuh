@@ -11,10 +11,12 @@
 // Accumulation.  The tensor core truncates its FP32 accumulator at every MMA,
 // a bias that grows with the number of MMAs (25 of them put -3.0e-6 dB on the
 // bins near the frame maximum, where the FFMA kernel's error is 2.7e-6 dB
-// RMS).  So K is cut into chunks of at most kps K-steps; each chunk starts
-// from zero, adds its five small products first (they are 2^-8 of the sum, so
-// their truncation does not count) and its hi hi products last, and the epilogue
-// adds the chunks up in FP32 registers with round-to-nearest.
+// RMS).  So K is cut into stages of at most kps K-steps; each starts from zero,
+// adds its small products first (they are 2^-8 of the sum, so their truncation
+// does not count) and its hi hi products last, and the epilogue adds the stages
+// up in FP32 registers with round-to-nearest.  (Two stages to an accumulator
+// measured 96 against 98 us on the 64 x 30 s batch, with errors up to 1.3 times
+// larger: not kept.)
 //
 // Bound.  Six products make 6 x 128,000 flops a frame at (N, M) = (400, 80):
 // 147 TFLOP for the 64 x 30 s batch, tensor-bound (its 184 MB of samples and
@@ -22,9 +24,13 @@
 // the MMAs' way: the basis (384 KB in three parts) does not fit shared memory
 // and neither do two converted tiles (125 KB each), but one K slab of both
 // does.  A slab is 16 columns of the polyphase rows Z[u][r] = x[(t0+u) H + r]
-// (all rows of the tile) and, for each slice j, the K-step n = j H + r of the
-// basis; the slices of a slab read the same A slab at row offset j, so every
-// sample is converted once.  Slabs and K-steps flow through two rings.
+// and, for each slice j, the K-step n = j H + r of the basis; the slices of a
+// slab read the same rows at row offset j, so a sample is converted once for
+// all of them.  A stage holds up to kps slices of a slab: the 128 + kps - 1 rows
+// that they read, converted, and their basis blocks.  Stages flow through one
+// ring (shared memory has 4 to 8), each with one barrier that both operands of
+// both CTAs complete.  With more slices than kps (short hops) a slab's rows are
+// converted once per stage.
 //
 // Clusters of two CTAs share each MMA (cta_group::2, M = 256: two tiles): the
 // even CTA holds the W_r rows of a K-step, the odd one the W_i rows, so each
@@ -60,16 +66,26 @@ namespace slab {
 using namespace ptx;
 
 constexpr int kF = kTileFrames;
-// Warps 0-7 epilogue; 8-10 and 12-14 converters; 11 and 15, on the scheduler
-// that no converter shares, MMA issue and basis producer.
-constexpr int kEpiWarps = 8, kCvtWarps = 6, kCvtWarp0 = 8, kMmaWarp = 11, kBWarp = 15;
-constexpr int kThreads = 512;  // 128 registers a thread
+// Warps 0-7 epilogue; 11 and 15, on one scheduler, MMA issue and basis
+// producer; the others from 8 on converters: six in the FP32 form, twelve where
+// there are fewer MMAs to a stage (its conversion took 6000 clocks a warp, 1000 a
+// stage with six, where P 2's MMAs take 480 to 720).
+constexpr int kEpiWarps = 8, kMmaWarp = 11, kBWarp = 15;
+constexpr int kCvtTeams = 6;  // stages in conversion at once
+__host__ __device__ constexpr int team_warps(int P) { return P == 3 ? 1 : 2; }  // warps that share a stage's rows
+__host__ __device__ constexpr int slab_threads(int P) { return 32 * (kEpiWarps + 2 + kCvtTeams * team_warps(P)); }
 constexpr int kBlockBins = 80;  // Mel bins of a block: 2 x 40 accumulators per epilogue thread
 constexpr int kGroupsPerWarp = kBlockBins / 16;  // groups of 8 bins per epilogue warp
 constexpr int kNacc = 3;        // TMEM accumulators of 2 x kBlockBins columns
-constexpr int kStageRows = 136; // rows of a slab that a converter warp stages at a time
-constexpr uint32_t kStageBytes = kStageRows * 64u;
-constexpr int kMaxSlots = 8;    // slots of either ring
+constexpr int kMaxKps = 8;
+// K-steps of a stage at most.  P 3: its truncations grow with them, its drains
+// with their number.
+__host__ __device__ constexpr int max_kps(int P) { return P == 3 ? 4 : kMaxKps; }
+constexpr int kRowsA = 132;     // rows of a stage's A operand: 128 + kps - 1 and up to 4 mod 8, so that the two core
+                                // columns of a converter store fall on other banks (kMaxKps - 1 more at most)
+constexpr int kStageRows = kF + kMaxKps;  // sample rows a converter warp copies for a stage
+constexpr uint32_t kRawBytes = kStageRows * 64u;
+constexpr int kMaxStages = 8;
 
 struct SlabParams {
   const float* wave;
@@ -82,31 +98,30 @@ struct SlabParams {
   float eps;
   int n_tiles, n_pairs, mp;
   int N, H, M, J, n_slab, ksteps, groups;
-  int zrows;           // Z rows of a tile: 128 + J - 1
   int n_last;          // samples of the last slice: N - (J - 1) H
   int nblk, wbg;       // blocks of wbg groups of 8 bins (the last may have fewer)
   int inner;           // blocks a unit takes in turn (MFCC: all of them, else 1)
   int n_units;
-  int kps;             // K-steps per basis slot (one accumulation chunk)
-  int NA, NB;          // slots of the A and basis rings
-  int ncv;             // converter warps at work: at most NA (a warp that took slab g waits for the slot of
-                       // slab g + ncv by one parity bit, which tells only neighbouring phases apart)
-  uint32_t lbo_a, a_part, a_slot, b_slot, step_bytes;
-  uint32_t off_a, off_b, off_st, off_bar, off_misc, off_dct, off_part;
+  int kps;             // K-steps (slices of a slab) per stage
+  int NS;              // stages of the ring
+  int ncv;             // converter teams at work: at most NS (a team that took stage g waits for the place of
+                       // stage g + ncv by one parity bit, which tells only neighbouring phases apart)
+  uint32_t lbo_a, a_part, a_bytes, stage, step_bytes;  // a stage: A (a_bytes: P parts of two core columns), then B
+  uint32_t off_raw, off_bar, off_misc, off_dct, off_part;
   int n_mfcc, n_out;
+  int early_inputs;    // the waveform's readers need not wait for the stream's previous kernel
 };
 
 struct SlabBars {
-  int a_full, a_empty, b_full, b_empty, t_full, t_empty, half, drain, total;
-  __host__ __device__ SlabBars(int NA, int NB) {
-    a_full = 0;               // both CTAs' converters (even CTA's copy is used)
-    a_empty = a_full + NA;    // MMA commit, both CTAs
-    b_full = a_empty + NA;    // this CTA's basis copies; even CTA: and the odd one's signal that its own are in
-    b_empty = b_full + NB;    // MMA commit, both CTAs
-    t_full = b_empty + NB;    // MMA commit, both CTAs
+  int full, empty, t_full, t_empty, part, drain, total;
+  __host__ __device__ SlabBars(int NS) {
+    full = 0;                 // a stage: this CTA's basis copies; even CTA: also both CTAs' converters and the odd
+                              // CTA's signal that its copies are in
+    empty = full + NS;        // MMA commit, both CTAs
+    t_full = empty + NS;      // MMA commit, both CTAs
     t_empty = t_full + kNacc; // both CTAs' epilogues (even CTA's copy is used)
-    half = t_empty + kNacc;   // MFCC, per lane quarter: part buffers 0, 1 filled; [16 B on] taken
-    drain = half + 16;
+    part = t_empty + kNacc;   // MFCC, per lane quarter: part buffers 0, 1 filled; [16 B on] taken
+    drain = part + 16;
     total = drain + 1;
   }
 };
@@ -116,6 +131,18 @@ struct Ctx {
   int cluster, n_clusters;
   volatile int* abort;
 };
+
+// Accumulators of a unit.  P 3: one per stage, added up in FP32 registers.  P 2
+// (whose operands carry 16 bits): two, each over half of the stages, added when
+// the epilogue reads them.  P 1: one (the sums of the form's other layouts).
+static __device__ __forceinline__ int unit_stages(const SlabParams& p) {
+  const int last = (p.n_last + 15) / 16;  // slabs that all slices reach
+  return last * ((p.J + p.kps - 1) / p.kps) + (p.n_slab - last) * ((p.J - 1 + p.kps - 1) / p.kps);
+}
+template <int P>
+static __device__ __forceinline__ int acc_stages(const SlabParams& p) {
+  return P == 3 ? 1 : P == 2 ? (unit_stages(p) + 1) / 2 : unit_stages(p);
+}
 
 // Ring position: slot and the parity its next completion has.
 struct Ring {
@@ -209,7 +236,7 @@ static __device__ __forceinline__ void prefetch_span(const SlabParams& p, const 
   for (int o = 0; o < avail; o += 8192) prefetch_l2(p.wave + td.in_off + o, (uint32_t)min(8192, avail - o) * 4u);
 }
 
-// ---- basis producer: each unit's K-steps of this CTA's half, a slot per chunk
+// ---- basis producer: each unit's K-steps of this CTA's half, stage by stage
 template <int P>
 static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const SlabBars& B) {
   const uint64_t pol = policy_evict_last();
@@ -225,13 +252,13 @@ static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const S
     for (int kk = 0; ok && kk < p.n_slab; ++kk) {
       const int js = slab_steps(p, kk);
       for (int j0 = 0; j0 < js; j0 += p.kps) {
-        if (!bar_wait(bar_at(p, c, B.b_empty + r.slot), r.phase ^ 1, c.abort, p.err)) {
+        if (!bar_wait(bar_at(p, c, B.empty + r.slot), r.phase ^ 1, c.abort, p.err)) {
           ok = false;
           break;
         }
         const int n = min(p.kps, js - j0);
-        const uint32_t full = bar_at(p, c, B.b_full + r.slot);
-        const uint32_t dst = c.sbase + p.off_b + r.slot * p.b_slot;
+        const uint32_t full = bar_at(p, c, B.full + r.slot);
+        const uint32_t dst = c.sbase + r.slot * p.stage + p.a_bytes;
         mbar_arrive_expect_tx(full, blk * n);
         if (blk == p.step_bytes) {
           bulk_g2s_hint(dst, src, blk * n, full, pol);
@@ -240,11 +267,11 @@ static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const S
         }
         src += (size_t)n * p.step_bytes;
         ++issued;
-        r.next(p.NB);
+        r.next(p.NS);
         if (!ahead) {
           // L2 prefetch of the samples, one unit ahead of the converters' copies
           ahead = true;
-          if (i == 0) pdl_wait();
+          if (i == 0 && !p.early_inputs) pdl_wait();
           int qn, bn;
           if (unit_at(p, c, i + 1, qn, bn) && (qn != q || i == 0)) prefetch_span(p, tile_of(p, c, qn));
         }
@@ -253,11 +280,11 @@ static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const S
   }
   // every issued copy has landed before the CTA can exit
   volatile int never = 0;
-  for (int k = max(0, issued - p.NB); k < issued; ++k)
-    mbar_wait(bar_at(p, c, B.b_full + k % p.NB), (k / p.NB) & 1, &never, p.err, kErrTimeout);
+  for (int k = max(0, issued - p.NS); k < issued; ++k)
+    mbar_wait(bar_at(p, c, B.full + k % p.NS), (k / p.NS) & 1, &never, p.err, kErrTimeout);
 }
 
-// ---- odd CTA: one arrival on the even CTA's b_full per filled slot
+// ---- odd CTA: one arrival on the even CTA's barrier per stage whose basis is in
 static __device__ void basis_signal(const SlabParams& p, const Ctx& c, const SlabBars& B) {
   Ring r;
   int q, b;
@@ -265,9 +292,9 @@ static __device__ void basis_signal(const SlabParams& p, const Ctx& c, const Sla
     for (int kk = 0; kk < p.n_slab; ++kk) {
       const int js = slab_steps(p, kk);
       for (int j0 = 0; j0 < js; j0 += p.kps) {
-        if (!bar_wait(bar_at(p, c, B.b_full + r.slot), r.phase, c.abort, p.err)) return;
-        mbar_arrive_cluster(mapa_shared(bar_at(p, c, B.b_full + r.slot), 0));
-        r.next(p.NB);
+        if (!bar_wait(bar_at(p, c, B.full + r.slot), r.phase, c.abort, p.err)) return;
+        mbar_arrive_cluster(mapa_shared(bar_at(p, c, B.full + r.slot), 0));
+        r.next(p.NS);
       }
     }
 }
@@ -289,102 +316,117 @@ static __device__ __forceinline__ void mma_pair(uint32_t d, uint32_t a, uint32_t
       "r"(a), "r"(a_hi), "r"(b), "r"(b_hi), "r"(idesc), "n"(ACC ? 1 : 0));
 }
 
+static __device__ __forceinline__ void mma_pair_if(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi,
+                                                   uint32_t idesc, bool acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 x, y;\n\t"
+      "mov.b64 x, {%1, %2};\n\tmov.b64 y, {%3, %4};\n\t"
+      "setp.ne.u32 p, %6, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], x, y, %5, p;\n\t}\n" ::"r"(d),
+      "r"(a), "r"(a_hi), "r"(b), "r"(b_hi), "r"(idesc), "r"((uint32_t)acc));
+}
+
 static __device__ __forceinline__ bool elect_one() {
   uint32_t r;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
   return r != 0;
 }
 
-// The products of a chunk of NK K-steps into accumulator d.  a, w: descriptors
-// (low words) of the first K-step's hi parts (parts 0 hi, 1 mid, 2 lo are ap
-// and 16 apart, K-steps 1 row of A and `step` of the basis, in 16-byte units).
-// The small products of every K-step first, then the hi hi products.
-template <int NK>
-static __device__ __forceinline__ void chunk_mmas(uint32_t d, uint32_t a, uint32_t ah, uint32_t w, uint32_t wh,
-                                                  uint32_t ap, uint32_t step, uint32_t idesc) {
+// Products of a stage's n K-steps into accumulator d.  a, w: descriptors (low
+// words) of the first K-step's hi parts (parts 0 hi, 1 mid, 2 lo are ap and 16
+// apart, K-steps 1 row of A and `step` of the basis, in 16-byte units).  SMALL:
+// the products with a mid or lo part, else hi hi.  Straight-line code with one
+// predicate per K-step: a switch over n cost 150 to 200 clocks a stage.
+template <int P, bool SMALL>
+static __device__ __forceinline__ void stage_mmas(int n, uint32_t d, uint32_t a, uint32_t ah, uint32_t w, uint32_t wh,
+                                                  uint32_t ap, uint32_t step, uint32_t idesc, bool first) {
   const uint32_t am = a + ap, al = am + ap;
 #pragma unroll
-  for (int k = 0; k < NK; ++k) {
+  for (int k = 0; k < max_kps(P); ++k) {
+    if (k >= n) break;
     const uint32_t wk = w + k * step;
-    if (k == 0) mma_pair<false>(d, al + k, ah, wk, wh, idesc);
-    else mma_pair<true>(d, al + k, ah, wk, wh, idesc);
-    mma_pair<true>(d, a + k, ah, wk + 32, wh, idesc);
-    mma_pair<true>(d, am + k, ah, wk + 16, wh, idesc);
-    mma_pair<true>(d, am + k, ah, wk, wh, idesc);
-    mma_pair<true>(d, a + k, ah, wk + 16, wh, idesc);
+    if constexpr (P == 1) {
+      if (k == 0) mma_pair_if(d, a, ah, wk, wh, idesc, !first);
+      else mma_pair<true>(d, a + k, ah, wk, wh, idesc);
+    } else if constexpr (!SMALL) {
+      mma_pair<true>(d, a + k, ah, wk, wh, idesc);
+    } else if constexpr (P == 2) {
+      if (k == 0) mma_pair_if(d, a, ah, wk + 16, wh, idesc, !first);
+      else mma_pair<true>(d, a + k, ah, wk + 16, wh, idesc);
+      mma_pair<true>(d, am + k, ah, wk, wh, idesc);
+    } else {
+      if (k == 0) mma_pair_if(d, al, ah, wk, wh, idesc, !first);
+      else mma_pair<true>(d, al + k, ah, wk, wh, idesc);
+      mma_pair<true>(d, a + k, ah, wk + 32, wh, idesc);
+      mma_pair<true>(d, am + k, ah, wk + 16, wh, idesc);
+      mma_pair<true>(d, am + k, ah, wk, wh, idesc);
+      mma_pair<true>(d, a + k, ah, wk + 16, wh, idesc);
+    }
   }
-#pragma unroll
-  for (int k = 0; k < NK; ++k) mma_pair<true>(d, a + k, ah, w + k * step, wh, idesc);
 }
 
-static __device__ __forceinline__ bool bar_done(uint32_t bar, uint32_t parity) { return mbar_test_wait(bar, parity); }
+// Both phases complete?  The two tests are in flight together.
+static __device__ __forceinline__ bool bar_wait2(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1, volatile int* abort,
+                                                 int* err) {
+  const bool x = mbar_test_wait(b0, p0), y = mbar_test_wait(b1, p1);
+  return (x || bar_wait(b0, p0, abort, err)) && (y || bar_wait(b1, p1, abort, err));
+}
 
 // ---- even CTA: every MMA of the pair.
-// A chunk's 15 to 24 MMAs take 1200 to 1900 clocks at 80 bins.  With its waits,
-// ring arithmetic, MMAs and commits one after another this thread took about
-// 1650 clocks a chunk and so bounded the kernel; it now looks at the next
-// chunk's barriers (all at once) before it issues the MMAs of this one.
+// What this thread does besides its MMAs has to stay below the time they take
+// (P 3: 960 to 1900 clocks a stage at 80 bins; P 2: 480 to 720), and it runs at
+// ten and more clocks an instruction beside the SM's other warps: with rings of
+// their own for A and the basis (three waits, three commits and three ring steps
+// a slab) it took 830 clocks and bounded the P 2 kernel.
 template <int P>
 static __device__ void mma_issue(const SlabParams& p, const Ctx& c, const SlabBars& B, uint32_t tmem) {
   constexpr uint32_t ah = (128u >> 4) | (1u << 14);         // SBO 128 B
   constexpr uint32_t wh = ((P * 256u) >> 4) | (1u << 14);   // SBO: the next group of 8 bins
-  const uint32_t a0 = ((c.sbase + p.off_a) >> 4) | ((p.lbo_a >> 4) << 16);
-  const uint32_t b0 = ((c.sbase + p.off_b) >> 4) | ((128u >> 4) << 16);    // LBO 128 B
-  const uint32_t ap = p.a_part >> 4, as = p.a_slot >> 4, bs = p.b_slot >> 4;
-  const uint32_t a_full = bar_at(p, c, B.a_full), a_empty = bar_at(p, c, B.a_empty);
-  const uint32_t b_full = bar_at(p, c, B.b_full), b_empty = bar_at(p, c, B.b_empty);
+  const uint32_t a0 = (c.sbase >> 4) | ((p.lbo_a >> 4) << 16);
+  const uint32_t b0 = ((c.sbase + p.a_bytes) >> 4) | ((128u >> 4) << 16);  // LBO 128 B
+  const uint32_t ap = p.a_part >> 4, stage = p.stage >> 4;
+  const uint32_t full = bar_at(p, c, B.full), empty = bar_at(p, c, B.empty);
   const uint32_t t_full = bar_at(p, c, B.t_full), t_empty = bar_at(p, c, B.t_empty);
-  const int kps = p.kps, J = p.J, n_last = p.n_last, n_slab = p.n_slab, NA = p.NA, NB = p.NB;
+  const int kps = p.kps, J = p.J, n_last = p.n_last, n_slab = p.n_slab, NS = p.NS;
   volatile int* abort = c.abort;
   int* err = p.err;
-  Ring ra, rb, rt;
-  uint32_t al = a0, bl = b0, d = tmem;
-  int i = 0, q, b, kk = 0, j0 = 0, js = slab_steps(p, 0);
-  bool more = unit_at(p, c, 0, q, b), ready = false;
-  uint32_t ng = more ? (uint32_t)blk_groups(p, b) : 0u;
-  while (more) {
-    const uint32_t bar_a = a_full + 8 * ra.slot, bar_b = b_full + 8 * rb.slot, bar_t = t_empty + 8 * rt.slot;
-    if (!ready && !(bar_wait(bar_a, ra.phase, abort, err) && bar_wait(bar_b, rb.phase, abort, err) &&
-                    bar_wait(bar_t, rt.phase ^ 1, abort, err)))
-      break;
-    tc_fence_after();
-    // this chunk, and the step to the next one
-    const uint32_t a = al + (uint32_t)j0, w = bl, acc = d, idesc = idesc_f32acc(1u, 2 * kF, 16u * ng);
-    const uint32_t step = ng * ((P * 256u) >> 4);
-    const uint32_t done_a = a_empty + 8 * ra.slot, done_b = b_empty + 8 * rb.slot, done_t = t_full + 8 * rt.slot;
-    const int n = min(kps, js - j0);
-    bl += bs;
-    rb.next(NB);
-    if (rb.slot == 0) bl = b0;
-    d += 2 * kBlockBins;
-    rt.next(kNacc);
-    if (rt.slot == 0) d = tmem;
-    j0 += kps;
-    const bool slab_end = j0 >= js;
-    if (slab_end) {
-      j0 = 0;
-      al += as;
-      ra.next(NA);
-      if (ra.slot == 0) al = a0;
-      if (++kk == n_slab) {
-        kk = 0;
-        more = unit_at(p, c, ++i, q, b);
-        if (more) ng = (uint32_t)blk_groups(p, b);
+  const int per_acc = acc_stages<P>(p);
+  Ring r, rt;
+  uint32_t at = 0, d = tmem;  // the stage's offset in 16-byte units, the accumulator
+  int q, b;
+  bool ok = true;
+  for (int i = 0; ok && unit_at(p, c, i, q, b); ++i) {
+    const uint32_t ng = (uint32_t)blk_groups(p, b);
+    const uint32_t idesc = idesc_f32acc(1u, 2 * kF, 16u * ng), step = ng * ((P * 256u) >> 4);
+    int kk = 0, left = J;  // slab, its slices to come (n_last > 0: the first slab has them all)
+    int in_acc = 0;                                      // stages in the accumulator
+    while (kk < n_slab) {
+      if (in_acc == 0)
+        ok = bar_wait2(full + 8 * r.slot, r.phase, t_empty + 8 * rt.slot, rt.phase ^ 1, abort, err);
+      else
+        ok = bar_wait(full + 8 * r.slot, r.phase, abort, err);
+      if (!ok) break;
+      tc_fence_after();
+      const int n = min(kps, left);
+      stage_mmas<P, true>(n, d, a0 + at, ah, b0 + at, wh, ap, step, idesc, in_acc == 0);
+      if constexpr (P > 1) stage_mmas<P, false>(n, d, a0 + at, ah, b0 + at, wh, ap, step, idesc, false);
+      mma_commit_pair_mc(empty + 8 * r.slot, 3);
+      at += stage;
+      r.next(NS);
+      if (r.slot == 0) at = 0;
+      left -= n;
+      if (left == 0) {
+        ++kk;
+        left = 16 * kk < n_last ? J : J - 1;
       }
-      js = 16 * kk < n_last ? J : J - 1;
+      if (++in_acc == per_acc || kk == n_slab) {
+        mma_commit_pair_mc(t_full + 8 * rt.slot, 3);
+        in_acc = 0;
+        d += 2 * kBlockBins;
+        rt.next(kNacc);
+        if (rt.slot == 0) d = tmem;
+      }
     }
-    const bool ok_a = bar_done(a_full + 8 * ra.slot, ra.phase), ok_b = bar_done(b_full + 8 * rb.slot, rb.phase),
-               ok_t = bar_done(t_empty + 8 * rt.slot, rt.phase ^ 1);
-    switch (n) {
-      case 1: chunk_mmas<1>(acc, a, ah, w, wh, ap, step, idesc); break;
-      case 2: chunk_mmas<2>(acc, a, ah, w, wh, ap, step, idesc); break;
-      case 3: chunk_mmas<3>(acc, a, ah, w, wh, ap, step, idesc); break;
-      default: chunk_mmas<4>(acc, a, ah, w, wh, ap, step, idesc); break;
-    }
-    mma_commit_pair_mc(done_b, 3);
-    mma_commit_pair_mc(done_t, 3);
-    if (slab_end) mma_commit_pair_mc(done_a, 3);
-    ready = ok_a && ok_b && ok_t;
   }
   // no pair MMA may still be running when either CTA releases TMEM
   mma_commit_pair_mc(bar_at(p, c, B.drain), 3);
@@ -402,86 +444,93 @@ static __device__ __forceinline__ void copy_quad(uint32_t dst, const float* src,
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid) : "memory");
 }
 
-// Rows [r0, r0 + kStageRows) of a slab (column r of lane quad qd, row u0 + 8 k)
-// into the warp's staging area.  Four lanes take the 16 samples of a row (64
-// contiguous bytes), so a warp's copies read whole sectors of 8 rows.
-static __device__ __forceinline__ void stage_rows(const SlabParams& p, const float* src, int nsamp, int rows, int r,
-                                                  uint32_t st, int r0, int u0) {
-  int s = (r0 + u0) * p.H + r;
-  const int n = min(rows - r0, kStageRows);
+// A stage's sample rows [0, rows) (column r of lane quad qd, row u0 + 8 k; s0:
+// sample of row 0, column r) into the warp's own area.  Four lanes take the 16
+// samples of a row (64 contiguous bytes), so a warp's copies read whole sectors
+// of 8 rows.
+template <int TW>
+static __device__ __forceinline__ void stage_rows(const SlabParams& p, const float* src, int nsamp, int rows, bool live,
+                                                  int s0, uint32_t to, int u0) {
+  int s = s0 + u0 * p.H;
+  if (s0 + rows * p.H <= nsamp && p.H % 16 == 0) {  // (the same for all lanes) no sample past the clip's end
+    const float* from = src + s;
 #pragma unroll 4
-  for (int u = u0; u < n; u += 8, s += 8 * p.H, st += 512) {
-    const int left = r < p.H ? min(max(nsamp - s, 0), 4) : 0;  // samples of the quad before the clip's end
-    copy_quad(st, src + (left ? s : 0), 4 * left);
+    for (int u = u0; u < rows; u += 8 * TW, from += 8 * TW * p.H, to += 512 * TW) copy_quad(to, from, 16);
+  } else {
+#pragma unroll 2
+    for (int u = u0; u < rows; u += 8 * TW, s += 8 * TW * p.H, to += 512 * TW) {
+      const int left = live ? min(max(nsamp - s, 0), 4) : 0;  // samples of the quad before the clip's end
+      copy_quad(to, src + (left ? s : 0), 4 * left);
+    }
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// ---- converters: warp w takes slabs w, w + ncv, ... of the CTA's stream.  Its
-// copies of the next slab are in flight while it waits for that slab's slot;
-// every lane converts what it copied itself.  Quad qd of row u goes, four BF16
+// ---- converters: team w takes stages w, w + ncv, ... of the CTA's stream (its
+// warps every other group of 8 rows).  The copies of the next one are in flight
+// while a warp waits for that stage's place; every lane converts what it copied itself.  Quad qd of row u goes, four BF16
 // values of each part, as 8 bytes to core column qd / 2, row u.
 template <int P>
 static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars& B) {
-  const int w = (int)(threadIdx.x >> 5) - kCvtWarp0 - (threadIdx.x >= 32 * kMmaWarp ? 1 : 0),
-            lane = threadIdx.x & 31;
-  const int qd = lane & 3, u0 = lane >> 2;
-  const uint32_t to = c.sbase + p.off_a + (uint32_t)(qd >> 1) * p.lbo_a + (uint32_t)(qd & 1) * 8u + 16u * u0;
-  const uint32_t st = c.sbase + p.off_st + w * kStageBytes + 16u * lane;
+  constexpr int TW = team_warps(P);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cw = warp - kEpiWarps - (warp > kMmaWarp ? 1 : 0) - (warp > kBWarp ? 1 : 0);  // converter warp
+  const int w = cw / TW;
+  const int qd = lane & 3, u0 = (lane >> 2) + 8 * (cw % TW);
+  const uint32_t to = c.sbase + (uint32_t)(qd >> 1) * p.lbo_a + (uint32_t)(qd & 1) * 8u + 16u * u0;
+  const uint32_t raw = c.sbase + p.off_raw + w * kRawBytes + 64u * u0 + 16u * qd;
   const uint32_t part = p.a_part;
   if (w >= p.ncv) return;
-  int q, b, i = 0, kk = w;  // unit ordinal and slab of it
-  Ring ra;
-  for (int k = 0; k < w; ++k) ra.next(p.NA);
-  while (kk >= p.n_slab) {
-    kk -= p.n_slab;
-    ++i;
-  }
-  if (!unit_at(p, c, i, q, b)) return;
-  TileDesc td = tile_of(p, c, q);
-  int rows = td.n_frames > 0 ? td.n_frames + p.J - 1 : 0;
-  stage_rows(p, p.wave + td.in_off, td.n_samples, rows, 16 * kk + 4 * qd, st, 0, u0);
-  for (;;) {
-    if (!warp_wait(bar_at(p, c, B.a_empty + ra.slot), ra.phase ^ 1, c.abort, p.err)) break;
-    const uint32_t slot = to + ra.slot * p.a_slot;
-    for (int r0 = 0; r0 < rows; r0 += kStageRows) {
-      if (r0 > 0) stage_rows(p, p.wave + td.in_off, td.n_samples, rows, 16 * kk + 4 * qd, st, r0, u0);
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      const int n = min(rows - r0, kStageRows);
-      uint32_t at = slot + 16u * r0, from = st;
+  int q = 0, b, i = 0, kk = 0, j0 = 0;  // unit ordinal, slab, first slice
+  Ring r;
+  TileDesc td;
+  bool more = unit_at(p, c, 0, q, b);
+  if (more) td = tile_of(p, c, q);
+  auto step = [&](int n) {  // n stages on
+    for (; more && n > 0; --n) {
+      r.next(p.NS);
+      j0 += p.kps;
+      if (j0 < slab_steps(p, kk)) continue;
+      j0 = 0;
+      if (++kk < p.n_slab) continue;
+      kk = 0;
+      const int was = q;
+      more = unit_at(p, c, ++i, q, b);
+      if (more && q != was) td = tile_of(p, c, q);
+    }
+  };
+  int rows = 0;
+  auto copy = [&] {
+    rows = td.n_frames > 0 ? td.n_frames + min(p.kps, slab_steps(p, kk) - j0) - 1 : 0;
+    const int col = 16 * kk + 4 * qd;
+    stage_rows<TW>(p, p.wave + td.in_off, td.n_samples, rows, col < p.H, j0 * p.H + col, raw, u0);
+  };
+  step(w);
+  if (more) copy();
+  while (more) {
+    if (!warp_wait(bar_at(p, c, B.empty + r.slot), r.phase ^ 1, c.abort, p.err)) break;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    uint32_t at = to + r.slot * p.stage, from = raw;
 #pragma unroll 2
-      for (int u = u0; u < n; u += 8, at += 128, from += 512) {
-        float a0, a1, a2, a3;
-        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a0), "=f"(a1), "=f"(a2), "=f"(a3) : "r"(from));
+    for (int u = u0; u < rows; u += 8 * TW, at += 128 * TW, from += 512 * TW) {
+      float a0, a1, a2, a3;
+      asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a0), "=f"(a1), "=f"(a2), "=f"(a3) : "r"(from));
 #pragma unroll
-        for (int t = 0; t < P; ++t) {
-          const uint32_t h0 = pack2(a0, a1), h1 = pack2(a2, a3);
-          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + t * part), "r"(h0), "r"(h1) : "memory");
-          if (t + 1 < P) {
-            a0 -= lo_f(h0);
-            a1 -= hi_f(h0);
-            a2 -= lo_f(h1);
-            a3 -= hi_f(h1);
-          }
+      for (int t = 0; t < P; ++t) {
+        const uint32_t h0 = pack2(a0, a1), h1 = pack2(a2, a3);
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + t * part), "r"(h0), "r"(h1) : "memory");
+        if (t + 1 < P) {
+          a0 -= lo_f(h0);
+          a1 -= hi_f(h0);
+          a2 -= lo_f(h1);
+          a3 -= hi_f(h1);
         }
       }
     }
     fence_proxy_async();
-    warp_arrive_leader(bar_at(p, c, B.a_full + ra.slot));
-    // the warp's next slab
-    for (int k = 0; k < p.ncv; ++k) ra.next(p.NA);
-    const int before = i;
-    kk += p.ncv;
-    while (kk >= p.n_slab) {
-      kk -= p.n_slab;
-      ++i;
-    }
-    if (i != before) {
-      if (!unit_at(p, c, i, q, b)) break;
-      td = tile_of(p, c, q);
-      rows = td.n_frames > 0 ? td.n_frames + p.J - 1 : 0;
-    }
-    stage_rows(p, p.wave + td.in_off, td.n_samples, rows, 16 * kk + 4 * qd, st, 0, u0);
+    warp_arrive_leader(bar_at(p, c, B.full + r.slot));
+    step(p.ncv);
+    if (more) copy();
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");  // no copy is in flight when the CTA exits
 }
@@ -541,6 +590,13 @@ static __device__ __forceinline__ void ld_wait8(float (&a)[8], float (&b)[8]) {
                : "memory");
 }
 
+// 32 bytes, one sector (address 32-byte aligned).
+static __device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+
 // ---- epilogue: adds the chunks of each unit, then power, log, (DCT) and store
 template <int P, bool MFCC>
 static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& c, const SlabBars& B, uint32_t tmem) {
@@ -556,157 +612,204 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
     const TileDesc td = tile_of(p, c, q);
     const int ng = blk_groups(p, b);
     const int g_n = ng / 2, g_lo = half * g_n;  // (blocks hold an even number of groups)
-    float acc[kGroupsPerWarp][2][8];
-#pragma unroll
-    for (int g = 0; g < kGroupsPerWarp; ++g)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) acc[g][0][e] = acc[g][1][e] = 0.f;
-    bool ok = true;
-    for (int kk = 0; ok && kk < p.n_slab; ++kk) {
-      const int js = slab_steps(p, kk);
-      for (int j0 = 0; j0 < js; j0 += p.kps) {
-        if (!warp_wait(bar_at(p, c, B.t_full + rt.slot), rt.phase, c.abort, p.err)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t t0 = tl + rt.slot * 2 * kBlockBins + 8 * g_lo;
-#pragma unroll
-        for (int g = 0; g < kGroupsPerWarp; ++g)
-          if (g < g_n) {
-            float re[8], im[8];
-            tmem_ld8(t0 + 8 * g, re);
-            tmem_ld8(t0 + 8 * ng + 8 * g, im);
-            ld_wait8(re, im);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              acc[g][0][e] += re[e];
-              acc[g][1][e] += im[e];
-            }
-          }
-        tc_fence_before();
-        warp_arrive_leader(bar_at(p, c, B.t_empty + rt.slot));
-        rt.next(kNacc);
-      }
-    }
-    if (!ok) break;
     const bool valid = row < td.n_frames;
     const int m_lo = 8 * (b * p.wbg + g_lo);  // first bin of this warp
-    bool finite = true;
-#pragma unroll
-    for (int g = 0; g < kGroupsPerWarp; ++g)
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float s = fmaf(acc[g][0][e], acc[g][0][e], acc[g][1][e] * acc[g][1][e]);
-        finite = finite && s < __int_as_float(0x7f800000);
-        acc[g][0][e] = __logf(s + p.eps);
+    if constexpr (P < 3) {
+      // the unit's one or two accumulators, group by group straight to the log
+      // and the row (as the other kernels of these forms evaluate it)
+      const uint32_t slot0 = rt.slot, t0 = tl + slot0 * 2 * kBlockBins + 8 * g_lo;
+      if (!warp_wait(bar_at(p, c, B.t_full + rt.slot), rt.phase, c.abort, p.err)) break;
+      rt.next(kNacc);
+      const bool two = P == 2 && unit_stages(p) > 1;
+      const uint32_t slot1 = rt.slot, t1 = tl + slot1 * 2 * kBlockBins + 8 * g_lo;
+      if (two) {
+        if (!warp_wait(bar_at(p, c, B.t_full + rt.slot), rt.phase, c.abort, p.err)) break;
+        rt.next(kNacc);
       }
-    const float* x = p.wave + td.in_off + (long long)row * p.H;
-    if constexpr (!MFCC) {
+      tc_fence_after();
       float* orow = p.out + (size_t)(td.out_row + row) * p.n_out;
-      if (valid) {
 #pragma unroll
-        for (int g = 0; g < kGroupsPerWarp; ++g)
-          if (g < g_n) {
+      for (int g = 0; g < kGroupsPerWarp; ++g)
+        if (g < g_n) {
+          float v[8], im[8];
+          tmem_ld8(t0 + 8 * g, v);
+          tmem_ld8(t0 + 8 * ng + 8 * g, im);
+          ld_wait8(v, im);
+          if (two) {
+            float r2[8], i2[8];
+            tmem_ld8(t1 + 8 * g, r2);
+            tmem_ld8(t1 + 8 * ng + 8 * g, i2);
+            ld_wait8(r2, i2);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              v[e] += r2[e];
+              im[e] += i2[e];
+            }
+          }
+          if (g + 1 == g_n) {
+            tc_fence_before();
+            warp_arrive_leader(bar_at(p, c, B.t_empty + slot0));
+            if (two) warp_arrive_leader(bar_at(p, c, B.t_empty + slot1));
+          }
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[e] = fast_ln(fmaf(v[e], v[e], fmaf(im[e], im[e], p.eps)));
+          if (valid) {
             const int m = m_lo + 8 * g;
             if (vec8 && m + 8 <= p.M) {
-              asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(orow + m),
-                           "f"(acc[g][0][0]), "f"(acc[g][0][1]), "f"(acc[g][0][2]), "f"(acc[g][0][3]),
-                           "f"(acc[g][0][4]), "f"(acc[g][0][5]), "f"(acc[g][0][6]), "f"(acc[g][0][7])
-                           : "memory");
+              store8(orow + m, v);
             } else {
 #pragma unroll
               for (int e = 0; e < 8; ++e)
-                if (m + e < p.M) orow[m + e] = acc[g][0][e];
+                if (m + e < p.M) orow[m + e] = v[e];
             }
           }
-      }
-      for (unsigned left = __ballot_sync(0xffffffffu, !finite && valid); left; left &= left - 1) {
-        const int l = __ffs(left) - 1, end = min(m_lo + 8 * g_n, p.M);
-        const float2 v = redo_row(p, x + (long long)(l - lane) * p.H, m_lo, end);
-        float* o = orow + (long long)(l - lane) * p.n_out + m_lo;
-        if (m_lo + lane < end) o[lane] = v.x;
-        if (m_lo + 32 + lane < end) o[32 + lane] = v.y;
-      }
+        }
     } else {
-      for (unsigned left = __ballot_sync(0xffffffffu, !finite && valid); left; left &= left - 1) {
-        const int l = __ffs(left) - 1;
-        const float2 v = redo_row(p, x + (long long)(l - lane) * p.H, m_lo, min(m_lo + 8 * g_n, p.M));
+      float acc[kGroupsPerWarp][2][8];
+      bool ok = true;
 #pragma unroll
         for (int g = 0; g < kGroupsPerWarp; ++g)
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float t = __shfl_sync(0xffffffffu, 8 * g + e < 32 ? v.x : v.y, (8 * g + e) & 31);
-            if (lane == l) acc[g][0][e] = t;
+          for (int e = 0; e < 8; ++e) acc[g][0][e] = acc[g][1][e] = 0.f;
+        for (int left = unit_stages(p); left > 0; --left) {
+          if (!warp_wait(bar_at(p, c, B.t_full + rt.slot), rt.phase, c.abort, p.err)) {
+            ok = false;
+            break;
           }
-      }
-      // bins past M (zero basis rows) take no part, whatever their log is
-#pragma unroll
-      for (int g = 0; g < kGroupsPerWarp; ++g)
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (m_lo + 8 * g + e >= p.M) acc[g][0][e] = 0.f;
-      // C = ln(S + eps) D^T over this warp's bins, eight coefficients at a time.
-      // The second warp of a lane quarter hands its part to the first through
-      // one of two buffers; the first adds both (and, above 80 bins, what the
-      // blocks before left in the row) and stores.
-      float* orow = p.out + (size_t)(td.out_row + row) * p.n_mfcc;
-      const bool add = b > 0 && valid && !half;
-      float prev[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) prev[k] = add && k < p.n_mfcc ? orow[k] : 0.f;
-      for (int k0 = 0; k0 < p.n_mfcc; k0 += 8) {
-        float v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          v[k] = prev[k];
-          prev[k] = add && k0 + 8 + k < p.n_mfcc ? orow[k0 + 8 + k] : 0.f;
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float* d = dct + (size_t)min(k0 + k, p.n_mfcc - 1) * (8 * p.groups) + m_lo;
+          tc_fence_after();
+          const uint32_t t0 = tl + rt.slot * 2 * kBlockBins + 8 * g_lo;
 #pragma unroll
           for (int g = 0; g < kGroupsPerWarp; ++g)
             if (g < g_n) {
-              const float4 d0 = *reinterpret_cast<const float4*>(d + 8 * g);
-              const float4 d1 = *reinterpret_cast<const float4*>(d + 8 * g + 4);
-              const float* l = acc[g][0];
-              v[k] = fmaf(l[0], d0.x, v[k]);
-              v[k] = fmaf(l[1], d0.y, v[k]);
-              v[k] = fmaf(l[2], d0.z, v[k]);
-              v[k] = fmaf(l[3], d0.w, v[k]);
-              v[k] = fmaf(l[4], d1.x, v[k]);
-              v[k] = fmaf(l[5], d1.y, v[k]);
-              v[k] = fmaf(l[6], d1.z, v[k]);
-              v[k] = fmaf(l[7], d1.w, v[k]);
+              float re[8], im[8];
+              tmem_ld8(t0 + 8 * g, re);
+              tmem_ld8(t0 + 8 * ng + 8 * g, im);
+              ld_wait8(re, im);
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                acc[g][0][e] += re[e];
+                acc[g][1][e] += im[e];
+              }
+            }
+          tc_fence_before();
+          warp_arrive_leader(bar_at(p, c, B.t_empty + rt.slot));
+          rt.next(kNacc);
+        }
+      if (!ok) break;
+      bool finite = true;
+#pragma unroll
+      for (int g = 0; g < kGroupsPerWarp; ++g)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float s = fmaf(acc[g][0][e], acc[g][0][e], acc[g][1][e] * acc[g][1][e]);
+          finite = finite && s < __int_as_float(0x7f800000);
+          acc[g][0][e] = __logf(s + p.eps);
+        }
+      const float* x = p.wave + td.in_off + (long long)row * p.H;
+      if constexpr (!MFCC) {
+        float* orow = p.out + (size_t)(td.out_row + row) * p.n_out;
+        if (valid) {
+#pragma unroll
+          for (int g = 0; g < kGroupsPerWarp; ++g)
+            if (g < g_n) {
+              const int m = m_lo + 8 * g;
+              if (vec8 && m + 8 <= p.M) {
+                store8(orow + m, acc[g][0]);
+              } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                  if (m + e < p.M) orow[m + e] = acc[g][0][e];
+              }
             }
         }
-        float* buf = reinterpret_cast<float*>(gbase + p.off_part) + rp.slot * 8 * kF + row;
-        const uint32_t full = bar_at(p, c, B.half + 4 * quarter + rp.slot), empty = full + 16;
-        if (half) {
-          if (!warp_wait(empty, rp.phase ^ 1, c.abort, p.err)) return;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) buf[k * kF] = v[k];
-          warp_arrive_local(full);
-        } else {
-          if (!warp_wait(full, rp.phase, c.abort, p.err)) return;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) v[k] += buf[k * kF];
-          warp_arrive_local(empty);
-          if (valid) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-              if (k0 + k < p.n_mfcc) orow[k0 + k] = v[k];
-          }
+        __syncwarp();  // (the rows' own stores come before the recomputed ones)
+        for (unsigned left = __ballot_sync(0xffffffffu, !finite && valid); left; left &= left - 1) {
+          const int l = __ffs(left) - 1, end = min(m_lo + 8 * g_n, p.M);
+          const float2 v = redo_row(p, x + (long long)(l - lane) * p.H, m_lo, end);
+          float* o = orow + (long long)(l - lane) * p.n_out + m_lo;
+          if (m_lo + lane < end) o[lane] = v.x;
+          if (m_lo + 32 + lane < end) o[32 + lane] = v.y;
         }
-        rp.next(2);
+      } else {
+        for (unsigned left = __ballot_sync(0xffffffffu, !finite && valid); left; left &= left - 1) {
+          const int l = __ffs(left) - 1;
+          const float2 v = redo_row(p, x + (long long)(l - lane) * p.H, m_lo, min(m_lo + 8 * g_n, p.M));
+#pragma unroll
+          for (int g = 0; g < kGroupsPerWarp; ++g)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              const float t = __shfl_sync(0xffffffffu, 8 * g + e < 32 ? v.x : v.y, (8 * g + e) & 31);
+              if (lane == l) acc[g][0][e] = t;
+            }
+        }
+        // bins past M (zero basis rows) take no part, whatever their log is
+#pragma unroll
+        for (int g = 0; g < kGroupsPerWarp; ++g)
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            if (m_lo + 8 * g + e >= p.M) acc[g][0][e] = 0.f;
+        // C = ln(S + eps) D^T over this warp's bins, eight coefficients at a time.
+        // The second warp of a lane quarter hands its part to the first through
+        // one of two buffers; the first adds both (and, above 80 bins, what the
+        // blocks before left in the row) and stores.
+        float* orow = p.out + (size_t)(td.out_row + row) * p.n_mfcc;
+        const bool add = b > 0 && valid && !half;
+        float prev[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) prev[k] = add && k < p.n_mfcc ? orow[k] : 0.f;
+        for (int k0 = 0; k0 < p.n_mfcc; k0 += 8) {
+          float v[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            v[k] = prev[k];
+            prev[k] = add && k0 + 8 + k < p.n_mfcc ? orow[k0 + 8 + k] : 0.f;
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const float* d = dct + (size_t)min(k0 + k, p.n_mfcc - 1) * (8 * p.groups) + m_lo;
+#pragma unroll
+            for (int g = 0; g < kGroupsPerWarp; ++g)
+              if (g < g_n) {
+                const float4 d0 = *reinterpret_cast<const float4*>(d + 8 * g);
+                const float4 d1 = *reinterpret_cast<const float4*>(d + 8 * g + 4);
+                const float* l = acc[g][0];
+                v[k] = fmaf(l[0], d0.x, v[k]);
+                v[k] = fmaf(l[1], d0.y, v[k]);
+                v[k] = fmaf(l[2], d0.z, v[k]);
+                v[k] = fmaf(l[3], d0.w, v[k]);
+                v[k] = fmaf(l[4], d1.x, v[k]);
+                v[k] = fmaf(l[5], d1.y, v[k]);
+                v[k] = fmaf(l[6], d1.z, v[k]);
+                v[k] = fmaf(l[7], d1.w, v[k]);
+              }
+          }
+          float* buf = reinterpret_cast<float*>(gbase + p.off_part) + rp.slot * 8 * kF + row;
+          const uint32_t full = bar_at(p, c, B.part + 4 * quarter + rp.slot), empty = full + 16;
+          if (half) {
+            if (!warp_wait(empty, rp.phase ^ 1, c.abort, p.err)) return;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) buf[k * kF] = v[k];
+            warp_arrive_local(full);
+          } else {
+            if (!warp_wait(full, rp.phase, c.abort, p.err)) return;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] += buf[k * kF];
+            warp_arrive_local(empty);
+            if (valid) {
+#pragma unroll
+              for (int k = 0; k < 8; ++k)
+                if (k0 + k < p.n_mfcc) orow[k0 + k] = v[k];
+            }
+          }
+          rp.next(2);
+        }
       }
     }
   }
 }
 
 template <int P, bool MFCC>
-__global__ void __launch_bounds__(kThreads, 1) melt_slab_kernel(const __grid_constant__ SlabParams p) {
+__global__ void __launch_bounds__(slab_threads(P), 1) melt_slab_kernel(const __grid_constant__ SlabParams p) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   Ctx c;
@@ -717,23 +820,19 @@ __global__ void __launch_bounds__(kThreads, 1) melt_slab_kernel(const __grid_con
   c.n_clusters = (int)(gridDim.x >> 1);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + p.off_misc);
   c.abort = reinterpret_cast<volatile int*>(gbase + p.off_misc + 4);
-  const SlabBars B(p.NA, p.NB);
+  const SlabBars B(p.NS);
   const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     auto bar = [&](int i) { return bar_at(p, c, i); };
-    for (int i = 0; i < p.NA; ++i) {
-      mbar_init(bar(B.a_full + i), 2);  // one converter warp of each CTA
-      mbar_init(bar(B.a_empty + i), 1);
-    }
-    for (int i = 0; i < p.NB; ++i) {
-      mbar_init(bar(B.b_full + i), c.rank == 0 ? 2 : 1);
-      mbar_init(bar(B.b_empty + i), 1);
+    for (int i = 0; i < p.NS; ++i) {
+      mbar_init(bar(B.full + i), c.rank == 0 ? 2 + 2 * team_warps(P) : 1);
+      mbar_init(bar(B.empty + i), 1);
     }
     for (int i = 0; i < kNacc; ++i) {
       mbar_init(bar(B.t_full + i), 1);
       mbar_init(bar(B.t_empty + i), 2 * kEpiWarps);
     }
-    for (int i = 0; i < 16; ++i) mbar_init(bar(B.half + i), 1);
+    for (int i = 0; i < 16; ++i) mbar_init(bar(B.part + i), 1);
     mbar_init(bar(B.drain), 1);
     *c.abort = 0;
     fence_mbar_init();
@@ -746,7 +845,7 @@ __global__ void __launch_bounds__(kThreads, 1) melt_slab_kernel(const __grid_con
     // D as [n_mfcc][8 groups] rows, zero past M
     float* d = reinterpret_cast<float*>(gbase + p.off_dct);
     const int ld = 8 * p.groups;
-    for (int i = threadIdx.x; i < p.n_mfcc * ld; i += kThreads) {
+    for (int i = threadIdx.x; i < p.n_mfcc * ld; i += slab_threads(P)) {
       const int k = i / ld, m = i - k * ld;
       d[i] = m < p.M ? p.dct[k * p.M + m] : 0.f;
     }
@@ -770,8 +869,8 @@ __global__ void __launch_bounds__(kThreads, 1) melt_slab_kernel(const __grid_con
   } else if (warp == kBWarp) {
     if (elect_one()) basis_producer<P>(p, c, B);
     __syncwarp();
-  } else if (warp >= kCvtWarp0) {
-    pdl_wait();
+  } else if (warp >= kEpiWarps) {
+    if (!p.early_inputs) pdl_wait();
     convert<P>(p, c, B);
     __syncwarp();
   } else {
