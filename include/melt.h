@@ -55,8 +55,7 @@ typedef enum { MELT_WIN_HANN_PERIODIC = 0, MELT_WIN_HANN_SYMMETRIC = 1 } melt_wi
  * this library's).  All accumulate in FP32 and take FP32 waveforms.
  *   MELT_FP32    FP32 samples x FP32 basis, each split exactly into three BF16
  *                parts, the six leading products on tcgen05 tensor cores, sums
- *                of at most four K-steps added in FP32 (CUDA cores, FFMA, for
- *                hops too short for that layout).
+ *                of at most four K-steps added in FP32.
  *   MELT_BF16    BF16 samples x BF16 basis on tcgen05 tensor cores.
  *   MELT_BF16X3  two-term BF16 splits of both operands, three products
  *                (hi*hi + hi*lo + lo*hi) on tcgen05 tensor cores.
@@ -147,6 +146,11 @@ melt_status melt_basis_get_fp64(const melt_basis* basis, double* freqs, double* 
  *                    tiles ahead the spans are prefetched into L2 besides;
  *                    basis_slots and ksteps_per_slot are ignored).  0: one
  *                    CTA per MMA.
+ *                    With basis_resident 0, BF16 and BF16X3 bases whose default
+ *                    layout that is run a kernel that streams both operands in
+ *                    slabs of 16 sample columns (its rings take what shared
+ *                    memory holds: a_buffers, basis_slots and ksteps_per_slot
+ *                    are ignored).
  *   schedule         CTA pairs only.  0: static, cluster c takes pairs c,
  *                    c + C, c + 2C, ... (C clusters).  1: dynamic, cluster c
  *                    takes pair c, then claims each next pair from a
@@ -239,8 +243,8 @@ enum { MELT_FWD_INPUT_READY = 1 };
  *          converts samples, and runs its MMAs, while the preceding kernel
  *          drains; it still stores features only after that kernel has
  *          finished.  A batch produced by a kernel on `stream` (for example
- *          melt_pad_reflect) must not use the flag.  The FP32 form and the
- *          dynamic pair schedule ignore it.
+ *          melt_pad_reflect) must not use the flag.  The dynamic pair
+ *          schedule ignores it.
  *   Other arguments and errors as melt_forward; MELT_ERR_ARG for an unknown flag.
  */
 melt_status melt_forward_ex(melt_basis* basis, const float* wave, const int64_t* offsets,

@@ -55,12 +55,12 @@ struct melt_basis {
   std::vector<double> freqs;   // [M]
   std::vector<double> w64;     // [2M][N]: W_r rows then W_i rows
   // device data
-  int mj = 0, mp = 0;          // SIMT: 16*mj padded mels
-  float* d_w32 = nullptr;      // SIMT basis [N][2*mp]
+  int mj = 0, mp = 0;          // FP32 basis: 16*mj padded mels
+  float* d_w32 = nullptr;      // FP32 basis [N][2*mp]
   float* d_dct = nullptr;      // [K][M]
   int* d_err = nullptr;        // latched kernel errors
   TcBasis tc;                  // tensor-core operand images (BF16/FP8 forms)
-  SlabBasis slab;              // operands of the slab kernel (no image: it does not run for this basis)
+  SlabBasis slab;              // operands of the slab kernel (no image where it does not run for this basis)
   Staging staging[kStagingSlots];
   int next_slot = 0;
   std::vector<TileDesc> plan;  // host scratch for planning
@@ -196,15 +196,16 @@ melt_status create_common(double sr, int n_fft, int hop, const double* freqs, in
     TcConfig c{n_fft, hop, n_freqs, precision, n_mfcc, stft_bands};
     st = tc_build(&b->tc, c, b->w64.data());
   }
-  // operands of the slab kernel: the FP32 form, and log-Mel of split BF16, and
-  // of BF16 where no layout keeps the basis in shared memory
+  // operands of the slab kernel: the FP32 form, and (where its rings fit) log-Mel
+  // of bases for which no layout keeps the basis in shared memory
   if (st == MELT_OK && precision == MELT_FP32)
     st = slab_build(&b->slab, n_fft, hop, n_freqs, n_mfcc, 3, b->w64.data());
   melt_plan first;
   if (st == MELT_OK && (precision == MELT_BF16 || precision == MELT_BF16X3) && n_freqs <= 128 && n_mfcc == 0 &&
-      stft_bands == 0 && tc_current_plan(&b->tc, &first) && (precision == MELT_BF16X3 || !first.basis_resident)) {
+      stft_bands == 0 && tc_current_plan(&b->tc, &first) && !first.basis_resident) {
     st = slab_build(&b->slab, n_fft, hop, n_freqs, 0, precision == MELT_BF16X3 ? 2 : 1, b->w64.data());
-    if (b->slab.d_img) b->tc.slab = &b->slab;
+    if (st == MELT_OK) b->tc.slab = &b->slab;
+    else if (st == MELT_ERR_UNSUPPORTED) st = MELT_OK;
   }
   if (st == MELT_OK) {
     cudaError_t e = melt::dev_alloc(&b->d_err, sizeof(int));
@@ -226,7 +227,7 @@ int64_t frames_of(const melt_basis* b, int64_t len) {
   return (len - b->n_fft) / b->hop + 1;
 }
 
-// The FP32 kernel's CTAs take tiles in list order, round by round, and a
+// The CUDA-core kernel's CTAs take tiles in list order, round by round, and a
 // tile costs it in proportion to its frames (warps past the tile's end
 // idle); with the longest tiles first, the last, partly filled round holds
 // the short tiles that end clips.  Tiles are independent (each writes its
@@ -235,15 +236,13 @@ void order_longest_first(TileDesc* t, long long n) {
   std::stable_sort(t, t + n, [](const TileDesc& a, const TileDesc& b) { return a.n_frames > b.n_frames; });
 }
 
-// The FP32 form over n_tiles device descriptors.  The tensor-core kernel with
-// three-part split operands runs wherever its rings fit shared memory (64 x 30 s,
-// N 400, 80 bins: 99 us against 508 us on the CUDA cores; 8 x 1 s: 13.5 against
-// 52 us; one 160 s clip, N 1200, 128 bins, 40 MFCCs: 59 against 421 us).  Hops
-// so short that a slab of all Z rows does not fit twice, and the raw
-// projections (mode 1), run on the CUDA cores.
+// The FP32 form over n_tiles device descriptors: the slab kernel with three-part
+// split operands (64 x 30 s, N 400, 80 bins: 97 us against 508 us as FFMAs on the
+// CUDA cores; 8 x 1 s: 13.5 against 52 us; one 160 s clip, N 1200, 128 bins, 40
+// MFCCs: 59 against 421 us), or (mode 1) the raw projections on the CUDA cores.
 cudaError_t launch_fp32(melt_basis* b, const float* wave, const TileDesc* tiles, int n_tiles, float* out, int mode,
                         unsigned flags, cudaStream_t stream) {
-  if (mode == 0 && b->slab.d_img) {
+  if (mode == 0) {
     SlabLaunch L;
     L.wave = wave; L.tiles = tiles; L.n_tiles = n_tiles; L.out = out;
     L.dct = b->d_dct; L.w32 = b->d_w32; L.mp = b->mp;
@@ -253,10 +252,8 @@ cudaError_t launch_fp32(melt_basis* b, const float* wave, const TileDesc* tiles,
   }
   SimtParams p;
   p.wave = wave; p.tiles = tiles; p.n_tiles = n_tiles;
-  p.w32 = b->d_w32; p.dct = b->d_dct; p.out = out;
-  p.n_fft = b->n_fft; p.hop = b->hop; p.n_mels = b->n_mels; p.mp = b->mp;
-  p.n_mfcc = b->n_mfcc; p.n_out = b->n_mfcc ? b->n_mfcc : b->n_mels;
-  p.eps = (float)b->eps; p.mode = mode;
+  p.w32 = b->d_w32; p.out = out;
+  p.n_fft = b->n_fft; p.hop = b->hop; p.n_mels = b->n_mels;
   return launch_simt(p, b->mj, b->sm_count, stream);
 }
 

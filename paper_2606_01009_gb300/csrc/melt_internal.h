@@ -29,17 +29,14 @@ static_assert(sizeof(TileDesc) == 32, "TileDesc is 32 bytes");
 // Error bits latched by kernels in the per-basis device error word.
 enum : int { kErrTimeout = 1, kErrBadTile = 2 };
 
-// Parameters of the FP32 SIMT kernel.
+// Parameters of the FP32 SIMT kernel (raw R | I projections).
 struct SimtParams {
   const float* wave;
   const TileDesc* tiles;
   int n_tiles;
   const float* w32;   // [n_fft][2*mp]: interleaved (W_r[m][n], W_i[m][n]) per mel, zero-padded to mp mels
-  const float* dct;   // [n_mfcc][n_mels] or nullptr
   float* out;
-  int n_fft, hop, n_mels, mp, n_mfcc, n_out;
-  float eps;
-  int mode;           // 0: log-Mel / MFCC, 1: raw R|I components
+  int n_fft, hop, n_mels;
 };
 
 // Every device allocation and every page-locked host allocation the library
@@ -59,7 +56,6 @@ inline cudaError_t host_alloc_pinned(T** p, size_t bytes) {
 // Launch the FP32 SIMT kernel for `p` (grid picked by the caller).
 // Persistent launch: as many CTAs as fit on sm_count SMs (at most one per tile).
 cudaError_t launch_simt(const SimtParams& p, int mj, int sm_count, cudaStream_t stream);
-int simt_smem_bytes(int mj, int n_mels, int n_mfcc);
 
 }  // namespace melt
 

@@ -1,11 +1,9 @@
-// Plain FP32 MelT on CUDA cores (FFMA, FP32 accumulate): the raw projections
-// (melt_forward_components), and the FP32 form at hops so short that the
-// tensor-core kernel's slabs do not fit shared memory.
+// Raw FP32 projections (melt_forward_components) on CUDA cores (FFMA, FP32
+// accumulate).
 //
 // Computes the projection of Sec. III-A, Eq. 6 ([R | I] = X [W_r; W_i]^T)
 // with implicit framing: frame f of a tile is read straight from the packed
-// waveform at in_off + f*H, never materialised in global memory.  The power
-// (Eq. 7), log (Eq. 8) and optional DCT-II (Eq. 9) are fused in the epilogue.
+// waveform at in_off + f*H, never materialised in global memory.
 //
 // CTA tile: 128 frames x all 2M basis rows; 256 threads as 16 (frame groups
 // of 8) x 16 (mel lanes); thread (ty, tx) owns frames 8ty..8ty+7 and mels
@@ -110,7 +108,7 @@ __global__ void __launch_bounds__(kThreads, MJ <= 5 ? 2 : 1) melt_simt_kernel(Si
 #pragma unroll
       for (int j = 0; j < MJ; ++j) acc[i][j][0] = acc[i][j][1] = 0.f;
 
-    __syncthreads();  // the previous tile's readers of both buffers (and the MFCC staging) are done
+    __syncthreads();  // the previous tile's readers of both buffers are done
     simt_copy_chunk<MJ>(p, td, 0, tid, smem, smem + kXs);
     cp_async_commit();
     int b = 0;
@@ -147,59 +145,15 @@ __global__ void __launch_bounds__(kThreads, MJ <= 5 ? 2 : 1) melt_simt_kernel(Si
       __syncthreads();  // this buffer's readers are done before it is refilled
     }
 
-    // ---- epilogue: power (Eq. 7), log (Eq. 8), optional DCT-II (Eq. 9)
-    if (p.mode == 1) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int f = ty * 8 + i;
-        if (f >= td.n_frames) continue;
-        float* orow = p.out + (size_t)(td.out_row + f) * (2 * M);
-#pragma unroll
-        for (int j = 0; j < MJ; ++j) {
-          const int m = tx + 16 * j;
-          if (m < M) { orow[m] = acc[i][j][0]; orow[M + m] = acc[i][j][1]; }
-        }
-      }
-      continue;
-    }
-    if (p.n_mfcc == 0) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int f = ty * 8 + i;
-        if (f >= td.n_frames) continue;
-        float* orow = p.out + (size_t)(td.out_row + f) * p.n_out;
-#pragma unroll
-        for (int j = 0; j < MJ; ++j) {
-          const int m = tx + 16 * j;
-          const float s = fmaf(acc[i][j][0], acc[i][j][0], acc[i][j][1] * acc[i][j][1]);
-          if (m < M) orow[m] = __logf(s + p.eps);
-        }
-      }
-      continue;
-    }
-    // MFCC: stage the tile's log-Mel rows in shared memory, then apply D.
-    __syncthreads();  // every thread is done reading the chunk buffers
-    float* L = smem;  // [kF][M]
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int f = ty * 8 + i;
-#pragma unroll
-      for (int j = 0; j < MJ; ++j) {
-        const int m = tx + 16 * j;
-        const float s = fmaf(acc[i][j][0], acc[i][j][0], acc[i][j][1] * acc[i][j][1]);
-        if (m < M) L[f * M + m] = __logf(s + p.eps);
-      }
-    }
-    __syncthreads();
-    const int K = p.n_mfcc;
     for (int i = 0; i < 8; ++i) {
       const int f = ty * 8 + i;
       if (f >= td.n_frames) continue;
-      for (int k = tx; k < K; k += 16) {
-        const float* drow = p.dct + (size_t)k * M;
-        float c = 0.f;
-        for (int m = 0; m < M; ++m) c = fmaf(L[f * M + m], __ldg(drow + m), c);
-        p.out[(size_t)(td.out_row + f) * K + k] = c;
+      float* orow = p.out + (size_t)(td.out_row + f) * (2 * M);
+#pragma unroll
+      for (int j = 0; j < MJ; ++j) {
+        const int m = tx + 16 * j;
+        if (m < M) { orow[m] = acc[i][j][0]; orow[M + m] = acc[i][j][1]; }
       }
     }
   }
@@ -207,19 +161,12 @@ __global__ void __launch_bounds__(kThreads, MJ <= 5 ? 2 : 1) melt_simt_kernel(Si
 
 }  // namespace
 
-int simt_smem_bytes(int mj, int n_mels, int n_mfcc) {
-  const int mp = 16 * mj;
-  int bytes = 2 * (kKC * (kF + kXPad) + kKC * 2 * mp) * (int)sizeof(float);  // two chunk buffers
-  if (n_mfcc > 0) {
-    const int l = kF * n_mels * (int)sizeof(float);
-    if (l > bytes) bytes = l;
-  }
-  return bytes;
-}
+// Two chunk buffers.
+static int simt_smem_bytes(int mj) { return 2 * (kKC * (kF + kXPad) + kKC * 32 * mj) * (int)sizeof(float); }
 
 template <int MJ>
 static cudaError_t launch_mj(const SimtParams& p, int sm_count, cudaStream_t stream) {
-  const int smem = simt_smem_bytes(MJ, p.n_mels, p.n_mfcc);
+  const int smem = simt_smem_bytes(MJ);
   cudaError_t e = cudaFuncSetAttribute(melt_simt_kernel<MJ>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "melt_slab_kernel.cuh"
@@ -38,8 +39,10 @@ uint32_t mfcc_bytes(const SlabParams& p, int n_mfcc) {
   return n_mfcc > 0 ? up(4u * n_mfcc * 8u * p.groups, 128) + 2u * 8u * kF * 4u : 0u;
 }
 
-// Geometry and shared-memory plan; false where two stages do not fit (never for
-// log-Mel; MFCC with a large DCT matrix).
+// Geometry and shared-memory plan.  P 3: false where two stages do not fit (three
+// or more do for every basis that can be created).  P 1, 2: false where a tile
+// has more rows than a converter copies at once, or its slabs and a few more do
+// not fit beside the basis ring.
 bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
   const int P = sb->parts;
   p.N = sb->n_fft;
@@ -50,31 +53,61 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
   p.ksteps = sb->ksteps;
   p.groups = sb->groups;
   p.n_last = p.N - (p.J - 1) * p.H;
-  // a slab's slices in equal stages
-  const int per_slab = (p.J + max_kps(P) - 1) / max_kps(P);
-  p.kps = (p.J + per_slab - 1) / per_slab;
+  // K-steps in equal stages of a slab's slices (P 3) or slots of a slice's slabs
+  const int total = P == 3 ? p.J : p.n_slab, runs = (total + max_kps(P) - 1) / max_kps(P);
+  p.kps = (total + runs - 1) / runs;
   p.step_bytes = (uint32_t)p.groups * P * 256u;
-  p.lbo_a = (uint32_t)(p.kps <= 5 ? kRowsA : kRowsA + 8) * 16u;
+  const int rows = kF + (P == 3 ? p.kps : p.J) - 1;
+  if (rows > kStageRows) return false;
+  p.lbo_a = (uint32_t)(rows <= kRowsA ? kRowsA : kRowsA + 8) * 16u;
   p.a_part = 2 * p.lbo_a;
   p.a_bytes = up(P * p.a_part, 128);
-  const int least = (p.groups + kBlockBins / 8 - 1) / (kBlockBins / 8);  // blocks, and groups of the widest one
+  const int least = (p.groups + max_groups(P) - 1) / max_groups(P);  // blocks, and groups of the widest one
   const int wbg = 2 * ((p.groups / 2 + least - 1) / least);
-  p.stage = p.a_bytes + up((uint32_t)wbg * P * 256u * p.kps, 128);
-  const uint32_t fixed = up(8u * SlabBars(kMaxStages).total, 128) + 128u + mfcc_bytes(p, n_mfcc) + 128u;
-  // as many stages as fit, each of the first kCvtTeams with a converter team's raw samples
-  for (int ns = kMaxStages; ns >= 2; --ns) {
-    const uint32_t raw = std::min(ns, kCvtTeams) * kRawBytes;
-    if (fixed + raw + ns * p.stage > kSmemMax) continue;
-    p.NS = ns;
-    p.ncv = std::min(ns, kCvtTeams);
-    p.off_raw = p.stage * ns;
-    p.off_bar = p.off_raw + raw;
-    p.off_misc = p.off_bar + up(8u * SlabBars(ns).total, 128);
-    p.off_dct = p.off_misc + 128u;
-    p.off_part = p.off_dct + up(4u * n_mfcc * 8u * p.groups, 128);
-    return true;
+  p.nacc = wbg <= 10 ? 3 : 2;
+  p.acc_cols = wbg <= 10 ? 160 : 256;
+  const uint32_t basis = up((uint32_t)wbg * P * 256u * p.kps, 128);
+  const uint32_t fixed = up(8u * SlabBars(P == 3 ? kMaxStages : kMaxA, P == 3 ? 0 : kMaxB).total, 128) + 128u +
+                         mfcc_bytes(p, n_mfcc) + 128u;
+  uint32_t end = 0;  // of the rings
+  if (P == 3) {
+    p.stage = p.a_bytes + basis;
+    // as many stages as fit, each of the first kMaxTeams with a converter warp's raw samples
+    for (int ns = kMaxStages; ns >= 2 && !end; --ns) {
+      p.NS = ns;
+      p.ncv = std::min(ns, kMaxTeams);
+      p.tw = 1;
+      if (fixed + p.ncv * kRawBytes + ns * p.stage <= kSmemMax) end = p.stage * ns;
+    }
+  } else {
+    p.stage = p.a_bytes;
+    p.b_slot = basis;
+    // As many converter teams and slabs beside the tile in use (up to another
+    // tile of them) as leave three basis slots; then more of those.  Measured,
+    // split BF16 256 x 10 s: 6 / 4 / 3 teams 76 / 77 / 81 us with 5 slabs, 2 / 8
+    // slabs (fewer teams) 82 / 78; BF16 at 22.05 kHz, 64 x 20 s: 10 / 7 / 4 slabs
+    // 42.4 / 43.8 / 45.2.
+    for (int least_nb = 3; least_nb >= 2; --least_nb)
+      for (int teams : {6, 4, 3, 2}) {
+        const uint32_t other = fixed + teams * kRawBytes;
+        if (end || other + least_nb * basis >= kSmemMax) continue;
+        const int na = std::min({(int)((kSmemMax - other - least_nb * basis) / p.stage), 2 * p.n_slab, kMaxA});
+        if (na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
+        p.NS = na;
+        p.NB = std::min<int>(kMaxB, (int)((kSmemMax - other - na * p.stage) / basis));
+        p.ncv = teams;
+        p.tw = cvt_warps(P) / teams;
+        p.off_b = p.stage * na;
+        end = p.off_b + basis * p.NB;
+      }
   }
-  return false;
+  if (!end) return false;
+  p.off_raw = end;
+  p.off_bar = p.off_raw + p.ncv * kRawBytes;
+  p.off_misc = p.off_bar + up(8u * SlabBars(p.NS, p.NB).total, 128);
+  p.off_dct = p.off_misc + 128u;
+  p.off_part = p.off_dct + up(4u * n_mfcc * 8u * p.groups, 128);
+  return true;
 }
 
 uint32_t smem_bytes(const SlabParams& p, int n_mfcc) { return p.off_dct + mfcc_bytes(p, n_mfcc) + 128u; }
@@ -93,23 +126,31 @@ melt_status slab_build(SlabBasis* sb, int n_fft, int hop, int n_mels, int n_mfcc
   sb->ksteps = sb->n_slab * (sb->J - 1) + (n_last + 15) / 16;
   SlabParams p;
   std::memset(&p, 0, sizeof(p));
-  if (!plan(sb, n_mfcc, p)) return MELT_OK;
+  if (!plan(sb, n_mfcc, p)) return MELT_ERR_UNSUPPORTED;
   const size_t half = (size_t)sb->ksteps * p.step_bytes;
   std::vector<uint16_t> img(half);  // two halves of half / 2 values each
+  // K-steps slab by slab over the slices (P 3), or slice by slice over the slabs
+  std::vector<std::pair<int, int>> steps;  // (slab, slice)
+  if (parts == 3) {
+    for (int kk = 0; kk < sb->n_slab; ++kk)
+      for (int j = 0; j < (16 * kk < n_last ? sb->J : sb->J - 1); ++j) steps.push_back({kk, j});
+  } else {
+    for (int j = 0; j < sb->J; ++j)
+      for (int kk = 0; kk < sb->n_slab && (j + 1 < sb->J || 16 * kk < n_last); ++kk) steps.push_back({kk, j});
+  }
   for (int h = 0; h < 2; ++h) {
     uint16_t* step = img.data() + (size_t)h * (half / 2);
-    for (int kk = 0; kk < sb->n_slab; ++kk) {
-      const int js = 16 * kk < n_last ? sb->J : sb->J - 1;
-      for (int j = 0; j < js; ++j, step += p.step_bytes / 2)
-        for (int m = 0; m < n_mels; ++m) {
-          const double* w = w64 + ((size_t)h * n_mels + m) * n_fft;
-          uint16_t* grp = step + (size_t)(m >> 3) * parts * 128 + (m & 7) * 8;
-          for (int e = 0; e < 16; ++e) {
-            const int r = 16 * kk + e, n = j * hop + r;
-            double v = r < hop && n < n_fft ? w[n] : 0.0;
-            for (int t = 0; t < parts; ++t) grp[t * 128 + (e >> 3) * 64 + (e & 7)] = take_bf16(&v);
-          }
+    for (const auto& sj : steps) {
+      for (int m = 0; m < n_mels; ++m) {
+        const double* w = w64 + ((size_t)h * n_mels + m) * n_fft;
+        uint16_t* grp = step + (size_t)(m >> 3) * parts * 128 + (m & 7) * 8;
+        for (int e = 0; e < 16; ++e) {
+          const int r = 16 * sj.first + e, n = sj.second * hop + r;
+          double v = r < hop && n < n_fft ? w[n] : 0.0;
+          for (int t = 0; t < parts; ++t) grp[t * 128 + (e >> 3) * 64 + (e & 7)] = take_bf16(&v);
         }
+      }
+      step += p.step_bytes / 2;
     }
   }
   if (melt::dev_alloc(&sb->d_img, 2 * half) != cudaSuccess) return MELT_ERR_OOM;
@@ -145,8 +186,7 @@ cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream)
                            : L.n_mfcc       ? melt_slab_kernel<3, true>
                                             : melt_slab_kernel<3, false>;
   const int smem = (int)smem_bytes(p, L.n_mfcc);
-  cudaLaunchConfig_t cfg;
-  std::memset(&cfg, 0, sizeof(cfg));
+  cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -177,7 +217,8 @@ cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream)
   // time: reading A from shared memory bounds its MMAs).  MFCC sums over all
   // bins, so its blocks stay in one cluster.
   const int pairs16 = p.groups / 2;
-  int best = (pairs16 + kBlockBins / 16 - 1) / (kBlockBins / 16);
+  const int most = max_groups(sb->parts) / 2;
+  int best = (pairs16 + most - 1) / most;
   if (L.n_mfcc == 0) {
     long long cost = -1;
     for (int nb = best, first = best; nb <= std::max(first, (pairs16 + 1) / 2); ++nb) {

@@ -31,8 +31,8 @@ struct SlabLaunch {
   bool early_inputs;   // MELT_FWD_INPUT_READY: the waveform readers need not wait for the kernel before
 };
 
-// Builds the operand image for `parts` BF16 parts; leaves d_img null (MELT_OK)
-// where the kernel's shared-memory layout does not fit the geometry.
+// Builds the operand image for `parts` BF16 parts; MELT_ERR_UNSUPPORTED (with
+// nothing allocated) where the rings of 1 or 2 parts do not fit shared memory.
 melt_status slab_build(SlabBasis* sb, int n_fft, int hop, int n_mels, int n_mfcc, int parts, const double* w64);
 void slab_free(SlabBasis* sb);
 cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream);

@@ -38,6 +38,14 @@
 // 80 (the epilogue's accumulators live in registers); a short batch is cut
 // into more blocks to use more SMs.
 //
+// Split BF16 and BF16 (P 2 and P 1).  The same pieces serve the log-Mel of split
+// BF16 (three products, two parts) and of BF16 bases whose half does not fit
+// resident (the 22.05 kHz geometry).  Their sums are those of their other
+// layouts, bit for bit: one accumulator per unit, K-steps slice by slice.  So a
+// tile's slabs stay in a ring of their own (A) until their last slice is
+// done, a third to a whole tile more than a tile has, and the basis flows beside them (B),
+// slots of up to 3 or 8 K-steps.
+//
 // Warps: 0-7 epilogue (two per TMEM lane quarter, each half of the block's
 // bins), 8-10 and 12-14 converters (each takes whole slabs by itself: its samples
 // arrive by asynchronous copies in a staging area of its own, one arrival per
@@ -68,24 +76,27 @@ using namespace ptx;
 constexpr int kF = kTileFrames;
 // Warps 0-7 epilogue; 11 and 15, on one scheduler, MMA issue and basis
 // producer; the others from 8 on converters: six in the FP32 form, twelve where
-// there are fewer MMAs to a stage (its conversion took 6000 clocks a warp, 1000 a
-// stage with six, where P 2's MMAs take 480 to 720).
+// there are fewer MMAs to a slab (a slab took a warp 6000 clocks, 1000 with six
+// at work, where P 2's MMAs take 480 to 720).
 constexpr int kEpiWarps = 8, kMmaWarp = 11, kBWarp = 15;
-constexpr int kCvtTeams = 6;  // stages in conversion at once
-__host__ __device__ constexpr int team_warps(int P) { return P == 3 ? 1 : 2; }  // warps that share a stage's rows
-__host__ __device__ constexpr int slab_threads(int P) { return 32 * (kEpiWarps + 2 + kCvtTeams * team_warps(P)); }
-constexpr int kBlockBins = 80;  // Mel bins of a block: 2 x 40 accumulators per epilogue thread
-constexpr int kGroupsPerWarp = kBlockBins / 16;  // groups of 8 bins per epilogue warp
-constexpr int kNacc = 3;        // TMEM accumulators of 2 x kBlockBins columns
+constexpr int kMaxTeams = 6;  // slabs in conversion at once, each by a team of tw warps
+__host__ __device__ constexpr int cvt_warps(int P) { return P == 3 ? 6 : 12; }
+__host__ __device__ constexpr int slab_threads(int P) { return 32 * (kEpiWarps + 2 + cvt_warps(P)); }
+// Groups of 8 Mel bins of a block at most: the FP32 form's sums live in the
+// epilogue's registers (80 per thread); split BF16's 128 bins in one block
+// leave its rings too few slots.
+__host__ __device__ constexpr int max_groups(int P) { return P == 1 ? 16 : 10; }
+constexpr int kMaxAcc = 3;      // TMEM accumulators of the widest block's columns: 3 up to 80 bins, else 2
 constexpr int kMaxKps = 8;
-// K-steps of a stage at most.  P 3: its truncations grow with them, its drains
-// with their number.
-__host__ __device__ constexpr int max_kps(int P) { return P == 3 ? 4 : kMaxKps; }
+// K-steps at most of a stage (P 3: its truncations grow with them, its drains
+// with their number) or of a basis slot.
+__host__ __device__ constexpr int max_kps(int P) { return P == 3 ? 4 : P == 2 ? 3 : kMaxKps; }
 constexpr int kRowsA = 132;     // rows of a stage's A operand: 128 + kps - 1 and up to 4 mod 8, so that the two core
                                 // columns of a converter store fall on other banks (kMaxKps - 1 more at most)
 constexpr int kStageRows = kF + kMaxKps;  // sample rows a converter warp copies for a stage
 constexpr uint32_t kRawBytes = kStageRows * 64u;
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 8;   // P 3
+constexpr int kMaxA = 48, kMaxB = 8;  // P 1, 2: slots of the two rings
 
 struct SlabParams {
   const float* wave;
@@ -102,25 +113,31 @@ struct SlabParams {
   int nblk, wbg;       // blocks of wbg groups of 8 bins (the last may have fewer)
   int inner;           // blocks a unit takes in turn (MFCC: all of them, else 1)
   int n_units;
-  int kps;             // K-steps (slices of a slab) per stage
-  int NS;              // stages of the ring
-  int ncv;             // converter teams at work: at most NS (a team that took stage g waits for the place of
-                       // stage g + ncv by one parity bit, which tells only neighbouring phases apart)
-  uint32_t lbo_a, a_part, a_bytes, stage, step_bytes;  // a stage: A (a_bytes: P parts of two core columns), then B
+  int kps;             // K-steps per stage (slices of a slab); P 1, 2: per basis slot (slabs of a slice)
+  int NS, NB;          // stages of the ring (NB 0); P 1, 2: slots of the A and basis rings
+  int nacc;            // TMEM accumulators, acc_cols columns apart
+  uint32_t acc_cols;
+  int ncv, tw;         // converter teams at work (at most NS: a team that took slab g waits for the place of slab
+                       // g + ncv by one parity bit, which tells only neighbouring phases apart), warps of a team
+  uint32_t lbo_a, a_part, a_bytes, stage, step_bytes;  // a stage: A (a_bytes: P parts of two core columns), then B;
+                                                       // P 1, 2: an A slot
+  uint32_t off_b, b_slot;  // P 1, 2: the basis ring
   uint32_t off_raw, off_bar, off_misc, off_dct, off_part;
   int n_mfcc, n_out;
   int early_inputs;    // the waveform's readers need not wait for the stream's previous kernel
 };
 
 struct SlabBars {
-  int full, empty, t_full, t_empty, part, drain, total;
-  __host__ __device__ SlabBars(int NS) {
-    full = 0;                 // a stage: this CTA's basis copies; even CTA: also both CTAs' converters and the odd
-                              // CTA's signal that its copies are in
+  int full, empty, b_full, b_empty, t_full, t_empty, part, drain, total;
+  // P 3: NS stages, NB = 0.  P 1, 2: NS A slots and NB basis slots.
+  __host__ __device__ SlabBars(int NS, int NB) {
+    full = 0;                 // converters of both CTAs (even CTA's copy is used); P 3: and the basis, as b_full
     empty = full + NS;        // MMA commit, both CTAs
-    t_full = empty + NS;      // MMA commit, both CTAs
-    t_empty = t_full + kNacc; // both CTAs' epilogues (even CTA's copy is used)
-    part = t_empty + kNacc;   // MFCC, per lane quarter: part buffers 0, 1 filled; [16 B on] taken
+    b_full = empty + NS;      // this CTA's basis copies; even CTA: and the odd one's signal that its own are in
+    b_empty = b_full + NB;    // MMA commit, both CTAs
+    t_full = b_empty + NB;    // MMA commit, both CTAs
+    t_empty = t_full + kMaxAcc;  // both CTAs' epilogues (even CTA's copy is used)
+    part = t_empty + kMaxAcc; // MFCC, per lane quarter: part buffers 0, 1 filled; [16 B on] taken
     drain = part + 16;
     total = drain + 1;
   }
@@ -132,16 +149,10 @@ struct Ctx {
   volatile int* abort;
 };
 
-// Accumulators of a unit.  P 3: one per stage, added up in FP32 registers.  P 2
-// (whose operands carry 16 bits): two, each over half of the stages, added when
-// the epilogue reads them.  P 1: one (the sums of the form's other layouts).
+// P 3: stages of a unit (an accumulator each; the epilogue adds them up).
 static __device__ __forceinline__ int unit_stages(const SlabParams& p) {
   const int last = (p.n_last + 15) / 16;  // slabs that all slices reach
   return last * ((p.J + p.kps - 1) / p.kps) + (p.n_slab - last) * ((p.J - 1 + p.kps - 1) / p.kps);
-}
-template <int P>
-static __device__ __forceinline__ int acc_stages(const SlabParams& p) {
-  return P == 3 ? 1 : P == 2 ? (unit_stages(p) + 1) / 2 : unit_stages(p);
 }
 
 // Ring position: slot and the parity its next completion has.
@@ -197,11 +208,15 @@ static __device__ __forceinline__ void warp_arrive_local(uint32_t bar) {
 
 // Unit of ordinal i of this cluster: tile pair q and block b; false past the end.
 static __device__ __forceinline__ bool unit_at(const SlabParams& p, const Ctx& c, int i, int& q, int& b) {
-  const int u = c.cluster + (i / p.inner) * c.n_clusters;
+  // (the divisions only where there are several blocks)
+  const int u = c.cluster + (p.inner > 1 ? i / p.inner : i) * c.n_clusters;
   if (u >= p.n_units) return false;
   if (p.inner > 1) {
     q = u;
     b = i % p.inner;
+  } else if (p.nblk == 1) {
+    q = u;
+    b = 0;
   } else {
     q = u / p.nblk;
     b = u - q * p.nblk;
@@ -284,6 +299,66 @@ static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const S
     mbar_wait(bar_at(p, c, B.full + k % p.NS), (k / p.NS) & 1, &never, p.err, kErrTimeout);
 }
 
+// The same for P 1, 2: slice by slice, up to kps slabs to a slot.
+template <int P>
+static __device__ void basis_producer_slices(const SlabParams& p, const Ctx& c, const SlabBars& B) {
+  const uint64_t pol = policy_evict_last();
+  const uint8_t* half = p.img + (size_t)c.rank * p.ksteps * p.step_bytes;
+  const int last = (p.n_last + 15) / 16;
+  Ring r;
+  int issued = 0, q, b;
+  bool ok = true;
+  for (int i = 0; ok && unit_at(p, c, i, q, b); ++i) {
+    const uint32_t blk = (uint32_t)blk_groups(p, b) * P * 256u;
+    const uint8_t* src = half + (size_t)b * p.wbg * P * 256u;
+    for (int j = 0; ok && j < p.J; ++j) {
+      const int nk = j + 1 < p.J ? p.n_slab : last;
+      for (int k0 = 0; k0 < nk; k0 += p.kps) {
+        if (!bar_wait(bar_at(p, c, B.b_empty + r.slot), r.phase ^ 1, c.abort, p.err)) {
+          ok = false;
+          break;
+        }
+        const int n = min(p.kps, nk - k0);
+        const uint32_t full = bar_at(p, c, B.b_full + r.slot);
+        const uint32_t dst = c.sbase + p.off_b + r.slot * p.b_slot;
+        mbar_arrive_expect_tx(full, blk * n);
+        if (blk == p.step_bytes) {
+          bulk_g2s_hint(dst, src, blk * n, full, pol);
+        } else {
+          for (int k = 0; k < n; ++k) bulk_g2s_hint(dst + k * blk, src + (size_t)k * p.step_bytes, blk, full, pol);
+        }
+        src += (size_t)n * p.step_bytes;
+        ++issued;
+        r.next(p.NB);
+      }
+      if (j == 0) {
+        // L2 prefetch of the samples, one unit ahead of the converters' copies
+        if (i == 0 && !p.early_inputs) pdl_wait();
+        int qn, bn;
+        if (unit_at(p, c, i + 1, qn, bn) && (qn != q || i == 0)) prefetch_span(p, tile_of(p, c, qn));
+      }
+    }
+  }
+  // every issued copy has landed before the CTA can exit
+  volatile int never = 0;
+  for (int k = max(0, issued - p.NB); k < issued; ++k)
+    mbar_wait(bar_at(p, c, B.b_full + k % p.NB), (k / p.NB) & 1, &never, p.err, kErrTimeout);
+}
+
+// ---- odd CTA, P 1, 2: one arrival on the even CTA's b_full per filled slot
+static __device__ void basis_signal_slices(const SlabParams& p, const Ctx& c, const SlabBars& B) {
+  const int last = (p.n_last + 15) / 16;
+  Ring r;
+  int q, b;
+  for (int i = 0; unit_at(p, c, i, q, b); ++i)
+    for (int j = 0; j < p.J; ++j)
+      for (int k0 = 0; k0 < (j + 1 < p.J ? p.n_slab : last); k0 += p.kps) {
+        if (!bar_wait(bar_at(p, c, B.b_full + r.slot), r.phase, c.abort, p.err)) return;
+        mbar_arrive_cluster(mapa_shared(bar_at(p, c, B.b_full + r.slot), 0));
+        r.next(p.NB);
+      }
+}
+
 // ---- odd CTA: one arrival on the even CTA's barrier per stage whose basis is in
 static __device__ void basis_signal(const SlabParams& p, const Ctx& c, const SlabBars& B) {
   Ring r;
@@ -332,30 +407,23 @@ static __device__ __forceinline__ bool elect_one() {
   return r != 0;
 }
 
-// Products of a stage's n K-steps into accumulator d.  a, w: descriptors (low
-// words) of the first K-step's hi parts (parts 0 hi, 1 mid, 2 lo are ap and 16
-// apart, K-steps 1 row of A and `step` of the basis, in 16-byte units).  SMALL:
-// the products with a mid or lo part, else hi hi.  Straight-line code with one
-// predicate per K-step: a switch over n cost 150 to 200 clocks a stage.
-template <int P, bool SMALL>
+// Products of a stage's n K-steps into accumulator d (P 3).  a, w: descriptors
+// (low words) of the first K-step's hi parts (parts 0 hi, 1 mid, 2 lo are ap and
+// 16 apart, K-steps 1 row of A and `step` of the basis, in 16-byte units).
+// SMALL: the products with a mid or lo part, else hi hi.  Straight-line code
+// with one predicate per K-step: a switch over n cost 150 to 200 clocks a stage.
+template <bool SMALL>
 static __device__ __forceinline__ void stage_mmas(int n, uint32_t d, uint32_t a, uint32_t ah, uint32_t w, uint32_t wh,
-                                                  uint32_t ap, uint32_t step, uint32_t idesc, bool first) {
+                                                  uint32_t ap, uint32_t step, uint32_t idesc) {
   const uint32_t am = a + ap, al = am + ap;
 #pragma unroll
-  for (int k = 0; k < max_kps(P); ++k) {
+  for (int k = 0; k < max_kps(3); ++k) {
     if (k >= n) break;
     const uint32_t wk = w + k * step;
-    if constexpr (P == 1) {
-      if (k == 0) mma_pair_if(d, a, ah, wk, wh, idesc, !first);
-      else mma_pair<true>(d, a + k, ah, wk, wh, idesc);
-    } else if constexpr (!SMALL) {
+    if constexpr (!SMALL) {
       mma_pair<true>(d, a + k, ah, wk, wh, idesc);
-    } else if constexpr (P == 2) {
-      if (k == 0) mma_pair_if(d, a, ah, wk + 16, wh, idesc, !first);
-      else mma_pair<true>(d, a + k, ah, wk + 16, wh, idesc);
-      mma_pair<true>(d, am + k, ah, wk, wh, idesc);
     } else {
-      if (k == 0) mma_pair_if(d, al, ah, wk, wh, idesc, !first);
+      if (k == 0) mma_pair<false>(d, al, ah, wk, wh, idesc);
       else mma_pair<true>(d, al + k, ah, wk, wh, idesc);
       mma_pair<true>(d, a + k, ah, wk + 32, wh, idesc);
       mma_pair<true>(d, am + k, ah, wk + 16, wh, idesc);
@@ -366,51 +434,48 @@ static __device__ __forceinline__ void stage_mmas(int n, uint32_t d, uint32_t a,
 }
 
 // Both phases complete?  The two tests are in flight together.
-static __device__ __forceinline__ bool bar_wait2(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1, volatile int* abort,
-                                                 int* err) {
+static __device__ __forceinline__ bool warp_wait2(uint32_t b0, uint32_t p0, uint32_t b1, uint32_t p1,
+                                                  volatile int* abort, int* err) {
   const bool x = mbar_test_wait(b0, p0), y = mbar_test_wait(b1, p1);
-  return (x || bar_wait(b0, p0, abort, err)) && (y || bar_wait(b1, p1, abort, err));
+  return (__all_sync(0xffffffffu, x) || warp_wait(b0, p0, abort, err)) &&
+         (__all_sync(0xffffffffu, y) || warp_wait(b1, p1, abort, err));
 }
 
-// ---- even CTA: every MMA of the pair.
-// What this thread does besides its MMAs has to stay below the time they take
-// (P 3: 960 to 1900 clocks a stage at 80 bins; P 2: 480 to 720), and it runs at
-// ten and more clocks an instruction beside the SM's other warps: with rings of
-// their own for A and the basis (three waits, three commits and three ring steps
-// a slab) it took 830 clocks and bounded the P 2 kernel.
-template <int P>
+// ---- even CTA: every MMA of the pair (P 3).
+// What this warp does besides its MMAs has to stay below the time they take
+// (960 to 1900 clocks a stage at 80 bins), and it runs at ten and more clocks an
+// instruction beside the SM's other warps: with rings of their own for A and the
+// basis (three waits, three commits and three ring steps a slab), acquires at
+// cluster scope and one lane at work it took 1650 clocks and bounded the kernel.
 static __device__ void mma_issue(const SlabParams& p, const Ctx& c, const SlabBars& B, uint32_t tmem) {
   constexpr uint32_t ah = (128u >> 4) | (1u << 14);         // SBO 128 B
-  constexpr uint32_t wh = ((P * 256u) >> 4) | (1u << 14);   // SBO: the next group of 8 bins
+  constexpr uint32_t wh = ((3 * 256u) >> 4) | (1u << 14);   // SBO: the next group of 8 bins
   const uint32_t a0 = (c.sbase >> 4) | ((p.lbo_a >> 4) << 16);
   const uint32_t b0 = ((c.sbase + p.a_bytes) >> 4) | ((128u >> 4) << 16);  // LBO 128 B
   const uint32_t ap = p.a_part >> 4, stage = p.stage >> 4;
   const uint32_t full = bar_at(p, c, B.full), empty = bar_at(p, c, B.empty);
   const uint32_t t_full = bar_at(p, c, B.t_full), t_empty = bar_at(p, c, B.t_empty);
   const int kps = p.kps, J = p.J, n_last = p.n_last, n_slab = p.n_slab, NS = p.NS;
-  volatile int* abort = c.abort;
-  int* err = p.err;
-  const int per_acc = acc_stages<P>(p);
   Ring r, rt;
   uint32_t at = 0, d = tmem;  // the stage's offset in 16-byte units, the accumulator
   int q, b;
   bool ok = true;
   for (int i = 0; ok && unit_at(p, c, i, q, b); ++i) {
     const uint32_t ng = (uint32_t)blk_groups(p, b);
-    const uint32_t idesc = idesc_f32acc(1u, 2 * kF, 16u * ng), step = ng * ((P * 256u) >> 4);
+    const uint32_t idesc = idesc_f32acc(1u, 2 * kF, 16u * ng), step = ng * ((3 * 256u) >> 4);
     int kk = 0, left = J;  // slab, its slices to come (n_last > 0: the first slab has them all)
-    int in_acc = 0;                                      // stages in the accumulator
     while (kk < n_slab) {
-      if (in_acc == 0)
-        ok = bar_wait2(full + 8 * r.slot, r.phase, t_empty + 8 * rt.slot, rt.phase ^ 1, abort, err);
-      else
-        ok = bar_wait(full + 8 * r.slot, r.phase, abort, err);
+      ok = warp_wait2(full + 8 * r.slot, r.phase, t_empty + 8 * rt.slot, rt.phase ^ 1, c.abort, p.err);
       if (!ok) break;
       tc_fence_after();
       const int n = min(kps, left);
-      stage_mmas<P, true>(n, d, a0 + at, ah, b0 + at, wh, ap, step, idesc, in_acc == 0);
-      if constexpr (P > 1) stage_mmas<P, false>(n, d, a0 + at, ah, b0 + at, wh, ap, step, idesc, false);
-      mma_commit_pair_mc(empty + 8 * r.slot, 3);
+      if (elect_one()) {
+        stage_mmas<true>(n, d, a0 + at, ah, b0 + at, wh, ap, step, idesc);
+        stage_mmas<false>(n, d, a0 + at, ah, b0 + at, wh, ap, step, idesc);
+        mma_commit_pair_mc(empty + 8 * r.slot, 3);
+        mma_commit_pair_mc(t_full + 8 * rt.slot, 3);
+      }
+      __syncwarp();
       at += stage;
       r.next(NS);
       if (r.slot == 0) at = 0;
@@ -419,17 +484,96 @@ static __device__ void mma_issue(const SlabParams& p, const Ctx& c, const SlabBa
         ++kk;
         left = 16 * kk < n_last ? J : J - 1;
       }
-      if (++in_acc == per_acc || kk == n_slab) {
-        mma_commit_pair_mc(t_full + 8 * rt.slot, 3);
-        in_acc = 0;
-        d += 2 * kBlockBins;
-        rt.next(kNacc);
-        if (rt.slot == 0) d = tmem;
-      }
+      d += p.acc_cols;
+      rt.next(p.nacc);
+      if (rt.slot == 0) d = tmem;
     }
   }
   // no pair MMA may still be running when either CTA releases TMEM
-  mma_commit_pair_mc(bar_at(p, c, B.drain), 3);
+  if (elect_one()) mma_commit_pair_mc(bar_at(p, c, B.drain), 3);
+}
+
+// The same for P 1, 2: slice by slice over the unit's slabs, a basis slot at a
+// time, each K-step's hi hi (hi lo, lo hi) into the unit's one accumulator, the
+// order of the other layouts' sums.  The first slice waits for each slab; a
+// slab's last one frees its place.
+template <int P>
+static __device__ void mma_issue_slices(const SlabParams& p, const Ctx& c, const SlabBars& B, uint32_t tmem) {
+  constexpr uint32_t ah = (128u >> 4) | (1u << 14);         // SBO 128 B
+  constexpr uint32_t wh = ((P * 256u) >> 4) | (1u << 14);   // SBO: the next group of 8 bins
+  const uint32_t a0 = (c.sbase >> 4) | ((p.lbo_a >> 4) << 16);
+  const uint32_t b0 = ((c.sbase + p.off_b) >> 4) | ((128u >> 4) << 16);  // LBO 128 B
+  const uint32_t ap = p.a_part >> 4, as = p.stage >> 4, a_end = as * (uint32_t)p.NS, bs = p.b_slot >> 4;
+  const uint32_t full = bar_at(p, c, B.full), empty = bar_at(p, c, B.empty);
+  const uint32_t b_full = bar_at(p, c, B.b_full), b_empty = bar_at(p, c, B.b_empty);
+  const int kps = p.kps, J = p.J, n_slab = p.n_slab, NS = p.NS, NB = p.NB, last = (p.n_last + 15) / 16;
+  Ring ra, rb, rt;
+  uint32_t bl = b0, d = tmem;
+  int q, b;
+  bool ok = true;
+  for (int i = 0; ok && unit_at(p, c, i, q, b); ++i) {
+    const uint32_t ng = (uint32_t)blk_groups(p, b);
+    const uint32_t idesc = idesc_f32acc(1u, 2 * kF, 16u * ng), step = ng * ((P * 256u) >> 4);
+    const int slot0 = ra.slot;  // the unit's first slab
+    ok = warp_wait(bar_at(p, c, B.t_empty + rt.slot), rt.phase ^ 1, c.abort, p.err);
+    for (int j = 0; ok && j < J; ++j) {
+      const int nk = j + 1 < J ? n_slab : last;
+      const int free_from = j + 1 == J ? 0 : j + 2 == J ? last : n_slab;  // slabs this slice is the last of
+      int slot = slot0;
+      uint32_t at = (uint32_t)slot0 * as;
+      for (int k0 = 0; k0 < nk; k0 += kps) {
+        const int n = min(kps, nk - k0);
+        ok = warp_wait(b_full + 8 * rb.slot, rb.phase, c.abort, p.err);
+        if (j == 0)
+          for (int k = 0; ok && k < n; ++k) {
+            ok = warp_wait(full + 8 * ra.slot, ra.phase, c.abort, p.err);
+            ra.next(NS);
+          }
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t a = a0 + (uint32_t)j;
+        if (elect_one()) {
+          uint32_t o = at, w = bl;
+#pragma unroll
+          for (int k = 0; k < max_kps(P); ++k) {
+            if (k >= n) break;
+            if (k == 0) mma_pair_if(d, a + o, ah, w, wh, idesc, j + k0 > 0);
+            else mma_pair<true>(d, a + o, ah, w, wh, idesc);
+            if constexpr (P == 2) {
+              mma_pair<true>(d, a + o, ah, w + 16, wh, idesc);
+              mma_pair<true>(d, a + o + ap, ah, w, wh, idesc);
+            }
+            w += step;
+            o += as;
+            if (o == a_end) o = 0;
+          }
+          mma_commit_pair_mc(b_empty + 8 * rb.slot, 3);
+          for (int k = max(0, free_from - k0); k < n; ++k) {
+            const int sl = slot + k < NS ? slot + k : slot + k - NS;
+            mma_commit_pair_mc(empty + 8 * sl, 3);
+          }
+        }
+        __syncwarp();
+        slot += n;
+        at += (uint32_t)n * as;
+        if (slot >= NS) {
+          slot -= NS;
+          at -= a_end;
+        }
+        bl += bs;
+        rb.next(NB);
+        if (rb.slot == 0) bl = b0;
+      }
+    }
+    if (!ok) break;
+    if (elect_one()) mma_commit_pair_mc(bar_at(p, c, B.t_full + rt.slot), 3);
+    __syncwarp();
+    d += p.acc_cols;
+    rt.next(p.nacc);
+    if (rt.slot == 0) d = tmem;
+  }
+  // no pair MMA may still be running when either CTA releases TMEM
+  if (elect_one()) mma_commit_pair_mc(bar_at(p, c, B.drain), 3);
 }
 
 static __device__ __forceinline__ uint32_t pack2(float a, float b) {
@@ -448,17 +592,16 @@ static __device__ __forceinline__ void copy_quad(uint32_t dst, const float* src,
 // sample of row 0, column r) into the warp's own area.  Four lanes take the 16
 // samples of a row (64 contiguous bytes), so a warp's copies read whole sectors
 // of 8 rows.
-template <int TW>
 static __device__ __forceinline__ void stage_rows(const SlabParams& p, const float* src, int nsamp, int rows, bool live,
-                                                  int s0, uint32_t to, int u0) {
+                                                  int s0, uint32_t to, int u0, int tw) {
   int s = s0 + u0 * p.H;
   if (s0 + rows * p.H <= nsamp && p.H % 16 == 0) {  // (the same for all lanes) no sample past the clip's end
     const float* from = src + s;
 #pragma unroll 4
-    for (int u = u0; u < rows; u += 8 * TW, from += 8 * TW * p.H, to += 512 * TW) copy_quad(to, from, 16);
+    for (int u = u0; u < rows; u += 8 * tw, from += 8 * tw * p.H, to += 512 * tw) copy_quad(to, from, 16);
   } else {
 #pragma unroll 2
-    for (int u = u0; u < rows; u += 8 * TW, s += 8 * TW * p.H, to += 512 * TW) {
+    for (int u = u0; u < rows; u += 8 * tw, s += 8 * tw * p.H, to += 512 * tw) {
       const int left = live ? min(max(nsamp - s, 0), 4) : 0;  // samples of the quad before the clip's end
       copy_quad(to, src + (left ? s : 0), 4 * left);
     }
@@ -472,7 +615,7 @@ static __device__ __forceinline__ void stage_rows(const SlabParams& p, const flo
 // values of each part, as 8 bytes to core column qd / 2, row u.
 template <int P>
 static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars& B) {
-  constexpr int TW = team_warps(P);
+  const int TW = P == 3 ? 1 : p.tw;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cw = warp - kEpiWarps - (warp > kMmaWarp ? 1 : 0) - (warp > kBWarp ? 1 : 0);  // converter warp
   const int w = cw / TW;
@@ -481,29 +624,44 @@ static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars
   const uint32_t raw = c.sbase + p.off_raw + w * kRawBytes + 64u * u0 + 16u * qd;
   const uint32_t part = p.a_part;
   if (w >= p.ncv) return;
-  int q = 0, b, i = 0, kk = 0, j0 = 0;  // unit ordinal, slab, first slice
+  // unit ordinal and stage of it; the slab and first slice of that stage.  The
+  // descriptor of the unit after is loaded one unit early.
+  const int U = P == 3 ? unit_stages(p) : p.n_slab, last = (p.n_last + 15) / 16;
+  const int per = P == 3 ? (p.J + p.kps - 1) / p.kps : 1, per2 = max(1, (p.J - 1 + p.kps - 1) / p.kps);  // stages of a slab
+  int i = 0, st = 0, kk = 0, j0 = 0, q, b;
   Ring r;
-  TileDesc td;
+  TileDesc td, nxt;
   bool more = unit_at(p, c, 0, q, b);
   if (more) td = tile_of(p, c, q);
+  bool more_n = more && unit_at(p, c, 1, q, b);
+  if (more_n) nxt = tile_of(p, c, q);
   auto step = [&](int n) {  // n stages on
-    for (; more && n > 0; --n) {
-      r.next(p.NS);
-      j0 += p.kps;
-      if (j0 < slab_steps(p, kk)) continue;
-      j0 = 0;
-      if (++kk < p.n_slab) continue;
-      kk = 0;
-      const int was = q;
-      more = unit_at(p, c, ++i, q, b);
-      if (more && q != was) td = tile_of(p, c, q);
+    for (int k = 0; k < n; ++k) r.next(p.NS);
+    st += n;
+    while (st >= U && more) {
+      st -= U;
+      ++i;
+      more = more_n;
+      td = nxt;
+      more_n = more && unit_at(p, c, i + 1, q, b);
+      if (more_n) nxt = tile_of(p, c, q);
+    }
+    if (per == 1) {
+      kk = st;
+    } else if (st < last * per) {
+      kk = st / per;
+      j0 = (st - kk * per) * p.kps;
+    } else {
+      const int s2 = st - last * per;
+      kk = last + s2 / per2;
+      j0 = (s2 % per2) * p.kps;
     }
   };
   int rows = 0;
   auto copy = [&] {
-    rows = td.n_frames > 0 ? td.n_frames + min(p.kps, slab_steps(p, kk) - j0) - 1 : 0;
+    rows = td.n_frames > 0 ? td.n_frames + (P == 3 ? min(p.kps, slab_steps(p, kk) - j0) : p.J) - 1 : 0;
     const int col = 16 * kk + 4 * qd;
-    stage_rows<TW>(p, p.wave + td.in_off, td.n_samples, rows, col < p.H, j0 * p.H + col, raw, u0);
+    stage_rows(p, p.wave + td.in_off, td.n_samples, rows, col < p.H, j0 * p.H + col, raw, u0, TW);
   };
   step(w);
   if (more) copy();
@@ -511,7 +669,7 @@ static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars
     if (!warp_wait(bar_at(p, c, B.empty + r.slot), r.phase ^ 1, c.abort, p.err)) break;
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     uint32_t at = to + r.slot * p.stage, from = raw;
-#pragma unroll 2
+#pragma unroll 4
     for (int u = u0; u < rows; u += 8 * TW, at += 128 * TW, from += 512 * TW) {
       float a0, a1, a2, a3;
       asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a0), "=f"(a1), "=f"(a2), "=f"(a3) : "r"(from));
@@ -600,6 +758,7 @@ static __device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
 // ---- epilogue: adds the chunks of each unit, then power, log, (DCT) and store
 template <int P, bool MFCC>
 static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& c, const SlabBars& B, uint32_t tmem) {
+  constexpr int kG = max_groups(P) / 2;  // groups of 8 bins per epilogue warp at most
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quarter = warp & 3, half = warp >> 2;
   const int row = 32 * quarter + lane;
@@ -615,60 +774,41 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
     const bool valid = row < td.n_frames;
     const int m_lo = 8 * (b * p.wbg + g_lo);  // first bin of this warp
     if constexpr (P < 3) {
-      // the unit's one or two accumulators, group by group straight to the log
-      // and the row (as the other kernels of these forms evaluate it)
-      const uint32_t slot0 = rt.slot, t0 = tl + slot0 * 2 * kBlockBins + 8 * g_lo;
+      // the unit's accumulator, group by group straight to the log and the row
+      // (as the other kernels of these forms evaluate it)
+      const uint32_t slot0 = rt.slot, t0 = tl + slot0 * p.acc_cols + 8 * g_lo;
       if (!warp_wait(bar_at(p, c, B.t_full + rt.slot), rt.phase, c.abort, p.err)) break;
-      rt.next(kNacc);
-      const bool two = P == 2 && unit_stages(p) > 1;
-      const uint32_t slot1 = rt.slot, t1 = tl + slot1 * 2 * kBlockBins + 8 * g_lo;
-      if (two) {
-        if (!warp_wait(bar_at(p, c, B.t_full + rt.slot), rt.phase, c.abort, p.err)) break;
-        rt.next(kNacc);
-      }
+      rt.next(p.nacc);
       tc_fence_after();
       float* orow = p.out + (size_t)(td.out_row + row) * p.n_out;
+#pragma unroll 1
+      for (int g = 0; g < g_n; ++g) {
+        float v[8], im[8];
+        tmem_ld8(t0 + 8 * g, v);
+        tmem_ld8(t0 + 8 * ng + 8 * g, im);
+        ld_wait8(v, im);
+        if (g + 1 == g_n) {
+          tc_fence_before();
+          warp_arrive_leader(bar_at(p, c, B.t_empty + slot0));
+        }
 #pragma unroll
-      for (int g = 0; g < kGroupsPerWarp; ++g)
-        if (g < g_n) {
-          float v[8], im[8];
-          tmem_ld8(t0 + 8 * g, v);
-          tmem_ld8(t0 + 8 * ng + 8 * g, im);
-          ld_wait8(v, im);
-          if (two) {
-            float r2[8], i2[8];
-            tmem_ld8(t1 + 8 * g, r2);
-            tmem_ld8(t1 + 8 * ng + 8 * g, i2);
-            ld_wait8(r2, i2);
+        for (int e = 0; e < 8; ++e) v[e] = fast_ln(fmaf(v[e], v[e], fmaf(im[e], im[e], p.eps)));
+        if (valid) {
+          const int m = m_lo + 8 * g;
+          if (vec8 && m + 8 <= p.M) {
+            store8(orow + m, v);
+          } else {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              v[e] += r2[e];
-              im[e] += i2[e];
-            }
-          }
-          if (g + 1 == g_n) {
-            tc_fence_before();
-            warp_arrive_leader(bar_at(p, c, B.t_empty + slot0));
-            if (two) warp_arrive_leader(bar_at(p, c, B.t_empty + slot1));
-          }
-#pragma unroll
-          for (int e = 0; e < 8; ++e) v[e] = fast_ln(fmaf(v[e], v[e], fmaf(im[e], im[e], p.eps)));
-          if (valid) {
-            const int m = m_lo + 8 * g;
-            if (vec8 && m + 8 <= p.M) {
-              store8(orow + m, v);
-            } else {
-#pragma unroll
-              for (int e = 0; e < 8; ++e)
-                if (m + e < p.M) orow[m + e] = v[e];
-            }
+            for (int e = 0; e < 8; ++e)
+              if (m + e < p.M) orow[m + e] = v[e];
           }
         }
+      }
     } else {
-      float acc[kGroupsPerWarp][2][8];
+      float acc[kG][2][8];
       bool ok = true;
 #pragma unroll
-        for (int g = 0; g < kGroupsPerWarp; ++g)
+        for (int g = 0; g < kG; ++g)
 #pragma unroll
           for (int e = 0; e < 8; ++e) acc[g][0][e] = acc[g][1][e] = 0.f;
         for (int left = unit_stages(p); left > 0; --left) {
@@ -677,9 +817,9 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
             break;
           }
           tc_fence_after();
-          const uint32_t t0 = tl + rt.slot * 2 * kBlockBins + 8 * g_lo;
+          const uint32_t t0 = tl + rt.slot * p.acc_cols + 8 * g_lo;
 #pragma unroll
-          for (int g = 0; g < kGroupsPerWarp; ++g)
+          for (int g = 0; g < kG; ++g)
             if (g < g_n) {
               float re[8], im[8];
               tmem_ld8(t0 + 8 * g, re);
@@ -693,12 +833,12 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
             }
           tc_fence_before();
           warp_arrive_leader(bar_at(p, c, B.t_empty + rt.slot));
-          rt.next(kNacc);
+          rt.next(p.nacc);
         }
       if (!ok) break;
       bool finite = true;
 #pragma unroll
-      for (int g = 0; g < kGroupsPerWarp; ++g)
+      for (int g = 0; g < kG; ++g)
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const float s = fmaf(acc[g][0][e], acc[g][0][e], acc[g][1][e] * acc[g][1][e]);
@@ -710,7 +850,7 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
         float* orow = p.out + (size_t)(td.out_row + row) * p.n_out;
         if (valid) {
 #pragma unroll
-          for (int g = 0; g < kGroupsPerWarp; ++g)
+          for (int g = 0; g < kG; ++g)
             if (g < g_n) {
               const int m = m_lo + 8 * g;
               if (vec8 && m + 8 <= p.M) {
@@ -735,7 +875,7 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
           const int l = __ffs(left) - 1;
           const float2 v = redo_row(p, x + (long long)(l - lane) * p.H, m_lo, min(m_lo + 8 * g_n, p.M));
 #pragma unroll
-          for (int g = 0; g < kGroupsPerWarp; ++g)
+          for (int g = 0; g < kG; ++g)
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
               const float t = __shfl_sync(0xffffffffu, 8 * g + e < 32 ? v.x : v.y, (8 * g + e) & 31);
@@ -744,7 +884,7 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
         }
         // bins past M (zero basis rows) take no part, whatever their log is
 #pragma unroll
-        for (int g = 0; g < kGroupsPerWarp; ++g)
+        for (int g = 0; g < kG; ++g)
 #pragma unroll
           for (int e = 0; e < 8; ++e)
             if (m_lo + 8 * g + e >= p.M) acc[g][0][e] = 0.f;
@@ -768,7 +908,7 @@ static __device__ void epilogue(const SlabParams& p, uint8_t* gbase, const Ctx& 
           for (int k = 0; k < 8; ++k) {
             const float* d = dct + (size_t)min(k0 + k, p.n_mfcc - 1) * (8 * p.groups) + m_lo;
 #pragma unroll
-            for (int g = 0; g < kGroupsPerWarp; ++g)
+            for (int g = 0; g < kG; ++g)
               if (g < g_n) {
                 const float4 d0 = *reinterpret_cast<const float4*>(d + 8 * g);
                 const float4 d1 = *reinterpret_cast<const float4*>(d + 8 * g + 4);
@@ -820,15 +960,19 @@ __global__ void __launch_bounds__(slab_threads(P), 1) melt_slab_kernel(const __g
   c.n_clusters = (int)(gridDim.x >> 1);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + p.off_misc);
   c.abort = reinterpret_cast<volatile int*>(gbase + p.off_misc + 4);
-  const SlabBars B(p.NS);
-  const int warp = threadIdx.x >> 5;
+  const SlabBars B(p.NS, p.NB);
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   if (threadIdx.x == 0) {
     auto bar = [&](int i) { return bar_at(p, c, i); };
     for (int i = 0; i < p.NS; ++i) {
-      mbar_init(bar(B.full + i), c.rank == 0 ? 2 + 2 * team_warps(P) : 1);
+      mbar_init(bar(B.full + i), P < 3 ? 2 * p.tw : c.rank == 0 ? 4 : 1);
       mbar_init(bar(B.empty + i), 1);
     }
-    for (int i = 0; i < kNacc; ++i) {
+    for (int i = 0; i < p.NB; ++i) {
+      mbar_init(bar(B.b_full + i), c.rank == 0 ? 2 : 1);
+      mbar_init(bar(B.b_empty + i), 1);
+    }
+    for (int i = 0; i < kMaxAcc; ++i) {
       mbar_init(bar(B.t_full + i), 1);
       mbar_init(bar(B.t_empty + i), 2 * kEpiWarps);
     }
@@ -859,15 +1003,24 @@ __global__ void __launch_bounds__(slab_threads(P), 1) melt_slab_kernel(const __g
   // the basis and the MMAs touch the library's own data only; what reads
   // tiles or samples or writes features waits for the stream's previous kernel
   if (warp == kMmaWarp) {
-    if (elect_one()) {
-      if (c.rank == 0) mma_issue<P>(p, c, B, tmem);
-      else basis_signal(p, c, B);
-      volatile int never = 0;
-      mbar_wait(bar_at(p, c, B.drain), 0, &never, p.err, kErrTimeout);
+    // (the whole warp walks the stages, so that descriptors and ring state can
+    // stay in uniform registers; one elected lane issues)
+    if constexpr (P == 3) {
+      if (c.rank == 0) mma_issue(p, c, B, __shfl_sync(0xffffffffu, tmem, 0));
+      else if (elect_one()) basis_signal(p, c, B);
+    } else {
+      if (c.rank == 0) mma_issue_slices<P>(p, c, B, __shfl_sync(0xffffffffu, tmem, 0));
+      else if (elect_one()) basis_signal_slices(p, c, B);
     }
     __syncwarp();
+    volatile int never = 0;
+    mbar_wait(bar_at(p, c, B.drain), 0, &never, p.err, kErrTimeout);
+    __syncwarp();
   } else if (warp == kBWarp) {
-    if (elect_one()) basis_producer<P>(p, c, B);
+    if (elect_one()) {
+      if constexpr (P == 3) basis_producer<P>(p, c, B);
+      else basis_producer_slices<P>(p, c, B);
+    }
     __syncwarp();
   } else if (warp >= kEpiWarps) {
     if (!p.early_inputs) pdl_wait();

@@ -165,7 +165,7 @@ bool try_layout(const TcBasis* tb, TcParams& p, const melt_plan& c, int n_mfcc) 
 bool try_layout_pair(const TcBasis* tb, TcParams& p, const melt_plan& c, int n_mfcc) {
   const bool fp8 = tb->precision == MELT_FP8E4M3;
   const bool x3 = tb->precision == MELT_BF16X3;
-  if (c.cta_pair != 1 || (tb->precision != MELT_BF16 && !fp8 && !x3) || (!tb->d_b2 && !x3) || p.nblk > 1 ||
+  if (c.cta_pair != 1 || (tb->precision != MELT_BF16 && !fp8 && !x3) || !tb->d_b2 || p.nblk > 1 ||
       tb->stft_bands > 0)
     return false;
   // FP8: a converter lane holds at most two quads of a Z row
@@ -359,15 +359,17 @@ int candidate_list(const TcBasis* tb, const TcParams& p, melt_plan* out, int cap
     for (int i = 0; i < n_alt && n < cap; ++i) out[n++] = alts[i];
     return n;
   }
-  // CTA pairs with each CTA's half basis streamed.  The slab kernel runs these
-  // where it is built for the basis (split BF16; BF16 whose half basis does not
-  // fit resident), and they come first there: 256 x 10 s split BF16 SLABX3 us
-  // against 114 us single-CTA; 22.05 kHz BF16, N = 1024, 64 x 20 s SLABB16
-  // against 51 us.  (The pair kernel's own streamed layout, which the shared
-  // grouped launch uses, measured no faster than the single-CTA ones.)
+  // CTA pairs with each CTA's half basis streamed: a 2-SM MMA shares every basis
+  // block between two tiles.  The slab kernel runs these where it is built for
+  // the basis, and they come first there (256 x 10 s split BF16 81 us against 114
+  // us single-CTA; BF16 at 22.05 kHz, N = 1024, 64 x 20 s 42 against 56 us; at
+  // N = 1200, 128 bins, 16 x 30 s 29 against 33 us).  The pair kernel's own
+  // streamed layout measured no faster than the single-CTA ones (64 x 30 s split
+  // BF16: 86.6 against 83.4 us), so elsewhere they come after those, for
+  // melt_autotune.
   auto streamed_pairs = [&] {
-    if ((tb->precision != MELT_BF16 || !tb->d_b2) && tb->precision != MELT_BF16X3) return;
-    if (tb->n_mfcc != 0 || tb->mlp_hd) return;
+    if ((tb->precision != MELT_BF16 && tb->precision != MELT_BF16X3) || !tb->d_b2 || tb->n_mfcc != 0 || tb->mlp_hd)
+      return;
     const int shapes[][2] = {{4, 4}, {4, 2}, {3, 4}, {2, 8}, {3, 2}, {2, 4}, {2, 2}, {2, 1}};
     for (int zb = 2; zb >= 1; --zb)
       for (const auto& sh : shapes) {
@@ -376,13 +378,11 @@ int candidate_list(const TcBasis* tb, const TcParams& p, melt_plan* out, int cap
         if (n < cap && try_layout_pair(tb, q, pc, 0) && q.NS >= 2) {
           if (q.NS < 4) pc.prefetch_tiles = 1;
           out[n++] = pc;
+          if (tb->slab) return;  // (they differ in nothing that the slab kernel takes from a plan)
         }
       }
   };
-  if (tb->slab) {
-    streamed_pairs();
-    if (n > 0 && tb->precision == MELT_BF16X3) return 1;  // one kernel whatever the layout
-  }
+  if (tb->slab) streamed_pairs();
   add(1, 2, 2, p.KS, 1);
   const int kps_hi = std::max(1, std::min(p.KS, 65536 / sb));   // <= 64 KB per slot
   for (int kps = kps_hi; kps >= 1; --kps)
@@ -407,18 +407,13 @@ melt_status tc_build(TcBasis* tb, const TcConfig& c, const double* w64) {
   const int MP = (M + 15) / 16 * 16, NC = 2 * MP;
   const int nblk = (MP + 127) / 128;
   const int J = (N + H - 1) / H;
-  // K-steps as (slice j, first sample r0): 16 samples of slice j, group by group
-  // of 16 columns over the slices (BF16) or slice by slice (split BF16), or 32,
-  // slice by slice (FP8)
+  // K-steps in (slice j, first sample r0 of the step) order; a step covers
+  // 16 samples of slice j (BF16 forms) or 32 (FP8)
   const int kstep = P == MELT_FP8E4M3 ? 32 : 16;
   std::vector<std::pair<int, int>> steps;
-  if (P != MELT_BF16) {
-    for (int j = 0; j < J; ++j)
-      for (int r0 = 0; r0 < std::min(H, N - j * H); r0 += kstep) steps.push_back({j, r0});
-  } else {
-    for (int r0 = 0; r0 < H; r0 += kstep)
-      for (int j = 0; j < J; ++j)
-        if (r0 < N - j * H) steps.push_back({j, r0});
+  for (int j = 0; j < J; ++j) {
+    const int kj = std::min(H, N - j * H);
+    for (int kk = 0; kk < (kj + kstep - 1) / kstep; ++kk) steps.push_back({j, kstep * kk});
   }
   const int KS = (int)steps.size();
   const size_t kstep_bytes = (size_t)NC * 32;  // 2 core columns x NC rows x 16 B
@@ -487,18 +482,22 @@ melt_status tc_build(TcBasis* tb, const TcConfig& c, const double* w64) {
     if (cudaMemcpy(tb->d_b, img.data(), img.size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return MELT_ERR_CUDA;
   }
-  if (P != MELT_BF16X3 && nblk == 1) {
+  if ((P == MELT_BF16 || P == MELT_FP8E4M3 || P == MELT_BF16X3) && nblk == 1) {
     // CTA-pair image: the K-step blocks of basis rows [0, MP) (W_r), then those
     // of rows [MP, 2 MP) (W_i); each block is 2 core columns x MP rows x 16 B
-    // (split BF16 runs in CTA pairs in the slab kernel, from its own image)
+    // per part (split BF16: the hi part, then the lo part)
     const size_t half_step = (size_t)MP * 32;
-    std::vector<uint8_t> img2((size_t)2 * KS * half_step, 0);
+    std::vector<uint8_t> img2((size_t)2 * KS * parts * half_step, 0);
     for (int h = 0; h < 2; ++h)
       for (int s = 0; s < KS; ++s)
-        for (int cc = 0; cc < 2; ++cc)
-          for (int r = 0; r < MP; ++r)
-            std::memcpy(img2.data() + ((size_t)h * KS + s) * half_step + (size_t)cc * MP * 16 + (size_t)r * 16,
-                        img.data() + (size_t)s * kstep_bytes + (size_t)cc * NC * 16 + (size_t)(h * MP + r) * 16, 16);
+        for (int pt = 0; pt < parts; ++pt)
+          for (int cc = 0; cc < 2; ++cc)
+            for (int r = 0; r < MP; ++r)
+              std::memcpy(img2.data() + (((size_t)h * KS + s) * parts + pt) * half_step + (size_t)cc * MP * 16 +
+                              (size_t)r * 16,
+                          img.data() + ((size_t)s * parts + pt) * kstep_bytes + (size_t)cc * NC * 16 +
+                              (size_t)(h * MP + r) * 16,
+                          16);
     if (melt::dev_alloc(&tb->d_b2, img2.size()) != cudaSuccess) return MELT_ERR_OOM;
     if (cudaMemcpy(tb->d_b2, img2.data(), img2.size(), cudaMemcpyHostToDevice) != cudaSuccess)
       return MELT_ERR_CUDA;
@@ -592,15 +591,13 @@ cudaError_t tc_launch(const TcBasis* tb, const TcLaunch& L, cudaStream_t stream)
   const bool fused = pair && p.Hd > 0 && L.mlp != nullptr;
   if (pair && p.Hd > 0 && !L.mlp) p.Hd = 0;  // plan made for a correction that is not passed
   KernelFn fn = fused ? kernel_for_pair_mlp(p.MP / 16)
-                : pair ? (tb->precision == MELT_FP8E4M3 ? kernel_for_pair_fp8(L.n_mfcc > 0, p.MP / 16, p.dct_tc)
-                                                        : kernel_for_pair(L.n_mfcc > 0, p.MP / 16, p.dct_tc))
+                : pair ? (tb->precision == MELT_FP8E4M3   ? kernel_for_pair_fp8(L.n_mfcc > 0, p.MP / 16, p.dct_tc)
+                          : tb->precision == MELT_BF16X3 ? kernel_for_pair_x3()
+                                                         : kernel_for_pair(L.n_mfcc > 0, p.MP / 16, p.dct_tc))
                        : (L.n_mfcc ? kernel_for_mfcc(tb->precision, p.MP / 16)
                                    : kernel_for_plain(tb->precision, p.MP / 16, L.stft_bands > 0));
   if (!fn) return cudaErrorInvalidValue;
-  // a streamed half basis runs in the slab kernel where that has the basis; so
-  // does split BF16 under any layout (64 x 30 s: the layouts differed by 5 %,
-  // the slab kernel's sums are more exact, and every layout gives the same bits)
-  if (tb->slab && (tb->precision == MELT_BF16X3 || (pair && !p.b_resident))) {
+  if (tb->slab && pair && !p.b_resident) {  // a streamed half basis runs in the slab kernel where that has the basis
     SlabLaunch S;
     S.wave = L.wave; S.tiles = L.tiles; S.n_tiles = L.n_tiles; S.out = L.out;
     S.dct = nullptr; S.w32 = nullptr; S.mp = 0; S.n_mfcc = 0;

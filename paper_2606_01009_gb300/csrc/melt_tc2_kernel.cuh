@@ -478,6 +478,9 @@ static __device__ void pair_mma(const TcParams& p, uint8_t* gbase, const PairCtx
   const uint32_t abuf16 = p.abuf_bytes >> 4;
   const int nacc = MLP ? 1 : p.nacc;  // the fused MLP's TMEM leaves room for one accumulator
   const uint32_t sfb = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * p.ZB);  // FP8: basis scale 2^-8
+  // split BF16: the lo part of an A buffer follows its hi part; the lo part
+  // of a K-step block of this CTA's basis half follows its hi part
+  const uint32_t apart16 = p.a_bytes >> 4, bpart16 = (p.step_bytes / 2) >> 4;
   // streamed half basis: slot descriptors (low word) and the fill count
   const uint32_t bslot0 = ((c.sbase + p.off_b) >> 4) | ((p.b_lbo >> 4) << 16);
   const uint32_t bslot16 = p.bslot_bytes >> 4, step16 = p.step_bytes >> 4;
@@ -525,6 +528,10 @@ static __device__ void pair_mma(const TcParams& p, uint8_t* gbase, const PairCtx
             asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(tx), "=r"(ty) : "r"(tab_s + 8u * (s0 + u)));
             const uint32_t bl = bslot0 + slot * bslot16 + u * step16;
             mma_f16_pair(d, hi | (alo + tx), hi | bl, p.idesc, s0 + u > 0);
+            if constexpr (PREC == MELT_BF16X3) {
+              mma_f16_pair(d, hi | (alo + tx), hi | (bl + bpart16), p.idesc, true);
+              mma_f16_pair(d, hi | (alo + tx + apart16), hi | bl, p.idesc, true);
+            }
           }
           mma_commit_pair_mc(pbar(p, c, B.bs_empty + slot), 3);
         }
@@ -554,6 +561,11 @@ static __device__ void pair_mma(const TcParams& p, uint8_t* gbase, const PairCtx
                            s0 + u > 0);
           } else {
             mma_f16_pair(d, hi | (alo + tx[u]), hi | ty[u], p.idesc, s0 + u > 0);
+            if constexpr (PREC == MELT_BF16X3) {
+              // hi*lo and lo*hi, in the order of the single-CTA kernel (bit-identical sums)
+              mma_f16_pair(d, hi | (alo + tx[u]), hi | (ty[u] + bpart16), p.idesc, true);
+              mma_f16_pair(d, hi | (alo + tx[u] + apart16), hi | ty[u], p.idesc, true);
+            }
           }
         }
     }
@@ -604,7 +616,7 @@ static __device__ void pair_mma(const TcParams& p, uint8_t* gbase, const PairCtx
 // (lanes read consecutive quads: conflict-free); quad hq is the low or high
 // half (hq & 1) of the Z row segment (row ul, 8-sample group kc) with
 // 8 * (hq >> 1) = (ul - ch*CH) H + 8 kc.
-template <int CT = kPCvtThreads>
+template <bool SPLIT, int CT = kPCvtThreads>
 static __device__ void pair_convert(const TcParams& p, const PairCtx& c, const PairBars& B, int cvt0) {
   const int ct = threadIdx.x - 32 * cvt0;
   const int H8 = p.H >> 3;
@@ -660,6 +672,12 @@ static __device__ void pair_convert(const TcParams& p, const PairCtx& c, const P
         if (qrow[q] < rows) {
           const uint32_t h0 = pack_bf16(x[q].x, x[q].y), h1 = pack_bf16(x[q].z, x[q].w);
           asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(zrow0 + qoff[q]), "r"(h0), "r"(h1));
+          if constexpr (SPLIT) {
+            // split BF16: lo = rn(x - hi), the second part p.a_bytes further
+            const uint32_t l0 = pack_bf16(x[q].x - __uint_as_float(h0 << 16), x[q].y - __uint_as_float(h0 & 0xffff0000u));
+            const uint32_t l1 = pack_bf16(x[q].z - __uint_as_float(h1 << 16), x[q].w - __uint_as_float(h1 & 0xffff0000u));
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(zrow0 + qoff[q] + p.a_bytes), "r"(l0), "r"(l1));
+          }
         }
       }
       warp_arrive(pbar(p, c, B.s_empty + slot));
@@ -1360,24 +1378,16 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
     uint2* tab = reinterpret_cast<uint2*>(gbase + p.off_tab);
     const uint32_t b_lo0 = ((sbase + p.off_b) >> 4) | ((p.b_lbo >> 4) << 16);
     const uint32_t step16 = p.step_bytes >> 4;
-    // BF16: steps of 16 samples in (16-column group kk, slice j) order, the order
-    // of the basis image and of the slab kernel's MMAs (the last slice may have
-    // fewer groups).  FP8: steps of 32 samples in (slice j, group kk) order, and
-    // j in bits 24..31 of the A entry for the scale-factor selection.
-    if constexpr (PREC == MELT_FP8E4M3) {
-      for (int j = 0, s0 = 0; j < p.J; ++j) {
-        const int steps = (min(p.H, p.N - j * p.H) + 31) / 32;
-        for (int kk = lane; kk < steps; kk += 32)
-          tab[s0 + kk] = make_uint2(((2u * kk * p.lbo_a + 16u * j) >> 4) | ((uint32_t)j << 24), b_lo0 + (s0 + kk) * step16);
-        s0 += steps;
-      }
-    } else {
-      const int last = (p.N - (p.J - 1) * p.H + 15) / 16;
-      for (int kk = lane; kk < p.H / 16; kk += 32) {
-        const int s0 = kk * (p.J - 1) + min(kk, last), steps = kk < last ? p.J : p.J - 1;
-        for (int j = 0; j < steps; ++j)
-          tab[s0 + j] = make_uint2((2u * kk * p.lbo_a + 16u * j) >> 4, b_lo0 + (s0 + j) * step16);
-      }
+    // steps in (slice j, K-group kk) order, the order of the basis image; a
+    // K-step is 16 samples (BF16) or 32 (FP8, which also keeps j in bits 24..31
+    // of the A entry for the scale-factor selection)
+    constexpr int kstep = PREC == MELT_FP8E4M3 ? 32 : 16;
+    for (int j = 0, s0 = 0; j < p.J; ++j) {
+      const int steps = (min(p.H, p.N - j * p.H) + kstep - 1) / kstep;
+      const uint32_t jtag = PREC == MELT_FP8E4M3 ? (uint32_t)j << 24 : 0u;
+      for (int kk = lane; kk < steps; kk += 32)
+        tab[s0 + kk] = make_uint2(((2u * kk * p.lbo_a + 16u * j) >> 4) | jtag, b_lo0 + (s0 + kk) * step16);
+      s0 += steps;
     }
   }
   if (warp == kPMmaWarp) {
@@ -1444,7 +1454,7 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
     if constexpr (PREC == MELT_FP8E4M3)
       pair_convert_fp8<CW>(p, gbase, c, B, kPCvtWarp0, tmem_base);
     else
-      pair_convert<32 * CW>(p, c, B, kPCvtWarp0);
+      pair_convert<PREC == MELT_BF16X3, 32 * CW>(p, c, B, kPCvtWarp0);
     __syncwarp();
   } else {
     pdl_wait();
@@ -1543,6 +1553,12 @@ KernelFn pick_pair_fp8_kernel(bool mfcc, int nch, bool dtc = false) {
     case 8: return melt_tc_pair_kernel<8, true, false, MELT_FP8E4M3>;
     default: return nullptr;
   }
+}
+
+// Split-BF16 (BF16x3) instantiation: log-Mel only.
+template <int = 0>
+KernelFn pick_pair_x3_kernel() {
+  return melt_tc_pair_kernel<1, false, false, MELT_BF16X3>;
 }
 
 // Fused-MLP instantiations: log-Mel rows of 16 * nch bands (the fused TMEM

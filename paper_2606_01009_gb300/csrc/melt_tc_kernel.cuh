@@ -795,22 +795,12 @@ __global__ void __launch_bounds__(kThreads, 1) melt_tc_kernel(const __grid_const
     uint2* tab = reinterpret_cast<uint2*>(gbase + p.off_tab);
     const uint32_t b_lo0 = ((sbase + p.off_b) >> 4) | (((uint32_t)p.NC * 16 >> 4) << 16);
     const uint32_t bslot16 = p.step_bytes >> 4;
-    // the order of the basis image: BF16 (16-column group kk, slice j), as in the
-    // slab kernel (the last slice may have fewer groups); split BF16 (slice j, group kk)
-    if constexpr (PREC == MELT_BF16X3) {
-      for (int j = 0, s0 = 0; j < p.J; ++j) {
-        const int steps = (min(p.H, p.N - j * p.H) + 15) / 16;
-        for (int kk = lane; kk < steps; kk += 32)
-          tab[s0 + kk] = make_uint2((2u * kk * p.lbo_a + 16u * j) >> 4, b_lo0 + (s0 + kk) * bslot16);
-        s0 += steps;
-      }
-    } else {
-      const int last = (p.N - (p.J - 1) * p.H + 15) / 16;
-      for (int kk = lane; kk < p.H / 16; kk += 32) {
-        const int s0 = kk * (p.J - 1) + min(kk, last), steps = kk < last ? p.J : p.J - 1;
-        for (int j = 0; j < steps; ++j)
-          tab[s0 + j] = make_uint2((2u * kk * p.lbo_a + 16u * j) >> 4, b_lo0 + (s0 + j) * bslot16);
-      }
+    // steps in (slice j, 16-column group kk) order, the order of the basis image
+    for (int j = 0, s0 = 0; j < p.J; ++j) {
+      const int steps = (min(p.H, p.N - j * p.H) + 15) / 16;
+      for (int kk = lane; kk < steps; kk += 32)
+        tab[s0 + kk] = make_uint2((2u * kk * p.lbo_a + 16u * j) >> 4, b_lo0 + (s0 + kk) * bslot16);
+      s0 += steps;
     }
   }
   if (warp == kMmaWarp) {
@@ -893,6 +883,8 @@ KernelFn kernel_for_pair(bool mfcc, int nch, bool dtc);
 KernelFn kernel_for_pair_mlp(int nch);
 // Defined in melt_tc2_fp8.cu: the CTA-pair kernel with FP8 e4m3 operands.
 KernelFn kernel_for_pair_fp8(bool mfcc, int nch, bool dtc);
+// Defined in melt_tc2_x3.cu: the CTA-pair kernel with split-BF16 operands.
+KernelFn kernel_for_pair_x3();
 
 }  // namespace tc
 }  // namespace melt

@@ -7,7 +7,8 @@ import numpy as np
 import pytest
 
 from oracle import melt_oracle as O
-from tests.helpers import U32, fp32_sum_error, gpu_features, log_error_bound, oracle_features
+from tests.helpers import (U32, acc_rel, fp32_sum_error, gpu_features, log_error_bound, oracle_features,
+                           rounded_log_bound)
 
 pytestmark = pytest.mark.gpu
 
@@ -29,9 +30,8 @@ def _clips(n_fft, hop, frames, seed):
 
 
 # (n_fft, hop): one K-step, hop = N, hops that leave 4, 8, 12 of a slab's 16
-# columns, a short last slice, one slice, many slices in chunks of four (the
-# last one shorter), more rows than are staged at once, and a hop whose slab
-# does not fit (CUDA cores)
+# columns, a short last slice, one slice, many slices in stages of four (the
+# last one shorter), and the shortest hop of the longest frame
 GEOM = [(16, 16), (64, 64), (400, 160), (400, 100), (404, 12), (200, 88), (1200, 160), (1024, 256), (400, 400),
         (400, 20), (480, 16), (4096, 1024), (4096, 4)]
 
@@ -99,3 +99,26 @@ def test_values_the_split_cannot_hold(melt, value, n_fft, hop):
         big = ~zero & (np.maximum(np.abs(spec.Wr[:, n]), np.abs(spec.Wi[:, n])) > 1e-15)
         if not np.isnan(value):
             assert np.all(got[f][big & ~np.broadcast_to(nan, big.shape)] == np.inf)
+
+
+@pytest.mark.parametrize("prec,n_fft,hop,n_mels,streamed", [
+    ("bf16x3", 400, 160, 80, True), ("bf16x3", 400, 80, 81, True), ("bf16x3", 404, 48, 128, True),
+    ("bf16x3", 1200, 160, 100, True), ("bf16", 1024, 256, 80, True), ("bf16", 1200, 160, 128, True),
+    ("bf16x3", 640, 64, 40, False)])
+@pytest.mark.parametrize("tiles", [1, 40])
+def test_rounded_forms(melt, prec, n_fft, hop, n_mels, streamed, tiles):
+    """Split BF16, and BF16 whose half basis is streamed (the slab kernel, or not where a tile has too
+    many rows), against the same rounded operands in FP64, within the tensor-core forms'
+    accumulation allowance (helpers.acc_rel), and against the single-CTA kernel."""
+    kw = dict(sr=16000.0, n_fft=n_fft, hop=hop, n_mels=n_mels, fmin=0.0, fmax=8000.0)
+    clips = _clips(n_fft, hop, [1, 128 * tiles + 3], n_fft + n_mels)
+    spec = O.MelTSpec(**kw)
+    fe = melt.Frontend(precision=prec, **kw)
+    plan = melt.melt_plan_get(fe.handle)
+    assert ((plan["cta_pair"], plan["basis_resident"]) == (1, 0)) == streamed
+    got, ref = gpu_features(fe, clips), oracle_features(spec, clips, rounded=prec)
+    assert np.all(np.abs(got - ref) <= rounded_log_bound(spec, clips, prec, acc_rel(prec, n_fft, hop)))
+    single = dict(basis_resident=0, a_buffers=1, prefetch_tiles=2, basis_slots=2, ksteps_per_slot=1, cta_pair=0,
+                  schedule=0)
+    melt.melt_plan_set(fe.handle, single)
+    np.testing.assert_array_equal(gpu_features(fe, clips), got)  # the single-CTA kernel's sums, bit for bit
