@@ -136,20 +136,46 @@ def _check(status: int, what: str):
         raise MeltError(status, what)
 
 
+# What a call costs on the host decides the smallest batches: the C call itself takes
+# 3 us, and Python objects made per call used to add 14 (one 4 s clip, BF16: 15 -> 9
+# us a call, where the kernel's own 9 us are the bound; eight 1 s clips, FP32: 15 ->
+# 9 us).  So pointers go to ctypes as integers, arrays as views of their buffers (0.4
+# us; a POINTER from data_as costs 1.7 us), and the current stream is read as a handle
+# (0.4 us) instead of a Stream object (2.9 us).
 def _stream_ptr(stream):
     if stream is None:
         import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
-        return C.c_void_p(stream)
-    return C.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _i64(a):
+    """(contiguous int64 array of `a`, what to pass for an int64_t * to it)."""
     if a is None:
         return None, None
-    arr = np.ascontiguousarray(np.asarray(a, dtype=np.int64))
-    return arr, arr.ctypes.data_as(_I64P)
+    arr = np.ascontiguousarray(a, dtype=np.int64)
+    try:
+        return arr, C.c_int64.from_buffer(arr)
+    except (TypeError, ValueError):  # read-only or empty
+        return arr, arr.ctypes.data_as(_I64P)
+
+
+def _i32(a):
+    """_i64 for int32_t."""
+    arr = np.ascontiguousarray(a, dtype=np.int32)
+    try:
+        return arr, C.c_int32.from_buffer(arr)
+    except (TypeError, ValueError):
+        return arr, arr.ctypes.data_as(C.POINTER(C.c_int32))
+
+
+def _ptr(t):
+    """Device address of a torch tensor or an int."""
+    return t if isinstance(t, int) else t.data_ptr()
 
 
 # ------------------------------------------------------------------ C names
@@ -221,9 +247,9 @@ def melt_forward(basis, wave, offsets, lengths, out, stream=None, batch=None):
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
     b = int(lens.shape[0]) if batch is None else int(batch)
-    wp = wave if isinstance(wave, int) else wave.data_ptr()
-    outp = out if isinstance(out, int) else out.data_ptr()
-    _check(lib.melt_forward(basis, C.c_void_p(wp), op, lp, b, C.c_void_p(outp), _stream_ptr(stream)),
+    wp = _ptr(wave)
+    outp = _ptr(out)
+    _check(lib.melt_forward(basis, wp, op, lp, b, outp, _stream_ptr(stream)),
            "melt_forward")
 
 
@@ -232,9 +258,9 @@ def melt_forward_ex(basis, wave, offsets, lengths, out, flags, stream=None):
     the stream since the last host synchronisation writes ``wave``)."""
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
-    wp = wave if isinstance(wave, int) else wave.data_ptr()
-    outp = out if isinstance(out, int) else out.data_ptr()
-    _check(lib.melt_forward_ex(basis, C.c_void_p(wp), op, lp, int(lens.shape[0]), C.c_void_p(outp),
+    wp = _ptr(wave)
+    outp = _ptr(out)
+    _check(lib.melt_forward_ex(basis, wp, op, lp, int(lens.shape[0]), outp,
                                _stream_ptr(stream), int(flags)), "melt_forward_ex")
 
 
@@ -242,9 +268,9 @@ def melt_forward_noalloc(basis, wave, offsets, lengths, out, stream=None):
     """melt_forward with its tile list in a fixed device array: allocates nothing."""
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
-    wp = wave if isinstance(wave, int) else wave.data_ptr()
-    outp = out if isinstance(out, int) else out.data_ptr()
-    _check(lib.melt_forward_noalloc(basis, C.c_void_p(wp), op, lp, int(lens.shape[0]), C.c_void_p(outp),
+    wp = _ptr(wave)
+    outp = _ptr(out)
+    _check(lib.melt_forward_noalloc(basis, wp, op, lp, int(lens.shape[0]), outp,
                                     _stream_ptr(stream)), "melt_forward_noalloc")
 
 
@@ -253,9 +279,9 @@ def melt_pad_reflect(wave, offsets, lengths, pad, out, out_offsets=None, stream=
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
     oo, oop = _i64(out_offsets)
-    wp = wave if isinstance(wave, int) else wave.data_ptr()
-    outp = out if isinstance(out, int) else out.data_ptr()
-    _check(lib.melt_pad_reflect(C.c_void_p(wp), op, lp, int(lens.shape[0]), int(pad), C.c_void_p(outp), oop,
+    wp = _ptr(wave)
+    outp = _ptr(out)
+    _check(lib.melt_pad_reflect(wp, op, lp, int(lens.shape[0]), int(pad), outp, oop,
                                 _stream_ptr(stream)), "melt_pad_reflect")
 
 
@@ -266,13 +292,13 @@ def melt_diag_wait_timeout(basis, stream=None):
 
 def melt_diag_log(x, y, stream=None):
     """The tensor-core epilogues' natural log on device tensors x -> y (float32)."""
-    _check(lib.melt_diag_log(C.c_void_p(x.data_ptr()), C.c_void_p(y.data_ptr()), int(x.numel()), _stream_ptr(stream)),
+    _check(lib.melt_diag_log(x.data_ptr(), y.data_ptr(), int(x.numel()), _stream_ptr(stream)),
            "melt_diag_log")
 
 
 def melt_diag_gelu(h, y, stream=None):
     """The fused correction epilogue's GELU on device tensors h -> y (float32)."""
-    _check(lib.melt_diag_gelu(C.c_void_p(h.data_ptr()), C.c_void_p(y.data_ptr()), int(h.numel()), _stream_ptr(stream)),
+    _check(lib.melt_diag_gelu(h.data_ptr(), y.data_ptr(), int(h.numel()), _stream_ptr(stream)),
            "melt_diag_gelu")
 
 
@@ -301,15 +327,15 @@ def melt_forward_host(basis, wave, offsets, lengths, out, stream=None):
 
     if isinstance(out, np.ndarray) and (out.dtype != np.float32 or not out.flags.c_contiguous):
         raise ValueError("out must be a contiguous float32 array")
-    _check(lib.melt_forward_host(basis, C.c_void_p(hptr(wave)), op, lp, int(lens.shape[0]),
-                                 C.c_void_p(hptr(out)), _stream_ptr(stream)), "melt_forward_host")
+    _check(lib.melt_forward_host(basis, hptr(wave), op, lp, int(lens.shape[0]),
+                                 hptr(out), _stream_ptr(stream)), "melt_forward_host")
 
 
 def melt_forward_components(basis, wave, offsets, lengths, out, stream=None):
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
-    _check(lib.melt_forward_components(basis, C.c_void_p(wave.data_ptr()), op, lp, int(lens.shape[0]),
-                                       C.c_void_p(out.data_ptr()), _stream_ptr(stream)),
+    _check(lib.melt_forward_components(basis, wave.data_ptr(), op, lp, int(lens.shape[0]),
+                                       out.data_ptr(), _stream_ptr(stream)),
            "melt_forward_components")
 
 
@@ -332,8 +358,8 @@ def melt_autotune(basis, wave, offsets, lengths, out, stream=None, reps=5) -> di
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
     pl = MeltPlan()
-    _check(lib.melt_autotune(basis, C.c_void_p(wave.data_ptr()), op, lp, int(lens.shape[0]),
-                             C.c_void_p(out.data_ptr()), _stream_ptr(stream), int(reps), C.byref(pl)),
+    _check(lib.melt_autotune(basis, wave.data_ptr(), op, lp, int(lens.shape[0]),
+                             out.data_ptr(), _stream_ptr(stream), int(reps), C.byref(pl)),
            "melt_autotune")
     return pl.as_dict()
 
@@ -344,8 +370,8 @@ def melt_autotune_file(basis, wave, offsets, lengths, out, path, stream=None, re
     offs, op = _i64(offsets)
     pl = MeltPlan()
     hit = C.c_int(0)
-    _check(lib.melt_autotune_file(basis, C.c_void_p(wave.data_ptr()), op, lp, int(lens.shape[0]),
-                                  C.c_void_p(out.data_ptr()),
+    _check(lib.melt_autotune_file(basis, wave.data_ptr(), op, lp, int(lens.shape[0]),
+                                  out.data_ptr(),
                                   _stream_ptr(stream), int(reps), os.fsencode(path), C.byref(pl), C.byref(hit)),
            "melt_autotune_file")
     return pl.as_dict(), bool(hit.value)
@@ -368,13 +394,13 @@ def melt_group_set_split(group, frac0):
 def melt_forward_grouped(group, wave, offsets, lengths, basis_of, out, stream=None):
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
-    ids = np.ascontiguousarray(np.asarray(basis_of, dtype=np.int32))
+    ids, ip = _i32(basis_of)
     if ids.shape[0] != lens.shape[0]:
         raise ValueError("basis_of and lengths differ in length")
-    wp = wave if isinstance(wave, int) else wave.data_ptr()
-    outp = out if isinstance(out, int) else out.data_ptr()
-    _check(lib.melt_forward_grouped(group, C.c_void_p(wp), op, lp, ids.ctypes.data_as(C.POINTER(C.c_int32)),
-                                    int(lens.shape[0]), C.c_void_p(outp), _stream_ptr(stream)),
+    wp = _ptr(wave)
+    outp = _ptr(out)
+    _check(lib.melt_forward_grouped(group, wp, op, lp, ip,
+                                    int(lens.shape[0]), outp, _stream_ptr(stream)),
            "melt_forward_grouped")
 
 
@@ -382,13 +408,13 @@ def melt_group_autotune(group, wave, offsets, lengths, basis_of, out, path=None,
     """Tunes the plans of the group's bases on this batch; returns True on a plan-cache hit."""
     lens, lp = _i64(lengths)
     offs, op = _i64(offsets)
-    ids = np.ascontiguousarray(np.asarray(basis_of, dtype=np.int32))
+    ids, ip = _i32(basis_of)
     if ids.shape[0] != lens.shape[0]:
         raise ValueError("basis_of and lengths differ in length")
     hit = C.c_int(0)
-    _check(lib.melt_group_autotune(group, C.c_void_p(wave.data_ptr()), op, lp,
-                                   ids.ctypes.data_as(C.POINTER(C.c_int32)), int(lens.shape[0]),
-                                   C.c_void_p(out.data_ptr()), _stream_ptr(stream), int(reps),
+    _check(lib.melt_group_autotune(group, wave.data_ptr(), op, lp,
+                                   ip, int(lens.shape[0]),
+                                   out.data_ptr(), _stream_ptr(stream), int(reps),
                                    None if path is None else os.fsencode(path), C.byref(hit)),
            "melt_group_autotune")
     return bool(hit.value)
@@ -410,7 +436,7 @@ def _dptr(t):
     """Device pointer of a torch tensor, an int, or None."""
     if t is None:
         return None
-    return C.c_void_p(t if isinstance(t, int) else t.data_ptr())
+    return t if isinstance(t, int) else t.data_ptr()
 
 
 def melt_mlp_num_params(n_in, n_hidden) -> int:
@@ -537,11 +563,12 @@ class Frontend:
         """Features of a batch.  input_ready=True passes MELT_FWD_INPUT_READY
         (no kernel enqueued on the stream since the last host synchronisation
         writes ``wave``); centred framing pads with a kernel and ignores it."""
-        import torch
         if out is None:
+            import torch
             out = torch.empty((self.total_frames(lengths), self.n_out), device=wave.device,
                               dtype=torch.float32)
         if self.center:
+            import torch
             lens, offs, total = padded_layout(lengths, self.pad)
             if self._pad_buf is None or self._pad_buf.numel() < total or self._pad_buf.device != wave.device:
                 self._pad_buf = torch.empty(max(total, 4), device=wave.device, dtype=torch.float32)
@@ -601,8 +628,8 @@ class GroupedFrontend:
         return sum(self.frontends[int(g)].num_frames(int(L)) for L, g in zip(lengths, basis_of))
 
     def __call__(self, wave, offsets, lengths, basis_of, out=None, stream=None):
-        import torch
         if out is None:
+            import torch
             out = torch.empty((self.total_frames(lengths, basis_of), self.n_out), device=wave.device,
                               dtype=torch.float32)
         melt_forward_grouped(self.handle, wave, offsets, lengths, basis_of, out, stream)
