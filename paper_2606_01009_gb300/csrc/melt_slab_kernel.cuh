@@ -401,12 +401,6 @@ static __device__ __forceinline__ void mma_pair_if(uint32_t d, uint32_t a, uint3
       "r"(a), "r"(a_hi), "r"(b), "r"(b_hi), "r"(idesc), "r"((uint32_t)acc));
 }
 
-static __device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
-  return r != 0;
-}
-
 // Products of a stage's n K-steps into accumulator d (P 3).  a, w: descriptors
 // (low words) of the first K-step's hi parts (parts 0 hi, 1 mid, 2 lo are ap and
 // 16 apart, K-steps 1 row of A and `step` of the basis, in 16-byte units).

@@ -284,8 +284,6 @@ bool try_layout_pair(const TcBasis* tb, TcParams& p, const melt_plan& c, int n_m
       off += p.Hd > 0 ? align_up(p.mlp_half, 128) : 0u;
       p.off_bar = off;
       off += align_up(8 * B.total, 128);
-      p.off_tab = off;
-      off += align_up(8 * p.KS, 128);
       p.off_misc = off;
       off += 128;
       p.off_codes = off;  // FP8: the scale code of every Z row of the tile, per A buffer

@@ -188,7 +188,7 @@ static __device__ int pair_next_warp(const TcParams& p, const PairCtx& c, const 
 
 // An epilogue warp counts itself out of the ring entry of its pair ordinal
 // k >= 1 on the even CTA's barrier.  It does so once the pair's accumulator
-// is full: by then both producers, both CTAs' converters and the MMA thread
+// is full: by then both producers, both CTAs' converters and the MMA warp
 // have read the entry, so once both epilogues have, the slot may be reused.
 static __device__ __forceinline__ void sched_release(const TcParams& p, const PairCtx& c,
                                                      const PairBars& B, int k) {
@@ -215,10 +215,11 @@ static __device__ bool sched_publish(const TcParams& p, const PairCtx& c, const 
   return true;
 }
 
-static __device__ __forceinline__ bool warp_wait_cl(uint32_t bar, uint32_t parity, volatile int* abort,
+// Wait of a whole warp (lane 0 polls).
+static __device__ __forceinline__ bool pair_warp_wait(uint32_t bar, uint32_t parity, volatile int* abort,
                                                     int* err) {
   bool ok = true;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait_cluster(bar, parity, abort, err, kErrTimeout);
+  if ((threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort, err, kErrTimeout);
   return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 
@@ -341,7 +342,7 @@ static __device__ void pair_basis_stream(const TcParams& p, const PairCtx& c, co
 
 // Streamed half basis, odd CTA (its idle MMA warp): as each of its slots
 // fills, one arrival on the even CTA's bs_peer barrier of that slot, which
-// the even CTA's MMA thread waits on beside its own bs_full.
+// the even CTA's MMA warp waits on beside its own bs_full.
 static __device__ void pair_basis_signal(const TcParams& p, const PairCtx& c, const PairBars& B) {
   int g = 0;
   for (int q = c.cluster; q < p.n_pairs; q += c.n_clusters)
@@ -391,7 +392,7 @@ static __device__ __forceinline__ uint32_t gelu_col(const TcParams& p, int cc) {
   return p.h_col + mlp_gelu_off(p.Hd / 16, cc);
 }
 
-// Fused MLP (even CTA's MMA thread), hidden layer: H = x-hat W1^T, K-step s
+// Fused MLP (even CTA's MMA warp), hidden layer: H = x-hat W1^T, K-step s
 // reading x-hat's band chunk s at a1_col + 16 s.  The caller has seen the
 // epilogues' release of the tile's accumulator, which follows the x-hat
 // stores.
@@ -399,7 +400,6 @@ static __device__ void pair_mlp_gemm1(const TcParams& p, const PairCtx& c, const
                                       uint32_t tmem_base) {
   const uint64_t hi = (uint64_t)p.desc_hi << 32;
   const uint32_t w1 = ((c.sbase + p.off_mlp) >> 4) | ((((uint32_t)p.Hd / 2 * 16) >> 4) << 16);
-  tc_fence_after();
   for (int s = 0; s < p.MP / 16; ++s)
     mma_f16_pair_ts(tmem_base + p.h_col, tmem_base + p.a1_col + 16 * s, hi | (w1 + s * (p.w1_step >> 4)),
                     p.idesc1, s > 0);
@@ -409,22 +409,13 @@ static __device__ void pair_mlp_gemm1(const TcParams& p, const PairCtx& c, const
 // Fused MLP, output layer of the tile with ordinal j: once both CTAs'
 // epilogues have written GELU(H + b1) back and x + b2 into the output
 // columns, Y = x + b2 + GELU(H) W2^T (every K-step accumulates).
-static __device__ bool pair_mlp_gemm2(const TcParams& p, const PairCtx& c, const PairBars& B,
-                                      uint32_t tmem_base, int j) {
+static __device__ void pair_mlp_gemm2(const TcParams& p, const PairCtx& c, const PairBars& B, uint32_t tmem_base) {
   const uint64_t hi = (uint64_t)p.desc_hi << 32;
   const uint32_t w2 = ((c.sbase + p.off_mlp + p.mlp_w2_off) >> 4) | ((((uint32_t)p.MP / 2 * 16) >> 4) << 16);
-  // the K-steps' A columns before the wait, so that the MMAs issue back to back
-  const int nh = p.Hd / 16;  // <= 16
-  uint32_t ta[16];
-#pragma unroll
-  for (int s = 0; s < 16; ++s) ta[s] = tmem_base + gelu_col(p, s < nh ? s : 0);
-  if (!mbar_wait_cluster(pbar(p, c, B.a2_full), j & 1, c.abort, p.err, kErrTimeout)) return false;
-  tc_fence_after();
-#pragma unroll
-  for (int s = 0; s < 16; ++s)
-    if (s < nh) mma_f16_pair_ts(tmem_base + p.y_col, ta[s], hi | (w2 + s * (p.w2_step >> 4)), p.idesc2, true);
+  const int nh = p.Hd / 16;
+  for (int s = 0; s < nh; ++s)
+    mma_f16_pair_ts(tmem_base + p.y_col, tmem_base + gelu_col(p, s), hi | (w2 + s * (p.w2_step >> 4)), p.idesc2, true);
   mma_commit_pair_mc(pbar(p, c, B.y_full), 3);
-  return true;
 }
 
 // This CTA's rows of the DCT-II matrix as the B operand of the tensor-core
@@ -459,7 +450,6 @@ static __device__ void pair_dct_gemm(const TcParams& p, const PairCtx& c, const 
   const uint32_t dlo = dhi + (p.dct_part >> 4);
   const uint32_t step16 = (2 * nh16) >> 4;
   const uint32_t d = tmem_base + p.dct_c;
-  tc_fence_after();
   for (int s = 0; s < p.MP / 16; ++s) {
     mma_f16_pair_ts(d, tmem_base + p.dct_ahi + 8 * s, hi | (dhi + s * step16), p.idesc_dct, s > 0);
     mma_f16_pair_ts(d, tmem_base + p.dct_ahi + 8 * s, hi | (dlo + s * step16), p.idesc_dct, true);
@@ -468,147 +458,190 @@ static __device__ void pair_dct_gemm(const TcParams& p, const PairCtx& c, const 
   mma_commit_pair_mc(pbar(p, c, B.h_full), 3);
 }
 
-// Even CTA only: one thread issues every pair MMA.
+// MMA operands of one tile's projection: K-step (slice j, group kk of a slice)
+// reads A at a + j + kk a_step and the basis at w + (K-steps before it) w_step
+// (descriptor low words, 16-byte units).
+struct PairSteps {
+  uint32_t a, a_step, w, w_step, hi, d, idesc;
+  uint32_t a_lo, w_lo;  // split BF16: from a hi part to its lo part
+  uint32_t sfa, sfb;    // FP8: scale columns of A's rows and of the basis
+};
+
+// Issues n <= U K-steps of slice j from group k0 on.
+template <int PREC, int U>
+static __device__ __forceinline__ void pair_steps(const PairSteps& m, int j, int k0, int n, uint32_t w) {
+  uint32_t a = m.a + (uint32_t)j + (uint32_t)k0 * m.a_step;
+#pragma unroll
+  for (int k = 0; k < U; ++k) {
+    if (k >= n) break;
+    const bool acc = k > 0 || j + k0 > 0;
+    if constexpr (PREC == MELT_FP8E4M3) {
+      // A row t of slice j is Z row t + j, whose scale is byte j % 4 of scale group j / 4
+      mma_f8_pair_bs(m.d, desc64(a, m.hi), desc64(w, m.hi), m.idesc | ((uint32_t)(j & 3) << 29),
+                     m.sfa + 4u * (uint32_t)(j >> 2), m.sfb, acc);
+    } else {
+      mma_f16_pair(m.d, desc64(a, m.hi), desc64(w, m.hi), m.idesc, acc);
+      if constexpr (PREC == MELT_BF16X3) {
+        // hi*lo and lo*hi, in the order of the single-CTA kernel (bit-identical sums)
+        mma_f16_pair(m.d, desc64(a, m.hi), desc64(w + m.w_lo, m.hi), m.idesc, true);
+        mma_f16_pair(m.d, desc64(a + m.a_lo, m.hi), desc64(w, m.hi), m.idesc, true);
+      }
+    }
+    a += m.a_step;
+    w += m.w_step;
+  }
+}
+
+// Even CTA only: every pair MMA, walked by a whole warp so that descriptors stay
+// in uniform registers; one elected lane issues.  (One lane that looked its
+// K-steps up in shared memory took about 200 clocks an MMA, where the MMA itself
+// takes 80 at 80 bins.  64 x 30 s: MFCC 45.4 -> 43.3 us, fused correction 84.8 ->
+// 82.3, FP8 51.0 -> 50.3, log-Mel 38.2 both ways, bound by its bytes in flight;
+// 4096 mixed clips 711 -> 692.)  The waits acquire at CTA scope, 100 clocks for
+// 250 at cluster scope: what the peer wrote is read by the MMAs only, through the
+// async proxy, after its writers' proxy fences.
 template <bool MLP, int PREC, bool DTC = false>
-static __device__ void pair_mma(const TcParams& p, uint8_t* gbase, const PairCtx& c,
-                                const PairBars& B, uint32_t tmem_base) {
-  const uint2* tab = reinterpret_cast<const uint2*>(gbase + p.off_tab);
-  const uint64_t hi = (uint64_t)p.desc_hi << 32;
-  const uint32_t a_lo0 = ((c.sbase + p.off_a) >> 4) | ((p.lbo_a >> 4) << 16);
-  const uint32_t abuf16 = p.abuf_bytes >> 4;
+static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairBars& B, uint32_t tmem_base) {
+  // K-steps issued in a run.  Longer ones pay only where the DCT's MMAs wait behind
+  // them (MFCC 43.6 us with 5, 44.3 with 1; log-Mel 38.5 and 38.2).
+  constexpr int kU = DTC ? 5 : 1;
+  constexpr int kstep = PREC == MELT_FP8E4M3 ? 32 : 16;
   const int nacc = MLP ? 1 : p.nacc;  // the fused MLP's TMEM leaves room for one accumulator
-  const uint32_t sfb = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * p.ZB);  // FP8: basis scale 2^-8
-  // split BF16: the lo part of an A buffer follows its hi part; the lo part
-  // of a K-step block of this CTA's basis half follows its hi part
-  const uint32_t apart16 = p.a_bytes >> 4, bpart16 = (p.step_bytes / 2) >> 4;
-  // streamed half basis: slot descriptors (low word) and the fill count
-  const uint32_t bslot0 = ((c.sbase + p.off_b) >> 4) | ((p.b_lbo >> 4) << 16);
-  const uint32_t bslot16 = p.bslot_bytes >> 4, step16 = p.step_bytes >> 4;
+  const int J = p.J, nk = (p.H + kstep - 1) / kstep, nk_last = (p.N - (p.J - 1) * p.H + kstep - 1) / kstep;
+  const uint32_t a0 = ((c.sbase + p.off_a) >> 4) | ((p.lbo_a >> 4) << 16);
+  // the resident half basis, or the first slot of a streamed one
+  const uint32_t b0 = ((c.sbase + p.off_b) >> 4) | ((p.b_lbo >> 4) << 16);
+  PairSteps m;
+  m.a_step = (2u * p.lbo_a) >> 4;
+  m.w_step = p.step_bytes >> 4;
+  m.hi = p.desc_hi;
+  m.idesc = p.idesc;
+  m.a_lo = p.a_bytes >> 4;  // the lo part of an A buffer, or of a K-step's basis block, follows its hi part
+  m.w_lo = (p.step_bytes / 2) >> 4;
+  m.sfb = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * p.ZB);  // FP8: basis scale 2^-8
+  const auto wait = [&](int bar, int phase) {
+    return __all_sync(0xffffffffu, mbar_wait(pbar(p, c, bar), (uint32_t)phase & 1u, c.abort, p.err, kErrTimeout)) != 0;
+  };
+  const auto commit = [&](int bar) { mma_commit_pair_mc(pbar(p, c, bar), 3); };
   int g = 0;
   int k = 0;
   bool ok = true;
   for (;; ++k) {
     const int q = k == 0 ? c.cluster : pair_next_thread(p, c, B, k, ok);
+    ok = __all_sync(0xffffffffu, ok);
     if (!ok || q >= p.n_pairs) break;
     const int zb = p.ZB == 2 ? (k & 1) : 0;
     const int acc = k % nacc;
-    ok = mbar_wait_cluster(pbar(p, c, B.t_empty + acc), ((k / nacc) & 1) ^ 1, c.abort, p.err,
-                           kErrTimeout);
+    ok = wait(B.t_empty + acc, (k / nacc) ^ 1);
     if constexpr (MLP) {
       // the previous tile's x-hat is in TMEM (its accumulator was just
       // released): its hidden layer goes to the tensor cores first, so the
       // epilogue can start on GELU while this tile's projection runs
-      if (ok && k > 0) pair_mlp_gemm1(p, c, B, tmem_base);
-    }
-    ok = ok && mbar_wait_cluster(pbar(p, c, B.z_full + zb), (p.ZB == 2 ? (k >> 1) : k) & 1, c.abort,
-                                 p.err, kErrTimeout);
-    if (ok && k == 0 && p.b_resident)
-      ok = mbar_wait(pbar(p, c, B.b_full), 0, c.abort, p.err, kErrTimeout) &&
-           mbar_wait_cluster(pbar(p, c, B.peer_b), 0, c.abort, p.err, kErrTimeout);
-    if (!ok) break;
-    tc_fence_after();
-    const uint32_t d = tmem_base + acc * p.acc_stride;
-    const uint32_t alo = a_lo0 + zb * abuf16;
-    const uint32_t tab_s = smem_u32(tab);
-    if constexpr (PREC != MELT_FP8E4M3 && !MLP && !DTC) {  // (the host plans a streamed basis for these only)
-      if (!p.b_resident) {
-        // streamed half basis: slot by slot, each once both CTAs' halves are in
-        for (int s0 = 0; s0 < p.KS; s0 += p.kps, ++g) {
-          const int slot = g % p.NB;
-          const uint32_t ph = (g / p.NB) & 1;
-          if (!mbar_wait(pbar(p, c, B.bs_full + slot), ph, c.abort, p.err, kErrTimeout) ||
-              !mbar_wait(pbar(p, c, B.bs_peer + slot), ph, c.abort, p.err, kErrTimeout)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const int n = min(p.kps, p.KS - s0);
-          for (int u = 0; u < n; ++u) {
-            uint32_t tx, ty;
-            asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(tx), "=r"(ty) : "r"(tab_s + 8u * (s0 + u)));
-            const uint32_t bl = bslot0 + slot * bslot16 + u * step16;
-            mma_f16_pair(d, hi | (alo + tx), hi | bl, p.idesc, s0 + u > 0);
-            if constexpr (PREC == MELT_BF16X3) {
-              mma_f16_pair(d, hi | (alo + tx), hi | (bl + bpart16), p.idesc, true);
-              mma_f16_pair(d, hi | (alo + tx + apart16), hi | bl, p.idesc, true);
-            }
-          }
-          mma_commit_pair_mc(pbar(p, c, B.bs_empty + slot), 3);
-        }
-        if (!ok) break;
-        mma_commit_pair_mc(pbar(p, c, B.z_empty + zb), 3);
-        mma_commit_pair_mc(pbar(p, c, B.t_full + acc), 3);
-        continue;
+      if (ok && k > 0) {
+        tc_fence_after();
+        if (elect_one()) pair_mlp_gemm1(p, c, B, tmem_base);
+        __syncwarp();
       }
     }
-#pragma unroll 1
-    for (int s0 = 0; s0 < p.KS; s0 += 8) {
-      uint32_t tx[8], ty[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];"
-                     : "=r"(tx[u]), "=r"(ty[u])
-                     : "r"(tab_s + 8u * min(s0 + u, p.KS - 1)));
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (s0 + u < p.KS) {
-          if constexpr (PREC == MELT_FP8E4M3) {
-            // K-step of slice j = tx >> 24: A row t is Z row t + j, whose scale is
-            // byte j % 4 of scale group j / 4 of this A buffer
-            const uint32_t j = tx[u] >> 24;
-            const uint32_t sfa = tmem_base + p.sf_col + (uint32_t)(4 * (p.sfg * zb)) + 4u * (j >> 2);
-            mma_f8_pair_bs(d, hi | (alo + (tx[u] & 0xFFFFFFu)), hi | ty[u], p.idesc | ((j & 3u) << 29), sfa, sfb,
-                           s0 + u > 0);
-          } else {
-            mma_f16_pair(d, hi | (alo + tx[u]), hi | ty[u], p.idesc, s0 + u > 0);
-            if constexpr (PREC == MELT_BF16X3) {
-              // hi*lo and lo*hi, in the order of the single-CTA kernel (bit-identical sums)
-              mma_f16_pair(d, hi | (alo + tx[u]), hi | (ty[u] + bpart16), p.idesc, true);
-              mma_f16_pair(d, hi | (alo + tx[u] + apart16), hi | ty[u], p.idesc, true);
-            }
+    ok = ok && wait(B.z_full + zb, p.ZB == 2 ? (k >> 1) : k);
+    if (ok && k == 0 && p.b_resident) ok = wait(B.b_full, 0) && wait(B.peer_b, 0);
+    if (!ok) break;
+    tc_fence_after();
+    m.d = tmem_base + acc * p.acc_stride;
+    m.a = a0 + zb * (p.abuf_bytes >> 4);
+    m.sfa = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * zb);
+    m.w = b0;
+    if (PREC != MELT_FP8E4M3 && !MLP && !DTC && !p.b_resident) {  // (planned for these only)
+      // streamed half basis: slot by slot, each once both CTAs' halves are in
+      int j = 0, k0 = 0;
+      for (int s0 = 0; s0 < p.KS; s0 += p.kps, ++g) {
+        const int slot = g % p.NB;
+        if (!wait(B.bs_full + slot, g / p.NB) || !wait(B.bs_peer + slot, g / p.NB)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        uint32_t w = b0 + (uint32_t)slot * (p.bslot_bytes >> 4);
+        for (int left = min(p.kps, p.KS - s0); left > 0;) {
+          const int n = min(min(kU, left), (j + 1 < J ? nk : nk_last) - k0);
+          if (elect_one()) pair_steps<PREC, kU>(m, j, k0, n, w);
+          __syncwarp();
+          w += (uint32_t)n * m.w_step;
+          left -= n;
+          k0 += n;
+          if (k0 == (j + 1 < J ? nk : nk_last)) {
+            k0 = 0;
+            ++j;
           }
         }
+        if (elect_one()) commit(B.bs_empty + slot);
+        __syncwarp();
+      }
+      if (!ok) break;
+    } else if (elect_one()) {
+      uint32_t w = b0;
+      for (int j = 0; j < J; ++j) {
+        const int nj = j + 1 < J ? nk : nk_last;
+        for (int k0 = 0; k0 < nj; k0 += kU) {
+          const int n = min(kU, nj - k0);
+          pair_steps<PREC, kU>(m, j, k0, n, w);
+          w += (uint32_t)n * m.w_step;
+        }
+      }
     }
-    mma_commit_pair_mc(pbar(p, c, B.z_empty + zb), 3);
-    mma_commit_pair_mc(pbar(p, c, B.t_full + acc), 3);
+    __syncwarp();
+    if (elect_one()) {
+      commit(B.z_empty + zb);
+      commit(B.t_full + acc);
+    }
+    __syncwarp();
     if constexpr (DTC) {
       // the previous tile's DCT once its epilogues released its accumulator
       // (their log-Mel rows are in TMEM by then); this tile's projection is
       // already queued ahead of it
       if (k > 0) {
-        const int pa = (k - 1) % nacc;
-        if (!mbar_wait_cluster(pbar(p, c, B.t_empty + pa), ((k - 1) / nacc) & 1, c.abort, p.err, kErrTimeout)) {
-          ok = false;
-          break;
-        }
-        pair_dct_gemm(p, c, B, tmem_base);
+        ok = wait(B.t_empty + (k - 1) % nacc, (k - 1) / nacc);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) pair_dct_gemm(p, c, B, tmem_base);
+        __syncwarp();
       }
     }
     if constexpr (MLP) {
       // the previous tile's output layer, once its GELU(H) is written
-      if (k > 0 && !pair_mlp_gemm2(p, c, B, tmem_base, k - 1)) {
-        ok = false;
-        break;
+      if (k > 0) {
+        ok = wait(B.a2_full, k - 1);
+        if (!ok) break;
+        tc_fence_after();
+        if (elect_one()) pair_mlp_gemm2(p, c, B, tmem_base);
+        __syncwarp();
       }
     }
   }
   if constexpr (MLP) {
     // the last tile's MLP: wait for its x-hat (the release of its accumulator)
-    if (ok && k > 0 &&
-        mbar_wait_cluster(pbar(p, c, B.t_empty), (k - 1) & 1, c.abort, p.err, kErrTimeout)) {
-      pair_mlp_gemm1(p, c, B, tmem_base);
-      pair_mlp_gemm2(p, c, B, tmem_base, k - 1);
+    if (ok && k > 0 && wait(B.t_empty, k - 1)) {
+      tc_fence_after();
+      if (elect_one()) pair_mlp_gemm1(p, c, B, tmem_base);
+      __syncwarp();
+      if (wait(B.a2_full, k - 1)) {
+        tc_fence_after();
+        if (elect_one()) pair_mlp_gemm2(p, c, B, tmem_base);
+        __syncwarp();
+      }
     }
   }
   if constexpr (DTC) {
     // the last tile's DCT
-    if (ok && k > 0 &&
-        mbar_wait_cluster(pbar(p, c, B.t_empty + (k - 1) % nacc), ((k - 1) / nacc) & 1, c.abort, p.err,
-                          kErrTimeout))
-      pair_dct_gemm(p, c, B, tmem_base);
+    if (ok && k > 0 && wait(B.t_empty + (k - 1) % nacc, (k - 1) / nacc)) {
+      tc_fence_after();
+      if (elect_one()) pair_dct_gemm(p, c, B, tmem_base);
+      __syncwarp();
+    }
   }
   // no pair MMA may still be running when either CTA releases TMEM
-  mma_commit_pair_mc(pbar(p, c, B.drain), 3);
+  if (elect_one()) mma_commit_pair_mc(pbar(p, c, B.drain), 3);
+  __syncwarp();
 }
 
 // Staged FP32 span chunks -> Z rows (bf16).  Chunk ch of a tile holds Z rows
@@ -640,7 +673,7 @@ static __device__ void pair_convert(const TcParams& p, const PairCtx& c, const P
     const int qp = k == 0 ? c.cluster : pair_next_warp(p, c, B, k, okq);
     if (!okq || qp >= p.n_pairs) break;
     const int zb = p.ZB == 2 ? (k & 1) : 0;
-    if (!warp_wait_cl(pbar(p, c, B.z_empty + zb), ((p.ZB == 2 ? (k >> 1) : k) & 1) ^ 1, c.abort,
+    if (!pair_warp_wait(pbar(p, c, B.z_empty + zb), ((p.ZB == 2 ? (k >> 1) : k) & 1) ^ 1, c.abort,
                       p.err))
       break;
     const TileDesc td = pair_tile(p, c, qp);
@@ -856,7 +889,7 @@ static __device__ void pair_convert_fp8(const TcParams& p, uint8_t* gbase, const
     // below, or none: a timeout in any of them stops all of them here
     if (!named_barrier_and(1, kThr, okq) || qp >= p.n_pairs) break;
     const int zb = p.ZB == 2 ? (k & 1) : 0;
-    bool ok = warp_wait_cl(pbar(p, c, B.z_empty + zb), ((p.ZB == 2 ? (k >> 1) : k) & 1) ^ 1, c.abort, p.err);
+    bool ok = pair_warp_wait(pbar(p, c, B.z_empty + zb), ((p.ZB == 2 ? (k >> 1) : k) & 1) ^ 1, c.abort, p.err);
     const TileDesc td = pair_tile(p, c, qp);
     const int nsamp = td.n_samples;
     const uint32_t zaddr = c.sbase + p.off_a + zb * p.abuf_bytes;
@@ -930,7 +963,7 @@ __device__ void pair_epilogue_dct(const TcParams& p, const PairCtx& c, const Pai
     const int acc = p.nacc == 2 ? (k & 1) : 0;
     const uint32_t tphase = p.nacc == 2 ? ((k >> 1) & 1) : (k & 1);
     const TileDesc td = pair_tile(p, c, q);
-    if (!warp_wait_cl(pbar(p, c, B.t_full + acc), tphase, c.abort, p.err)) break;
+    if (!pair_warp_wait(pbar(p, c, B.t_full + acc), tphase, c.abort, p.err)) break;
     sched_release(p, c, B, k);
     tc_fence_after();
     const bool live = td.n_frames > 0;
@@ -975,7 +1008,7 @@ __device__ void pair_epilogue_dct(const TcParams& p, const PairCtx& c, const Pai
     }
     tc_fence_before();
     warp_arrive_leader(pbar(p, c, B.t_empty + acc));
-    if (!warp_wait_cl(pbar(p, c, B.h_full), k & 1, c.abort, p.err)) break;
+    if (!pair_warp_wait(pbar(p, c, B.h_full), k & 1, c.abort, p.err)) break;
     tc_fence_after();
     if (live) {
       float* orow = p.out + (size_t)(td.out_row + row) * p.n_mfcc;
@@ -1021,7 +1054,7 @@ __device__ void pair_epilogue(const TcParams& p, uint8_t* gbase, const PairCtx& 
     const int acc = p.nacc == 2 ? (k & 1) : 0;
     const uint32_t tphase = p.nacc == 2 ? ((k >> 1) & 1) : (k & 1);
     const TileDesc td = pair_tile(p, c, q);
-    if (!warp_wait_cl(pbar(p, c, B.t_full + acc), tphase, c.abort, p.err)) break;
+    if (!pair_warp_wait(pbar(p, c, B.t_full + acc), tphase, c.abort, p.err)) break;
     sched_release(p, c, B, k);
     tc_fence_after();
     const bool valid = row < td.n_frames;
@@ -1203,7 +1236,7 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
   const int h_lo = part_lo_tail(p.Hd / 16, kMlpParts, part), h_hi = part_lo_tail(p.Hd / 16, kMlpParts, part + 1);
   if (c.cluster >= p.n_pairs) return;
   TileDesc td = pair_tile(p, c, c.cluster);
-  if (!warp_wait_cl(pbar(p, c, B.t_full), 0, c.abort, p.err)) return;
+  if (!pair_warp_wait(pbar(p, c, B.t_full), 0, c.abort, p.err)) return;
   tc_fence_after();
   bool live = td.n_frames > 0;
   float v[16 * NV];
@@ -1238,7 +1271,7 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
     // 2. once H is in (x-hat consumed): x + b2 of the lower 8 bands into the
     // output columns (over x-hat), then GELU(H + b1) in BF16 over H (see
     // gelu_col), the next chunk's load in flight while one chunk is evaluated
-    if (!warp_wait_cl(pbar(p, c, B.h_full), k & 1, c.abort, p.err)) break;
+    if (!pair_warp_wait(pbar(p, c, B.h_full), k & 1, c.abort, p.err)) break;
     tc_fence_after();
     if (live) {
       float ha[16], hb[16];
@@ -1282,14 +1315,14 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
     bool live_n = false;
     if (more) {
       tn = pair_tile(p, c, qn);
-      if (!warp_wait_cl(pbar(p, c, B.t_full), (k + 1) & 1, c.abort, p.err)) break;
+      if (!pair_warp_wait(pbar(p, c, B.t_full), (k + 1) & 1, c.abort, p.err)) break;
       sched_release(p, c, B, k + 1);
       tc_fence_after();
       live_n = tn.n_frames > 0;
       if (live_n) mlp_logmel<NV>(p, tl, c_lo, c_hi, v);  // (this step's v is in TMEM as x + b2)
     }
     // 4. the output layer's sum for this warp's bands
-    if (!warp_wait_cl(pbar(p, c, B.y_full), k & 1, c.abort, p.err)) break;
+    if (!pair_warp_wait(pbar(p, c, B.y_full), k & 1, c.abort, p.err)) break;
     tc_fence_after();
     if (live) {
 #pragma unroll
@@ -1373,23 +1406,6 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
     *c.abort = 0;
     fence_mbar_init();
   }
-  if (warp == kPBWarp) {
-    // K-step table: A start offset (16-byte units, polyphase j-shift) and B low word
-    uint2* tab = reinterpret_cast<uint2*>(gbase + p.off_tab);
-    const uint32_t b_lo0 = ((sbase + p.off_b) >> 4) | ((p.b_lbo >> 4) << 16);
-    const uint32_t step16 = p.step_bytes >> 4;
-    // steps in (slice j, K-group kk) order, the order of the basis image; a
-    // K-step is 16 samples (BF16) or 32 (FP8, which also keeps j in bits 24..31
-    // of the A entry for the scale-factor selection)
-    constexpr int kstep = PREC == MELT_FP8E4M3 ? 32 : 16;
-    for (int j = 0, s0 = 0; j < p.J; ++j) {
-      const int steps = (min(p.H, p.N - j * p.H) + kstep - 1) / kstep;
-      const uint32_t jtag = PREC == MELT_FP8E4M3 ? (uint32_t)j << 24 : 0u;
-      for (int kk = lane; kk < steps; kk += 32)
-        tab[s0 + kk] = make_uint2(((2u * kk * p.lbo_a + 16u * j) >> 4) | jtag, b_lo0 + (s0 + kk) * step16);
-      s0 += steps;
-    }
-  }
   if (warp == kPMmaWarp) {
     tmem_alloc_pair(smem_u32(tmem_slot), p.tmem_cols);
     tmem_relinquish_pair();
@@ -1434,13 +1450,11 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
   // wait, so a launch fills and converts its first tiles while the previous
   // one drains; the epilogue, which stores features, always waits.
   if (warp == kPMmaWarp) {
-    if (lane == 0) {
-      if (c.rank == 0) pair_mma<MLP, PREC, DTC>(p, gbase, c, B, tmem_base);
-      else if (!p.b_resident) pair_basis_signal(p, c, B);  // the odd CTA's slots, to the even CTA
-      drain_wait(pbar(p, c, B.drain), 0, p.err);
-    } else if (MLP && lane == 1) {
-      pair_basis_producer(p, c, B);
-    }
+    if (MLP && lane == 0) pair_basis_producer(p, c, B);
+    __syncwarp();
+    if (c.rank == 0) pair_mma<MLP, PREC, DTC>(p, c, B, __shfl_sync(0xffffffffu, tmem_base, 0));
+    else if (lane == 0 && !p.b_resident) pair_basis_signal(p, c, B);  // the odd CTA's slots, to the even CTA
+    if (lane == 0) drain_wait(pbar(p, c, B.drain), 0, p.err);
     __syncwarp();
   } else if (warp == kPBWarp) {
     if (lane == 0) pair_basis_producer(p, c, B);
