@@ -90,7 +90,7 @@ __host__ __device__ constexpr int part_lo_tail(int n, int parts, int j) {
 // the warps, half the chain).  The MFCC kernels with the DCT on the CUDA
 // cores keep 4 (their epilogue warps and registers fill the block).  With
 // the fused MLP, 3: the warps go to the epilogue (64 x 30 s: 2 / 3 / 4 converter
-// warps 74.3 / 71.9 / 74 us; 8 or 16 epilogue warps 74 and more).
+// warps 75.3 / 73.8 / 76.2 us; 8 or 16 epilogue warps 75 and more).
 __host__ __device__ constexpr int pair_cvt_warps(int prec, bool mfcc, int nch, bool dtc = false, bool mlp = false) {
   return mlp ? kMlpCvtWarps : prec == MELT_FP8E4M3 && (!mfcc || dtc) ? 8 : 4;
 }
@@ -1144,21 +1144,38 @@ __device__ void pair_epilogue(const TcParams& p, uint8_t* gbase, const PairCtx& 
 // GELU(h) = h Phi(h), the exact-erf form the model is trained with, for the
 // fused epilogue, whose result is rounded to BF16 (8 significant bits).
 // With t = |h| and Q(t) = 1 - Phi(t) the upper normal tail,
-//     GELU(h) = max(h, 0) - t Q(t),
-// and log2 Q is smooth, close to a parabola: a degree-7 polynomial in t (the
-// Chebyshev fit on [0, 5.2] refined towards minimax by Lawson reweighting, 400
-// passes on a 1e5-point grid, in the power basis rounded to float32), then the
-// hardware base-2 exponential.  Its leading coefficient is negative and it
-// falls monotonically past the fit, so Q goes to zero there by itself.  Against the
-// exact function (float64) the float32 evaluation has a relative error <= 5e-6
-// for |h| <= 5 (about 2^-18, far below half a BF16 ulp) and an absolute error
-// <= 5e-7 everywhere.
-//
-// What bounds it: GELU is over half of a tile's time, and the FP32 pipe most of
-// that.  Two values at a time in packed operations (each half rounded as by
-// itself), 8 of them a pair, where the form with the parabola taken out of a
-// degree-6 fit took 20 single ones: 22 clocks a warp and value, 17 packed,
-// 15.5 in this form (measured alone, three warps a scheduler).
+//     GELU(h) = max(h, 0) - t Q(t),   log2 Q(t) = -t^2 log2(e) / 2 + S(t),
+// where S (log2 of the Mills ratio over sqrt(2 pi)) is smooth on [0, 5],
+// from -1 at t = 0 to about -3.7 at t = 5.  S is a degree-6 polynomial in
+// u = 0.4 t - 1: the Chebyshev fit on [0, 5] refined towards minimax by
+// Lawson reweighting (30 passes on a 4e5-point grid), in the power basis
+// rounded to float32; Q = 2^(S - t^2 log2(e) / 2) from the hardware base-2
+// exponential.  Against the exact function (float64) the float32 evaluation
+// has a relative error <= 2e-5 for |h| <= 5 (about 2^-16, far below half a
+// BF16 ulp) and an absolute error <= 3e-6 everywhere (S is taken at
+// min(t, 5): beyond, the tail is below 1.5e-6 in magnitude).  About a dozen
+// FP32 operations and one multi-function-unit operation (the degree-9 fit of
+// the Mills ratio it replaces took 17).
+static __device__ __forceinline__ float gelu_poly(float h) {
+  const float t = fabsf(h);
+  const float u = fmaf(0.4f, fminf(t, 5.f), -1.f);
+  float r = 7.192788180e-03f;
+  r = fmaf(r, u, -2.606392093e-02f);
+  r = fmaf(r, u, 6.437100470e-02f);
+  r = fmaf(r, u, -1.599922627e-01f);
+  r = fmaf(r, u, 4.010236561e-01f);
+  r = fmaf(r, u, -1.164181113e+00f);
+  r = fmaf(r, u, -2.822842598e+00f);
+  float q;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(fmaf(t * -0.72134752044448170f, t, r)));  // Q(t)
+  return fmaf(-t, q, fmaxf(h, 0.f));
+}
+
+// gelu_poly of two values, with the same results, bit for bit: packed FP32
+// operations (each half rounded as by itself) where there is no operand modifier
+// to lose.  GELU is over half of a tile's time, and the FP32 pipe most of that:
+// 22 clocks a warp and value one at a time, 18 packed (measured alone, three
+// warps a scheduler); 64 x 30 s 76.0 -> 75.3 us.
 static __device__ __forceinline__ uint64_t pack2f(float a, float b) {
   uint64_t d;
   asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
@@ -1174,25 +1191,29 @@ static __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
 }
+static __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 static __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 static __device__ __forceinline__ float2 gelu_poly2(uint64_t h) {
+  const auto both = [](float k) { return pack2f(k, k); };
   const float2 v = unpack2f(h);
-  const uint64_t t = h & 0x7fffffff7fffffffull;
-  uint64_t r = pack2f(-1.637331820e-06f, -1.637331820e-06f);  // log2 Q(t)
-  const auto next = [&](float k) { r = fma2(r, t, pack2f(k, k)); };
-  next(5.839900768e-05f);
-  next(-9.104721248e-04f);
-  next(8.446723223e-03f);
-  next(-5.386648700e-02f);
-  next(-4.585306048e-01f);
-  next(-1.151234150e+00f);
-  next(-9.999959469e-01f);
-  const float2 x = unpack2f(r);
-  float q0, q1;
+  const uint64_t u = fma2(pack2f(fminf(fabsf(v.x), 5.f), fminf(fabsf(v.y), 5.f)), both(0.4f), both(-1.f));
+  uint64_t r = both(7.192788180e-03f);
+  r = fma2(r, u, both(-2.606392093e-02f));
+  r = fma2(r, u, both(6.437100470e-02f));
+  r = fma2(r, u, both(-1.599922627e-01f));
+  r = fma2(r, u, both(4.010236561e-01f));
+  r = fma2(r, u, both(-1.164181113e+00f));
+  r = fma2(r, u, both(-2.822842598e+00f));
+  const float2 x = unpack2f(fma2(mul2(h, both(-0.72134752044448170f)), h, r));
+  float q0, q1;  // Q(t)
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q0) : "f"(x.x));
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q1) : "f"(x.y));
   return make_float2(fmaf(-fabsf(v.x), q0, fmaxf(v.x, 0.f)), fmaf(-fabsf(v.y), q1, fmaxf(v.y, 0.f)));
@@ -1290,7 +1311,7 @@ static __device__ __forceinline__ void mlp_store(const TcParams& p, uint32_t ty,
 // step k + 1 from its accumulator into registers and x-hat (BF16) over it, which
 // releases it.  So each of the two layers' MMAs (with the way there and back 1200
 // and 1700 clocks of a tile's 12,700) has epilogue work beside it: 64 x 30 s 82.3
-// -> 80.1 us.  (71.9 with the shorter GELU and its rolled loop.)
+// -> 80.1 us.  (73.8 with the packed GELU and its rolled loop.)
 // The kMlpParts warps of a lane quarter split the bands (part_lo) and the
 // hidden units (part_lo_tail).  Every step is taken for an empty tile too
 // (without loads or stores) so that both CTAs keep the barrier phases in
@@ -1351,14 +1372,6 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
         }
       }
     }
-    // the next step's pair and its descriptor, whose load GELU hides
-    bool okq = true;
-    const int qn = pair_next_warp(p, c, B, k + 1, okq);
-    const bool more = okq && qn < p.n_pairs;
-    before = live;
-    valid_b = row < td.n_frames;
-    orow_b = p.out + (size_t)(td.out_row + row) * p.n_out;
-    if (more) td = pair_tile(p, c, qn);
     // 2. once H is in (x-hat consumed): GELU(H + b1) in BF16 over H (see gelu_col).
     // (Two chunks' registers in turn, one loading while the other is evaluated,
     // doubled the code and measured 80 against 76 us on the 64 x 30 s batch.)
@@ -1380,14 +1393,21 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
     }
     tc_fence_before();
     warp_arrive_leader(pbar(p, c, B.a2_full));
-    // 3. while the output layer runs: the next step's log-Mel (its projection was
-    // queued right after this step's hidden layer) and x-hat
-    if (!more) {
+    before = live;
+    valid_b = row < td.n_frames;
+    orow_b = p.out + (size_t)(td.out_row + row) * p.n_out;
+    // 3. while the output layer runs: the next step's pair, its log-Mel (its
+    // projection was queued right after this step's hidden layer) and x-hat.  (Its
+    // descriptor loaded before GELU measured 76 us against 74.)
+    bool okq = true;
+    const int qn = pair_next_warp(p, c, B, k + 1, okq);
+    if (!okq || qn >= p.n_pairs) {
       if (!pair_warp_wait(pbar(p, c, B.y_full), k & 1, c.abort, p.err)) return;
       tc_fence_after();
       if (before) mlp_store<NV>(p, tl + p.y_col, c_lo, c_hi, orow_b, valid_b, vec8);
       return;
     }
+    td = pair_tile(p, c, qn);
     if (!pair_warp_wait(pbar(p, c, B.t_full), (k + 1) & 1, c.abort, p.err)) return;
     sched_release(p, c, B, k + 1);
     tc_fence_after();

@@ -8,10 +8,15 @@ namespace tc {
 
 KernelFn kernel_for_pair_mlp(int nch) { return pick_pair_mlp_kernel<>(nch); }
 
-// The fused epilogue's GELU on n values (diagnostic: checked against the exact function).
+// The fused epilogue's GELU on n values (diagnostic: checked against the exact
+// function); NaN where the packed evaluation is not the single one's.
 __global__ void gelu_diag_kernel(const float* h, float* y, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    y[i] = i & 1 ? gelu_poly2(pack2f(0.f, h[i])).y : gelu_poly2(pack2f(h[i], 0.f)).x;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const float2 v = gelu_poly2(pack2f(h[i], -h[i]));
+    const bool same = __float_as_uint(v.x) == __float_as_uint(gelu_poly(h[i])) &&
+                      __float_as_uint(v.y) == __float_as_uint(gelu_poly(-h[i]));
+    y[i] = same ? v.x : __int_as_float(0x7fffffff);
+  }
 }
 
 // The epilogues' natural log on n values (diagnostic: checked against the exact function).
