@@ -442,17 +442,22 @@ static __device__ __forceinline__ void fill_dct_split(const TcParams& p, uint8_t
 // written a tile's log-Mel rows (split into BF16 hi + lo) to TMEM, the
 // coefficients C = L D^T accumulate as hi*hi + hi*lo + lo*hi over the K-steps
 // of 16 Mel bins (the lo*lo term, below 2^-16 of each product, is dropped).
-static __device__ void pair_dct_gemm(const TcParams& p, const PairCtx& c, const PairBars& B, uint32_t tmem_base) {
-  const uint64_t hi = (uint64_t)p.desc_hi << 32;
+static __device__ __forceinline__ void pair_dct_gemm(const TcParams& p, const PairCtx& c, const PairBars& B,
+                                                     uint32_t tmem_base) {
   const uint32_t nh16 = (uint32_t)p.dct_n / 2 * 16;  // bytes between the two K core columns of a K-step
-  const uint32_t dhi = ((c.sbase + p.off_dct) >> 4) | ((nh16 >> 4) << 16);
-  const uint32_t dlo = dhi + (p.dct_part >> 4);
-  const uint32_t step16 = (2 * nh16) >> 4;
+  uint32_t dhi = ((c.sbase + p.off_dct) >> 4) | ((nh16 >> 4) << 16);
+  const uint32_t lo = p.dct_part >> 4, step16 = (2 * nh16) >> 4;
   const uint32_t d = tmem_base + p.dct_c;
-  for (int s = 0; s < p.MP / 16; ++s) {
-    mma_f16_pair_ts(d, tmem_base + p.dct_ahi + 8 * s, hi | (dhi + s * step16), p.idesc_dct, s > 0);
-    mma_f16_pair_ts(d, tmem_base + p.dct_ahi + 8 * s, hi | (dlo + s * step16), p.idesc_dct, true);
-    mma_f16_pair_ts(d, tmem_base + p.dct_alo + 8 * s, hi | (dhi + s * step16), p.idesc_dct, true);
+  uint32_t ah = tmem_base + p.dct_ahi, al = tmem_base + p.dct_alo;
+#pragma unroll
+  for (int s = 0; s < 8; ++s) {  // (M <= 128)
+    if (16 * s >= p.MP) break;
+    mma_f16_pair_ts(d, ah, desc64(dhi, p.desc_hi), p.idesc_dct, s > 0);
+    mma_f16_pair_ts(d, ah, desc64(dhi + lo, p.desc_hi), p.idesc_dct, true);
+    mma_f16_pair_ts(d, al, desc64(dhi, p.desc_hi), p.idesc_dct, true);
+    dhi += step16;
+    ah += 8;
+    al += 8;
   }
   mma_commit_pair_mc(pbar(p, c, B.h_full), 3);
 }
@@ -958,13 +963,12 @@ __device__ void pair_epilogue_dct(const TcParams& p, const PairCtx& c, const Pai
   int c_lo, c_hi, k_lo, k_hi;
   half_chunks(p.MP >> 4, EPW / 4, half, c_lo, c_hi);
   half_chunks(p.dct_n >> 4, EPW / 4, half, k_lo, k_hi);
-  for (int k = 0;; ++k) {
-    bool okq = true;
-    const int q = k == 0 ? c.cluster : pair_next_warp(p, c, B, k, okq);
-    if (!okq || q >= p.n_pairs) break;
+  int q = c.cluster;
+  TileDesc td;
+  if (q < p.n_pairs) td = pair_tile(p, c, q);
+  for (int k = 0; q < p.n_pairs; ++k) {
     const int acc = p.nacc == 2 ? (k & 1) : 0;
     const uint32_t tphase = p.nacc == 2 ? ((k >> 1) & 1) : (k & 1);
-    const TileDesc td = pair_tile(p, c, q);
     if (!pair_warp_wait(pbar(p, c, B.t_full + acc), tphase, c.abort, p.err)) break;
     sched_release(p, c, B, k);
     tc_fence_after();
@@ -1010,11 +1014,17 @@ __device__ void pair_epilogue_dct(const TcParams& p, const PairCtx& c, const Pai
     }
     tc_fence_before();
     warp_arrive_leader(pbar(p, c, B.t_empty + acc));
+    float* orow = p.out + (size_t)(td.out_row + row) * p.n_mfcc;
+    const bool valid = row < td.n_frames;
+    // the next pair's descriptor (1000 clocks and more from memory, the batch's
+    // samples having passed through L2) while the DCT runs
+    bool okq = true;
+    q = pair_next_warp(p, c, B, k + 1, okq);
+    if (!okq) q = p.n_pairs;
+    if (q < p.n_pairs) td = pair_tile(p, c, q);
     if (!pair_warp_wait(pbar(p, c, B.h_full), k & 1, c.abort, p.err)) break;
     tc_fence_after();
     if (live) {
-      float* orow = p.out + (size_t)(td.out_row + row) * p.n_mfcc;
-      const bool valid = row < td.n_frames;
 #pragma unroll 1
       for (int kc = k_lo; kc < k_hi; ++kc) {
         float v[16];
