@@ -20,7 +20,7 @@
 // Z row t + j, selected by the scale-factor byte j) and 2^-8 to the basis,
 // which is stored as e4m3(W 2^8).  The accumulator holds R and I directly.
 //
-// Warp roles per CTA (11 warps; 17 with the fused MLP):
+// Warp roles per CTA (11 warps; 17 with the fused MLP, up to 23 in FP8):
 //   warps 0-3   epilogue: TMEM -> registers, R^2 + I^2, log, (DCT), store (with
 //               the fused MLP, warps 0-11: warps e, e+4 and e+8 read the same
 //               32 TMEM lanes (frames) and split the bands and hidden units)
@@ -28,7 +28,7 @@
 //   next warp   basis producer: this CTA's half of the basis, once (with the
 //               fused MLP, the MMA warp before its first tile)
 //   next warp   waveform producer: bulk copies of the tile's FP32 span into a ring
-//   last four   converters: staged FP32 samples -> polyphase Z rows (BF16, or
+//   last        converters (four; FP8 up to 16): staged FP32 samples -> polyphase Z rows (BF16, or
 //               e4m3 with per-row scales written to TMEM; three warps with the
 //               fused MLP)
 //
@@ -84,16 +84,21 @@ __host__ __device__ constexpr int part_lo(int n, int parts, int j) {
 __host__ __device__ constexpr int part_lo_tail(int n, int parts, int j) {
   return j * (n / parts) + (j > parts - n % parts ? j - (parts - n % parts) : 0);
 }
-// Converter warps: 4 (BF16: each sample converted once, short chains), 8 for
-// FP8's log-Mel kernel and its MFCC kernel with the DCT on the tensor cores,
-// whose per-row max makes each chunk one dependent chain per row set (twice
-// the warps, half the chain).  The MFCC kernels with the DCT on the CUDA
-// cores keep 4 (their epilogue warps and registers fill the block).  With
+// Converter warps: 4 (BF16: each sample converted once, short chains); 16 for
+// FP8's log-Mel kernel, whose per-row max makes each chunk one dependent chain per
+// row set (64 x 30 s: 8 warps a chunk 50.3 us; two groups of 4, 48.9; of 8, 47.4;
+// three or four of 4, 52 and 66); 8 for its MFCC kernel with the DCT on the tensor
+// cores (groups of 4: 62.7 -> 60.8), beside 8 epilogue warps.  The MFCC kernels
+// with the DCT on the CUDA cores keep 4 (their epilogue warps and registers fill
+// the block).  With
 // the fused MLP, 3: the warps go to the epilogue (64 x 30 s: 2 / 3 / 4 converter
 // warps 75.3 / 73.8 / 76.2 us; 8 or 16 epilogue warps 75 and more).
 __host__ __device__ constexpr int pair_cvt_warps(int prec, bool mfcc, int nch, bool dtc = false, bool mlp = false) {
-  return mlp ? kMlpCvtWarps : prec == MELT_FP8E4M3 && (!mfcc || dtc) ? 8 : 4;
+  return mlp ? kMlpCvtWarps : prec != MELT_FP8E4M3 ? 4 : !mfcc ? 16 : dtc ? 8 : 4;
 }
+// Converter warps that share a staged chunk: half of FP8's, the halves taking
+// chunks in turn, so that two chunks' chains overlap.
+__host__ __device__ constexpr int pair_cvt_group(int prec, int cw) { return prec == MELT_FP8E4M3 && cw >= 8 ? cw / 2 : cw; }
 __host__ __device__ constexpr int pair_threads(bool mlp, int prec = MELT_BF16, bool mfcc = false, int nch = 1,
                                                bool dtc = false) {
   return 32 * (pair_epi_warps(mlp, mfcc, nch, dtc) + (mlp ? 2 : 3) + pair_cvt_warps(prec, mfcc, nch, dtc, mlp));
@@ -771,15 +776,42 @@ static __device__ __forceinline__ float4 clip_quad_sel(float4 x, int s, int nsam
   return x;
 }
 
+// Two FP32 values in a register pair, and operations on both (each rounded as by
+// itself).
+static __device__ __forceinline__ uint64_t pack2f(float a, float b) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+static __device__ __forceinline__ float2 unpack2f(uint64_t a) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(a));
+  return v;
+}
+static __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+static __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+static __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 // FP8 e4m3 converter: staged FP32 chunks -> polyphase Z rows of e4m3 with a
 // power-of-two scale per row, and the rows' scale codes in TMEM.
 //
 // Eight lanes share a Z row: lane l8 of a group holds quads l8, l8 + 8, ...
 // of the row (H <= 256: at most 8 each), so the row's max |x| is a local max
 // and three butterfly shuffles inside the group.  A warp takes four rows at a
-// time and both of its row sets of a chunk (rows 4 w + g and 4 w + g + 16,
-// chunks of at most 32 rows) at once: all of a chunk's loads are in flight
-// together and the two reductions overlap.  The row's exponent is the least
+// time, and all its row sets of a chunk (of at most 32 rows) at once: a chunk's
+// loads are in flight
+// together and the reductions overlap.  The row's exponent is the least
 // e with amax 2^-e <= 448; its samples are multiplied by 2^-e (exact) and
 // converted with saturating round-to-nearest-even.  Z element (u, r) sits at
 // (r / 16) lbo_a + 16 u + r % 16, so quad q of row u is 4 bytes at core
@@ -791,7 +823,7 @@ static __device__ __forceinline__ float4 clip_quad_sel(float4 x, int s, int nsam
 // column t / 32 of the group).
 constexpr int kF8LanesPerRow = 8;
 constexpr int kF8MaxQuads = 8;   // quads per lane per row: H <= 4 * 8 * 8 = 256
-constexpr int kF8MaxRows = 32;   // rows per staged chunk: two sets of 4 rows per warp
+constexpr int kF8MaxRows = 32;   // rows per staged chunk: 32 / (4 warps of a group) sets of 4 rows per warp
 
 // One staged chunk of the FP8 converter (rows [r0, r0 + rows) of the tile's
 // Z rows): NQ = quads per lane per row (ceil(H / 32)), a compile-time count
@@ -804,6 +836,7 @@ static __device__ __forceinline__ void fp8_convert_chunk(const TcParams& p, uint
   const int h4 = p.H >> 2;
   const int s_base = r0 * p.H;
   const bool tail = s_base + rows * p.H > nsamp;
+  const bool whole = rows == kF8MaxRows && h4 == kF8LanesPerRow * NQ;  // every quad below is one of the chunk's
   // loads at clamped (always valid) addresses; quads outside the chunk's rows
   // or past H are zeroed by selects after
   float4 x[NS][NQ];
@@ -824,14 +857,16 @@ static __device__ __forceinline__ void fp8_convert_chunk(const TcParams& p, uint
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const int j = kF8LanesPerRow * q + l8;
-      const bool live = u < rows && j < h4;
       float4 v = x[h][q];
-      if (tail) v = clip_quad_sel(v, s_base + u * p.H + 4 * j, nsamp);
-      v.x = live ? v.x : 0.f;
-      v.y = live ? v.y : 0.f;
-      v.z = live ? v.z : 0.f;
-      v.w = live ? v.w : 0.f;
-      x[h][q] = v;
+      if (tail || !whole) {
+        const bool live = u < rows && j < h4;
+        if (tail) v = clip_quad_sel(v, s_base + u * p.H + 4 * j, nsamp);
+        v.x = live ? v.x : 0.f;
+        v.y = live ? v.y : 0.f;
+        v.z = live ? v.z : 0.f;
+        v.w = live ? v.w : 0.f;
+        x[h][q] = v;
+      }
       m[h] = fmaxf(m[h], fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
     }
   }
@@ -845,12 +880,15 @@ static __device__ __forceinline__ void fp8_convert_chunk(const TcParams& p, uint
     const bool row_live = u < rows;
     const uint32_t code = fp8_row_code(__float_as_uint(m[h]));
     const float inv = __uint_as_float((254u - code) << 23);  // 2^-e, e = code - 127
+    const uint64_t inv2 = pack2f(inv, inv);
     sts8_if(codes_s + (uint32_t)(r0 + u), code, row_live && l8 == 0);
     const uint32_t zrow = zaddr + 16u * (uint32_t)(r0 + u);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const int j = kF8LanesPerRow * q + l8;
-      const uint32_t w = pack_e4m3x4(x[h][q].x * inv, x[h][q].y * inv, x[h][q].z * inv, x[h][q].w * inv);
+      const float2 lo = unpack2f(mul2(pack2f(x[h][q].x, x[h][q].y), inv2));
+      const float2 hi = unpack2f(mul2(pack2f(x[h][q].z, x[h][q].w), inv2));
+      const uint32_t w = pack_e4m3x4(lo.x, lo.y, hi.x, hi.y);
       sts32_if(zrow + (uint32_t)(j >> 2) * p.lbo_a + 4u * (uint32_t)(j & 3), w, row_live && j < h4);
     }
   }
@@ -887,7 +925,8 @@ static __device__ void pair_convert_fp8(const TcParams& p, uint8_t* gbase, const
   for (uint32_t o = 16u * (uint32_t)(threadIdx.x - 32 * cvt0); o < p.abuf_bytes * p.ZB; o += 16u * kThr)
     sts128(c.sbase + p.off_a + o, make_uint4(0u, 0u, 0u, 0u));
   fence_proxy_async();
-  int slot = 0;
+  constexpr int GW = pair_cvt_group(MELT_FP8E4M3, CW);
+  int slot = 0, turn = 0;  // whose chunk it is
   uint32_t sphase = 0;
   for (int k = 0;; ++k) {
     bool okq = true;
@@ -903,14 +942,17 @@ static __device__ void pair_convert_fp8(const TcParams& p, uint8_t* gbase, const
     uint8_t* codes = codes_all + zb * p.codes_stride;
     const uint32_t codes_s = smem_u32(codes);
     for (int ch = 0; ok && td.n_frames > 0 && ch < p.NCHUNK; ++ch) {
-      if (!warp_wait(pbar(p, c, B.s_full + slot), sphase, c.abort, p.err)) {
-        ok = false;
-        break;
+      if (turn == cw / GW) {
+        if (!warp_wait(pbar(p, c, B.s_full + slot), sphase, c.abort, p.err)) {
+          ok = false;
+          break;
+        }
+        const int r0 = ch * p.CH;
+        fp8_convert_chunk_any<GW>(p, nqr, st0 + slot * p.st_bytes, zaddr, codes_s, r0, min(p.CH, p.zrows - r0),
+                                  nsamp, cw % GW, g, l8);
+        warp_arrive(pbar(p, c, B.s_empty + slot));
       }
-      const int r0 = ch * p.CH;
-      fp8_convert_chunk_any<CW>(p, nqr, st0 + slot * p.st_bytes, zaddr, codes_s, r0, min(p.CH, p.zrows - r0),
-                                nsamp, cw, g, l8);
-      warp_arrive(pbar(p, c, B.s_empty + slot));
+      if (++turn == CW / GW) turn = 0;
       if (++slot == p.NS) {
         slot = 0;
         sphase ^= 1;
@@ -1186,31 +1228,6 @@ static __device__ __forceinline__ float gelu_poly(float h) {
 // to lose.  GELU is over half of a tile's time, and the FP32 pipe most of that:
 // 22 clocks a warp and value one at a time, 18 packed (measured alone, three
 // warps a scheduler); 64 x 30 s 76.0 -> 75.3 us.
-static __device__ __forceinline__ uint64_t pack2f(float a, float b) {
-  uint64_t d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
-  return d;
-}
-static __device__ __forceinline__ float2 unpack2f(uint64_t a) {
-  float2 v;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(a));
-  return v;
-}
-static __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-static __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-static __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
 static __device__ __forceinline__ float2 gelu_poly2(uint64_t h) {
   const auto both = [](float k) { return pack2f(k, k); };
   const float2 v = unpack2f(h);
@@ -1457,7 +1474,7 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
     auto bar = [&](int i) { return sbase + p.off_bar + 8 * i; };
     for (int i = 0; i < p.NS; ++i) {
       mbar_init(bar(B.s_full + i), 1);
-      mbar_init(bar(B.s_empty + i), CW);
+      mbar_init(bar(B.s_empty + i), pair_cvt_group(PREC, CW));
     }
     for (int i = 0; i < p.ZB; ++i) {
       mbar_init(bar(B.z_full + i), 2 * CW);  // converters of both CTAs (even CTA's copy is used)
