@@ -50,7 +50,7 @@
 // bins), 8-10 and 12-14 converters (each takes whole slabs by itself: its samples
 // arrive by asynchronous copies in a staging area of its own, one arrival per
 // slab), 11 MMA issue (odd CTA: forwards its basis fills to the even one), 15
-// basis producer and L2 prefetch.
+// basis producer.
 //
 // Code size counts here: the issue thread's few hundred instructions per chunk
 // run once per 1200 clocks between three other warps on its scheduler, and it
@@ -244,14 +244,10 @@ static __device__ __forceinline__ int slab_steps(const SlabParams& p, int kk) {
   return 16 * kk < p.n_last ? p.J : p.J - 1;
 }
 
-// Bulk prefetch of a tile's samples into L2 (pieces of <= 32 KB).
-static __device__ __forceinline__ void prefetch_span(const SlabParams& p, const TileDesc& td) {
-  if (td.n_frames == 0) return;
-  const int avail = min((td.n_samples & 3) ? (td.n_samples | 3) + 1 : td.n_samples, (td.n_frames + p.J - 1) * p.H);
-  for (int o = 0; o < avail; o += 8192) prefetch_l2(p.wave + td.in_off + o, (uint32_t)min(8192, avail - o) * 4u);
-}
-
 // ---- basis producer: each unit's K-steps of this CTA's half, stage by stage
+// (A bulk prefetch of the next tile's samples into L2 from here, a unit ahead of the
+// converters, cost more than it gave: 64 x 30 s FP32 91.6 us with, 90.2 without; 256
+// x 10 s split BF16 76.2, 73.5; BF16 at 22.05 kHz, 64 x 20 s 42.1, 40.8.)
 template <int P>
 static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const SlabBars& B) {
   const uint64_t pol = policy_evict_last();
@@ -263,7 +259,6 @@ static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const S
     const int ng = blk_groups(p, b);
     const uint32_t blk = (uint32_t)ng * P * 256u;
     const uint8_t* src = half + (size_t)b * p.wbg * P * 256u;
-    bool ahead = false;  // the next unit's span has been sent for
     for (int kk = 0; ok && kk < p.n_slab; ++kk) {
       const int js = slab_steps(p, kk);
       for (int j0 = 0; j0 < js; j0 += p.kps) {
@@ -283,13 +278,6 @@ static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const S
         src += (size_t)n * p.step_bytes;
         ++issued;
         r.next(p.NS);
-        if (!ahead) {
-          // L2 prefetch of the samples, one unit ahead of the converters' copies
-          ahead = true;
-          if (i == 0 && !p.early_inputs) pdl_wait();
-          int qn, bn;
-          if (unit_at(p, c, i + 1, qn, bn) && (qn != q || i == 0)) prefetch_span(p, tile_of(p, c, qn));
-        }
       }
     }
   }
@@ -330,12 +318,6 @@ static __device__ void basis_producer_slices(const SlabParams& p, const Ctx& c, 
         src += (size_t)n * p.step_bytes;
         ++issued;
         r.next(p.NB);
-      }
-      if (j == 0) {
-        // L2 prefetch of the samples, one unit ahead of the converters' copies
-        if (i == 0 && !p.early_inputs) pdl_wait();
-        int qn, bn;
-        if (unit_at(p, c, i + 1, qn, bn) && (qn != q || i == 0)) prefetch_span(p, tile_of(p, c, qn));
       }
     }
   }
