@@ -237,8 +237,8 @@ void order_longest_first(TileDesc* t, long long n) {
 }
 
 // The FP32 form over n_tiles device descriptors: the slab kernel with three-part
-// split operands (64 x 30 s, N 400, 80 bins: 97 us against 508 us as FFMAs on the
-// CUDA cores; 8 x 1 s: 13.5 against 52 us; one 160 s clip, N 1200, 128 bins, 40
+// split operands (64 x 30 s, N 400, 80 bins: 96 us against 505 us as FFMAs on the
+// CUDA cores; 8 x 1 s: 9.4 against 53 us; one 160 s clip, N 1200, 128 bins, 40
 // MFCCs: 59 against 421 us), or (mode 1) the raw projections on the CUDA cores.
 cudaError_t launch_fp32(melt_basis* b, const float* wave, const TileDesc* tiles, int n_tiles, float* out, int mode,
                         unsigned flags, cudaStream_t stream) {

@@ -358,8 +358,8 @@ int candidate_list(const TcBasis* tb, const TcParams& p, melt_plan* out, int cap
   }
   // CTA pairs with each CTA's half basis streamed: a 2-SM MMA shares every basis
   // block between two tiles.  The slab kernel runs these where it is built for
-  // the basis, and they come first there (256 x 10 s split BF16 81 us against 114
-  // us single-CTA; BF16 at 22.05 kHz, N = 1024, 64 x 20 s 42 against 56 us; at
+  // the basis, and they come first there (256 x 10 s split BF16 77 us against 114
+  // us single-CTA; BF16 at 22.05 kHz, N = 1024, 64 x 20 s 41 against 56 us; at
   // N = 1200, 128 bins, 16 x 30 s 29 against 33 us).  The pair kernel's own
   // streamed layout measured no faster than the single-CTA ones (64 x 30 s split
   // BF16: 86.6 against 83.4 us), so elsewhere they come after those, for

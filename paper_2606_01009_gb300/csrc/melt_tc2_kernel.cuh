@@ -564,7 +564,9 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
     m.sfa = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * zb);
     m.w = b0;
     if (PREC != MELT_FP8E4M3 && !MLP && !DTC && !p.b_resident) {  // (planned for these only)
-      // streamed half basis: slot by slot, each once both CTAs' halves are in
+      // streamed half basis: slot by slot, each once both CTAs' halves are in.  (One
+      // election for a slot, not one a K-step: two bases' 4096 clips in one launch 1066
+      // us for 1146; split BF16 at N = 640, hop 64, 64 x 20 s 132 for 170.)
       int j = 0, k0 = 0;
       for (int s0 = 0; s0 < p.KS; s0 += p.kps, ++g) {
         const int slot = g % p.NB;
@@ -574,20 +576,22 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
         }
         tc_fence_after();
         uint32_t w = b0 + (uint32_t)slot * (p.bslot_bytes >> 4);
-        for (int left = min(p.kps, p.KS - s0); left > 0;) {
-          const int n = min(min(kU, left), (j + 1 < J ? nk : nk_last) - k0);
-          if (elect_one()) pair_steps<PREC, kU>(m, j, k0, n, w);
+        for (int left = min(p.kps, p.KS - s0); left > 0;) {  // (a slot may run on into the next slice)
+          const int nj = j + 1 < J ? nk : nk_last, n = min(left, nj - k0);
+          if (elect_one()) {
+#pragma unroll 1
+            for (int u = 0; u < n; u += 4) pair_steps<PREC, 4>(m, j, k0 + u, min(4, n - u), w + (uint32_t)u * m.w_step);
+            if (left == n) commit(B.bs_empty + slot);
+          }
           __syncwarp();
           w += (uint32_t)n * m.w_step;
           left -= n;
           k0 += n;
-          if (k0 == (j + 1 < J ? nk : nk_last)) {
+          if (k0 == nj) {
             k0 = 0;
             ++j;
           }
         }
-        if (elect_one()) commit(B.bs_empty + slot);
-        __syncwarp();
       }
       if (!ok) break;
     } else if (elect_one()) {
