@@ -509,7 +509,7 @@ static __device__ __forceinline__ void pair_steps(const PairSteps& m, int j, int
 // 4096 mixed clips 711 -> 692.)  The waits acquire at CTA scope, 100 clocks for
 // 250 at cluster scope: what the peer wrote is read by the MMAs only, through the
 // async proxy, after its writers' proxy fences.
-template <bool MLP, int PREC, bool DTC = false>
+template <bool MLP, int PREC, bool DTC, bool GRP>
 static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairBars& B, uint32_t tmem_base) {
   // K-steps issued in a run.  Longer ones pay only where the DCT's MMAs wait behind
   // them (MFCC 43.6 us with 5, 44.3 with 1; log-Mel 38.5 and 38.2).
@@ -564,9 +564,12 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
     m.sfa = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * zb);
     m.w = b0;
     if (PREC != MELT_FP8E4M3 && !MLP && !DTC && !p.b_resident) {  // (planned for these only)
-      // streamed half basis: slot by slot, each once both CTAs' halves are in.  (One
-      // election for a slot, not one a K-step: two bases' 4096 clips in one launch 1066
-      // us for 1146; split BF16 at N = 640, hop 64, 64 x 20 s 132 for 170.)
+      // streamed half basis: slot by slot, each once both CTAs' halves are in.  One
+      // election for a slot where streaming is what the kernel is for (two bases' 4096
+      // clips in one launch 1074 us for 1146; split BF16 at N = 640, hop 64, 64 x 20 s
+      // 134 for 170); one a K-step in the BF16 log-Mel kernel, whose resident loop is
+      // 0.8 % slower beside any other form of this one (38.4 for 38.05 us)
+      constexpr bool kSlotRuns = GRP || PREC == MELT_BF16X3;
       int j = 0, k0 = 0;
       for (int s0 = 0; s0 < p.KS; s0 += p.kps, ++g) {
         const int slot = g % p.NB;
@@ -576,22 +579,38 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
         }
         tc_fence_after();
         uint32_t w = b0 + (uint32_t)slot * (p.bslot_bytes >> 4);
-        for (int left = min(p.kps, p.KS - s0); left > 0;) {  // (a slot may run on into the next slice)
-          const int nj = j + 1 < J ? nk : nk_last, n = min(left, nj - k0);
-          if (elect_one()) {
+        if constexpr (kSlotRuns) {
+          for (int left = min(p.kps, p.KS - s0); left > 0;) {  // (a slot may run on into the next slice)
+            const int nj = j + 1 < J ? nk : nk_last, n = min(left, nj - k0);
+            if (elect_one()) {
 #pragma unroll 1
-            for (int u = 0; u < n; u += 4) pair_steps<PREC, 4>(m, j, k0 + u, min(4, n - u), w + (uint32_t)u * m.w_step);
-            if (left == n) commit(B.bs_empty + slot);
+              for (int u = 0; u < n; ++u) pair_steps<PREC, 1>(m, j, k0 + u, 1, w + (uint32_t)u * m.w_step);
+            }
+            __syncwarp();
+            w += (uint32_t)n * m.w_step;
+            left -= n;
+            k0 += n;
+            if (k0 == nj) {
+              k0 = 0;
+              ++j;
+            }
           }
-          __syncwarp();
-          w += (uint32_t)n * m.w_step;
-          left -= n;
-          k0 += n;
-          if (k0 == nj) {
-            k0 = 0;
-            ++j;
+        } else {
+          for (int left = min(p.kps, p.KS - s0); left > 0;) {
+            const int n = min(min(kU, left), (j + 1 < J ? nk : nk_last) - k0);
+            if (elect_one()) pair_steps<PREC, kU>(m, j, k0, n, w);
+            __syncwarp();
+            w += (uint32_t)n * m.w_step;
+            left -= n;
+            k0 += n;
+            if (k0 == (j + 1 < J ? nk : nk_last)) {
+              k0 = 0;
+              ++j;
+            }
           }
         }
+        if (elect_one()) commit(B.bs_empty + slot);
+        __syncwarp();
       }
       if (!ok) break;
     } else if (elect_one()) {
@@ -1454,7 +1473,7 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
 
 // The work of one CTA of a pair kernel: cluster `cluster` of `n_clusters`
 // clusters that share the tile list of `p`.
-template <int NCH, bool MFCC, bool MLP, int PREC, bool DTC>
+template <int NCH, bool MFCC, bool MLP, int PREC, bool DTC, bool GRP = false>  // GRP: of a two-basis launch
 __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_clusters) {
   constexpr int EPW = pair_epi_warps(MLP, MFCC, NCH, DTC);
   // (fused MLP: the MMA warp is the basis producer first)
@@ -1552,7 +1571,7 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
   if (warp == kPMmaWarp) {
     if (MLP && lane == 0) pair_basis_producer(p, c, B);
     __syncwarp();
-    if (c.rank == 0) pair_mma<MLP, PREC, DTC>(p, c, B, __shfl_sync(0xffffffffu, tmem_base, 0));
+    if (c.rank == 0) pair_mma<MLP, PREC, DTC, GRP>(p, c, B, __shfl_sync(0xffffffffu, tmem_base, 0));
     else if (lane == 0 && !p.b_resident) pair_basis_signal(p, c, B);  // the odd CTA's slots, to the even CTA
     if (lane == 0) drain_wait(pbar(p, c, B.drain), 0, p.err);
     __syncwarp();
@@ -1619,7 +1638,7 @@ __global__ void __launch_bounds__(pair_threads(MLP, PREC, MFCC, NCH, DTC), 1)
     melt_tc_pair_group_kernel(const __grid_constant__ TcGroupParams q) {
   const int cl = (int)(blockIdx.x >> 1), nc = (int)(gridDim.x >> 1);
   const bool second = cl >= q.split;
-  pair_cta<NCH, MFCC, MLP, PREC, DTC>(second ? q.g[1] : q.g[0], second ? cl - q.split : cl,
+  pair_cta<NCH, MFCC, MLP, PREC, DTC, true>(second ? q.g[1] : q.g[0], second ? cl - q.split : cl,
                                       second ? nc - q.split : q.split);
 }
 
