@@ -11,7 +11,7 @@ the stream, so each launch stages samples while the previous one drains).
   e2e       frames/s through the public Python API with pinned HOST buffers:
             H2D of the step's waveforms, the forward, D2H of its features
   roofline  dominant kernel vs the measured HBM copy bandwidth
-            (bound "hbm", for FP32 "tensor": its six BF16 products)
+            (bound "hbm" for the tensor-core forms, "alu" for FP32 SIMT)
   cpu_baseline  the FP64 oracle on the host cores on a bounded sample
 
 Inputs larger than L2: the step's inputs and outputs rotate over several
@@ -405,10 +405,12 @@ def roofline(cfg, W, r, peaks, peak_kind):
     alg_bytes = algorithmic_bytes(W.lens, cfg["n_fft"], cfg["hop"], n_out)
     sec = r["launch_ms"] / 1e3
     if prec == "fp32":
-        peak, ach = peaks["bf16_tflops"], 6 * flops / sec / 1e12
-        return {"bound": "tensor", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-                "traffic": None, "peak_note": f"bf16_tflops of {peak_kind} peaks; six BF16 products of the split operands",
-                "algorithmic_flops_per_launch": 6 * flops, "launch_ms": r["launch_ms"]}
+        peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+        ach = flops / sec / 1e12
+        return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                "traffic": None, "peak_note": "FP32 FFMA peak derived: 152 SMs x 128 lanes x 2 FLOP x "
+                f"{peaks.get('sm_max_mhz', 2070.0):.0f} MHz max SM clock",
+                "algorithmic_flops_per_launch": flops, "launch_ms": r["launch_ms"]}
     ach = alg_bytes / sec / 1e9
     peak = peaks["hbm_gbs"]
     key = f"{prec}/{W.name}/n_mels={cfg['n_mels']}/n_out={n_out}"
@@ -863,8 +865,9 @@ def frontend_leg(melt, dev, clips, cfg, precision, n_mfcc=0, steps=10, peaks=Non
            "frames_per_s": T / (ms / 1e3), "hbm_gbs": alg / (ms / 1e3) / 1e9}
     if peaks:
         if precision == "fp32":
-            flops = 6 * 2 * cfg["n_fft"] * 2 * cfg["n_mels"] * T
-            res["roofline_frac"], res["bound"] = flops / (ms / 1e3) / (peaks["bf16_tflops"] * 1e12), "tensor"
+            flops = 2 * cfg["n_fft"] * 2 * cfg["n_mels"] * T
+            peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6
+            res["roofline_frac"], res["bound"] = flops / (ms / 1e3) / peak, "alu"
         else:
             res["roofline_frac"], res["bound"] = res["hbm_gbs"] / peaks["hbm_gbs"], "hbm"
     if oracle_clips:
