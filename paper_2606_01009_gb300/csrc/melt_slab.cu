@@ -86,13 +86,13 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
     // tile of them) as leave three basis slots; then more of those.  Measured,
     // split BF16 256 x 10 s: 6 / 4 / 3 teams 76 / 77 / 81 us with 5 slabs, 2 / 8
     // slabs (fewer teams) 82 / 78; BF16 at 22.05 kHz, 64 x 20 s: 10 / 7 / 4 slabs
-    // 42.4 / 43.8 / 45.2.
+    // 42.4 / 43.8 / 45.2.  (Never more teams than slots: see SlabParams::ncv.)
     for (int least_nb = 3; least_nb >= 2; --least_nb)
       for (int teams : {6, 4, 3, 2}) {
         const uint32_t other = fixed + teams * kRawBytes;
         if (end || other + least_nb * basis >= kSmemMax) continue;
         const int na = std::min({(int)((kSmemMax - other - least_nb * basis) / p.stage), 2 * p.n_slab, kMaxA});
-        if (na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
+        if (teams > na || na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
         p.NS = na;
         p.NB = std::min<int>(kMaxB, (int)((kSmemMax - other - na * p.stage) / basis));
         p.ncv = teams;
