@@ -67,8 +67,8 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
   p.nacc = wbg <= 10 ? 3 : 2;
   p.acc_cols = wbg <= 10 ? 160 : 256;
   const uint32_t basis = up((uint32_t)wbg * P * 256u * p.kps, 128);
-  const uint32_t fixed = up(8u * SlabBars(P == 3 ? kMaxStages : kMaxA, P == 3 ? 0 : kMaxB).total, 128) + 128u +
-                         mfcc_bytes(p, n_mfcc) + 128u;
+  const auto bars = [](int ns, int nb) { return up(8u * SlabBars(ns, nb).total, 128); };
+  const uint32_t fixed = mfcc_bytes(p, n_mfcc) + 256u;
   uint32_t end = 0;  // of the rings
   if (P == 3) {
     p.stage = p.a_bytes + basis;
@@ -77,7 +77,7 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
       p.NS = ns;
       p.ncv = std::min(ns, kMaxTeams);
       p.tw = 1;
-      if (fixed + p.ncv * kRawBytes + ns * p.stage <= kSmemMax) end = p.stage * ns;
+      if (fixed + bars(kMaxStages, 0) + p.ncv * kRawBytes + ns * p.stage <= kSmemMax) end = p.stage * ns;
     }
   } else {
     p.stage = p.a_bytes;
@@ -90,11 +90,13 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
     for (int least_nb = 3; least_nb >= 2; --least_nb)
       for (int teams : {6, 4, 3, 2}) {
         const uint32_t other = fixed + teams * kRawBytes;
-        if (end || other + least_nb * basis >= kSmemMax) continue;
-        const int na = std::min({(int)((kSmemMax - other - least_nb * basis) / p.stage), 2 * p.n_slab, kMaxA});
+        const auto left = [&](int na, int nb) { return (int)(kSmemMax - other - bars(na, nb)) - (int)p.stage * na; };
+        if (end || left(0, least_nb) < (int)(least_nb * basis)) continue;
+        int na = std::min({(left(0, least_nb) - (int)(least_nb * basis)) / (int)p.stage, 2 * p.n_slab, kMaxA});
+        if (left(na, least_nb) < (int)(least_nb * basis)) --na;  // (its own barriers)
         if (teams > na || na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
         p.NS = na;
-        p.NB = std::min<int>(kMaxB, (int)((kSmemMax - other - na * p.stage) / basis));
+        p.NB = std::max(least_nb, std::min(kMaxB, left(na, kMaxB) / (int)basis));
         p.ncv = teams;
         p.tw = cvt_warps(P) / teams;
         p.off_b = p.stage * na;
@@ -104,7 +106,7 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
   if (!end) return false;
   p.off_raw = end;
   p.off_bar = p.off_raw + p.ncv * kRawBytes;
-  p.off_misc = p.off_bar + up(8u * SlabBars(p.NS, p.NB).total, 128);
+  p.off_misc = p.off_bar + bars(p.NS, p.NB);
   p.off_dct = p.off_misc + 128u;
   p.off_part = p.off_dct + up(4u * n_mfcc * 8u * p.groups, 128);
   return true;

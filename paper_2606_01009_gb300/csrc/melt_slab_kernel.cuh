@@ -120,7 +120,7 @@ struct SlabParams {
   int nacc;            // TMEM accumulators, acc_cols columns apart
   uint32_t acc_cols;
   int ncv, tw;         // converter teams at work (at most NS: a team that took slab g waits for the place of slab
-                       // g + ncv by one parity bit, which tells only neighbouring phases apart), warps of a team
+                       // g + ncv by a parity, which tells only neighbouring phases apart), warps of a team
   uint32_t lbo_a, a_part, a_bytes, stage, step_bytes;  // a stage: A (a_bytes: P parts of two core columns), then B;
                                                        // P 1, 2: an A slot
   uint32_t off_b, b_slot;  // P 1, 2: the basis ring
@@ -129,13 +129,33 @@ struct SlabParams {
   int early_inputs;    // the waveform's readers need not wait for the stream's previous kernel
 };
 
+// P 1, 2: the `empty` barrier that the MMAs of slot `slot`'s turn `turn` (0, 1,
+// ...) complete, and the one and its phase parity that a converter waits for
+// before it fills a slot.
+// Two barriers a slot, one for its even turns and one for the odd ones.  A team
+// waits only for its own slabs' places, and the slabs of a tile are freed out of
+// order (those past the last slice's end a slice early), so when a team comes to
+// slab g even slab g - 2 NS may not be freed, and the parity of one barrier cannot
+// tell that from g - NS being freed.  Slab g - 3 NS is: the team took the place of
+// slab h = g - ncv - NS >= g - 2 NS; the MMAs begin slabs in order, so all up to h
+// had been filled when h was freed, g - 2 NS into the place of g - 3 NS.
+__host__ __device__ constexpr int freed_bar(int NS, int slot, uint32_t turn) { return slot + (turn & 1 ? NS : 0); }
+// `pos`: the slab's place among two turns of the slots (slot + NS in odd turns),
+// `phase`: how often these have come round.  The barrier is the turn before's (at
+// the start the parity is that of the phase before its first, which passes).
+__host__ __device__ constexpr int place_bar(int NS, int pos) { return pos >= NS ? pos - NS : pos + NS; }
+__host__ __device__ constexpr uint32_t place_parity(int NS, int pos, uint32_t phase) {
+  return (phase ^ (pos >= NS ? 0u : 1u)) & 1u;
+}
+
 struct SlabBars {
   int full, empty, b_full, b_empty, t_full, t_empty, part, drain, total;
   // P 3: NS stages, NB = 0.  P 1, 2: NS A slots and NB basis slots.
   __host__ __device__ SlabBars(int NS, int NB) {
     full = 0;                 // converters of both CTAs (even CTA's copy is used); P 3: and the basis, as b_full
-    empty = full + NS;        // MMA commit, both CTAs
-    b_full = empty + NS;      // this CTA's basis copies; even CTA: and the odd one's signal that its own are in
+    empty = full + NS;        // MMA commit, both CTAs; P 1, 2: two a slot (freed_bar)
+    b_full = empty + (NB > 0 ? 2 : 1) * NS;  // this CTA's basis copies; even CTA: and the odd one's signal that its own
+                                             // are in
     b_empty = b_full + NB;    // MMA commit, both CTAs
     t_full = b_empty + NB;    // MMA commit, both CTAs
     t_empty = t_full + kMaxAcc;  // both CTAs' epilogues (even CTA's copy is used)
@@ -492,12 +512,12 @@ static __device__ void mma_issue_slices(const SlabParams& p, const Ctx& c, const
   for (int i = 0; ok && unit_at(p, c, i, q, b); ++i) {
     const uint32_t ng = (uint32_t)blk_groups(p, b);
     const uint32_t idesc = idesc_f32acc(1u, 2 * kF, 16u * ng), step = ng * ((P * 256u) >> 4);
-    const int slot0 = ra.slot;  // the unit's first slab
+    const int slot0 = ra.slot, free0 = freed_bar(NS, ra.slot, ra.phase);  // the unit's first slab
     ok = warp_wait(bar_at(p, c, B.t_empty + rt.slot), rt.phase ^ 1, c.abort, p.err);
     for (int j = 0; ok && j < J; ++j) {
       const int nk = j + 1 < J ? n_slab : last;
       const int free_from = j + 1 == J ? 0 : j + 2 == J ? last : n_slab;  // slabs this slice is the last of
-      int slot = slot0;
+      int fr = free0;  // (slabs in order take these barriers round and round)
       uint32_t at = (uint32_t)slot0 * as;
       for (int k0 = 0; k0 < nk; k0 += kps) {
         const int n = min(kps, nk - k0);
@@ -527,17 +547,15 @@ static __device__ void mma_issue_slices(const SlabParams& p, const Ctx& c, const
           }
           mma_commit_pair_mc(b_empty + 8 * rb.slot, 3);
           for (int k = max(0, free_from - k0); k < n; ++k) {
-            const int sl = slot + k < NS ? slot + k : slot + k - NS;
-            mma_commit_pair_mc(empty + 8 * sl, 3);
+            const int f = fr + k < 2 * NS ? fr + k : fr + k - 2 * NS;
+            mma_commit_pair_mc(empty + 8 * f, 3);
           }
         }
         __syncwarp();
-        slot += n;
+        fr += n;
+        if (fr >= 2 * NS) fr -= 2 * NS;
         at += (uint32_t)n * as;
-        if (slot >= NS) {
-          slot -= NS;
-          at -= a_end;
-        }
+        if (at >= a_end) at -= a_end;
         bl += bs;
         rb.next(NB);
         if (rb.slot == 0) bl = b0;
@@ -607,6 +625,7 @@ static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars
   const int U = P == 3 ? unit_stages(p) : p.n_slab, last = (p.n_last + 15) / 16;
   const int per = P == 3 ? (p.J + p.kps - 1) / p.kps : 1, per2 = max(1, (p.J - 1 + p.kps - 1) / p.kps);  // stages of a slab
   int i = 0, st = 0, kk = 0, j0 = 0, q, b;
+  const int round = P < 3 ? 2 * p.NS : p.NS;  // P 1, 2: two turns of the slots (place_bar)
   Ring r;
   TileDesc td, nxt;
   bool more = unit_at(p, c, 0, q, b);
@@ -614,7 +633,11 @@ static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars
   bool more_n = more && unit_at(p, c, 1, q, b);
   if (more_n) nxt = tile_of(p, c, q);
   auto step = [&](int n) {  // n stages on
-    for (int k = 0; k < n; ++k) r.next(p.NS);
+    r.slot += n;  // (n <= ncv <= NS)
+    if (r.slot >= round) {
+      r.slot -= round;
+      r.phase ^= 1;
+    }
     st += n;
     while (st >= U && more) {
       st -= U;
@@ -644,9 +667,12 @@ static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars
   step(w);
   if (more) copy();
   while (more) {
-    if (!warp_wait(bar_at(p, c, B.empty + r.slot), r.phase ^ 1, c.abort, p.err)) break;
+    const int slot = P < 3 && r.slot >= p.NS ? r.slot - p.NS : r.slot;
+    if (!warp_wait(bar_at(p, c, B.empty + (P < 3 ? place_bar(p.NS, r.slot) : slot)),
+                   P < 3 ? place_parity(p.NS, r.slot, r.phase) : r.phase ^ 1, c.abort, p.err))
+      break;
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    uint32_t at = to + r.slot * p.stage, from = raw;
+    uint32_t at = to + slot * p.stage, from = raw;
 #pragma unroll 4
     for (int u = u0; u < rows; u += 8 * TW, at += 128 * TW, from += 512 * TW) {
       float a0, a1, a2, a3;
@@ -664,7 +690,7 @@ static __device__ void convert(const SlabParams& p, const Ctx& c, const SlabBars
       }
     }
     fence_proxy_async();
-    warp_arrive_leader(bar_at(p, c, B.full + r.slot));
+    warp_arrive_leader(bar_at(p, c, B.full + slot));
     step(p.ncv);
     if (more) copy();
   }
@@ -942,10 +968,8 @@ __global__ void __launch_bounds__(slab_threads(P), 1) melt_slab_kernel(const __g
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   if (threadIdx.x == 0) {
     auto bar = [&](int i) { return bar_at(p, c, i); };
-    for (int i = 0; i < p.NS; ++i) {
-      mbar_init(bar(B.full + i), P < 3 ? 2 * p.tw : c.rank == 0 ? 4 : 1);
-      mbar_init(bar(B.empty + i), 1);
-    }
+    for (int i = 0; i < p.NS; ++i) mbar_init(bar(B.full + i), P < 3 ? 2 * p.tw : c.rank == 0 ? 4 : 1);
+    for (int i = B.empty; i < B.b_full; ++i) mbar_init(bar(i), 1);
     for (int i = 0; i < p.NB; ++i) {
       mbar_init(bar(B.b_full + i), c.rank == 0 ? 2 : 1);
       mbar_init(bar(B.b_empty + i), 1);

@@ -7,6 +7,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("prec,n_fft,hop,n_mels", [
     ("bf16x3", 256, 32, 128), ("bf16x3", 272, 32, 100),  # two slabs a tile: the shortest ring
+    # rings that are no multiple of the converter teams, with a last slice of few slabs
+    ("bf16x3", 512, 160, 80), ("bf16x3", 1024, 240, 80), ("bf16x3", 400, 160, 80), ("bf16", 1000, 480, 80),
+    ("bf16", 2048, 400, 128), ("bf16", 800, 384, 128), ("bf16", 1024, 256, 80), ("bf16x3", 404, 48, 128),
 ])
 def test_many_units(prec, n_fft, hop, n_mels):
     import torch
