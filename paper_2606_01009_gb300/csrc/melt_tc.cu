@@ -291,6 +291,7 @@ bool try_layout_pair(const TcBasis* tb, TcParams& p, const melt_plan& c, int n_m
       off += align_up(p.dct_tc ? 2 * p.dct_part : 4 * ((n_mfcc + 3) & ~3) * p.MP, 128);
       if (off + 128 > kSmemLimit) continue;
       p.NS = ns;
+      p.cvt_groups = fp8 && (n_mfcc == 0 || p.dct_tc) ? pair_cvt_groups(ns, p.NCHUNK) : 1;
       p.smem_total = off + 128;
       p.tmem_cols = fp8 || p.dct_tc ? 512 : p.NC <= 32 ? 64 : p.NC <= 64 ? 128 : p.NC <= 128 ? 256 : 512;
       p.acc_stride = p.tmem_cols / 2;
@@ -588,7 +589,8 @@ cudaError_t tc_launch(const TcBasis* tb, const TcLaunch& L, cudaStream_t stream)
   const bool fused = pair && p.Hd > 0 && L.mlp != nullptr;
   if (pair && p.Hd > 0 && !L.mlp) p.Hd = 0;  // plan made for a correction that is not passed
   KernelFn fn = fused ? kernel_for_pair_mlp(p.MP / 16)
-                : pair ? (tb->precision == MELT_FP8E4M3   ? kernel_for_pair_fp8(L.n_mfcc > 0, p.MP / 16, p.dct_tc)
+                : pair ? (tb->precision == MELT_FP8E4M3
+                              ? kernel_for_pair_fp8(L.n_mfcc > 0, p.MP / 16, p.dct_tc, p.cvt_groups)
                           : tb->precision == MELT_BF16X3 ? kernel_for_pair_x3()
                                                          : kernel_for_pair(L.n_mfcc > 0, p.MP / 16, p.dct_tc))
                        : (L.n_mfcc ? kernel_for_mfcc(tb->precision, p.MP / 16)
@@ -651,16 +653,17 @@ cudaError_t tc_launch(const TcBasis* tb, const TcLaunch& L, cudaStream_t stream)
   attr[1].val.clusterDim.x = 2;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
-  cfg.blockDim = dim3(pair_threads(fused, tb->precision, L.n_mfcc > 0, p.MP / 16, p.dct_tc), 1, 1);
+  cfg.blockDim = dim3(pair_threads(fused, tb->precision, L.n_mfcc > 0, p.MP / 16, p.dct_tc, p.cvt_groups), 1, 1);
   cfg.numAttrs = 2;
   TcBasis* mtb = const_cast<TcBasis*>(tb);
-  if (mtb->pair_clusters < 0 || mtb->pair_smem != smem) {
+  if (mtb->pair_clusters < 0 || mtb->pair_smem != smem || mtb->pair_block != (int)cfg.blockDim.x) {
     cfg.gridDim = dim3(2 * (L.sm_count / 2), 1, 1);
     int n = 0;
     cudaError_t e = cudaOccupancyMaxActiveClusters(&n, fn, &cfg);
     if (e != cudaSuccess) return e;
     mtb->pair_clusters = n;
     mtb->pair_smem = smem;
+    mtb->pair_block = (int)cfg.blockDim.x;
   }
   if (mtb->pair_clusters < 1) return cudaErrorInvalidConfiguration;
   const int clusters = std::min(p.n_pairs, mtb->pair_clusters);

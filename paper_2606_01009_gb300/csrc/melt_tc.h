@@ -30,6 +30,7 @@ struct TcBasis {
   int stft_bands = 0;      // fused STFT + Mel comparator: bands per frame (its table sits in shared memory)
   int pair_clusters = -1;  // co-resident 2-CTA clusters of the pair kernel (-1: not queried)
   int pair_smem = 0;       // shared memory size that count was queried for
+  int pair_block = 0;      // ... and threads per CTA
   // correction MLP fused in the CTA-pair kernel's epilogue (0 hidden units: none)
   int mlp_hd = 0;
   void* d_mlp_img = nullptr;  // BF16 weight image, two halves of mlp_half bytes

@@ -5,7 +5,9 @@
 namespace melt {
 namespace tc {
 
-KernelFn kernel_for_pair_fp8(bool mfcc, int nch, bool dtc) { return pick_pair_fp8_kernel<>(mfcc, nch, dtc); }
+KernelFn kernel_for_pair_fp8(bool mfcc, int nch, bool dtc, int groups) {
+  return pick_pair_fp8_kernel<>(mfcc, nch, dtc, groups);
+}
 
 }  // namespace tc
 }  // namespace melt

@@ -84,24 +84,32 @@ __host__ __device__ constexpr int part_lo(int n, int parts, int j) {
 __host__ __device__ constexpr int part_lo_tail(int n, int parts, int j) {
   return j * (n / parts) + (j > parts - n % parts ? j - (parts - n % parts) : 0);
 }
-// Converter warps: 4 (BF16: each sample converted once, short chains); 16 for
-// FP8's log-Mel kernel, whose per-row max makes each chunk one dependent chain per
-// row set (64 x 30 s: 8 warps a chunk 50.3 us; two groups of 4, 48.9; of 8, 47.4;
-// three or four of 4, 52 and 66); 8 for its MFCC kernel with the DCT on the tensor
-// cores (groups of 4: 62.7 -> 60.8), beside 8 epilogue warps.  The MFCC kernels
-// with the DCT on the CUDA cores keep 4 (their epilogue warps and registers fill
-// the block).  With
+// Converter warps: 4 (BF16: each sample converted once, short chains).  FP8's
+// per-row max makes each chunk one dependent chain per row set, so there the warps
+// form `groups` groups that take the staged chunks in turn, two chunks' chains side
+// by side: log-Mel 8 warps a group (64 x 30 s: one group 50.3 us, two 47.4; two
+// groups of 4, 48.9; three or four of 4, 52 and 66), the MFCC kernel with the DCT on
+// the tensor cores 8 warps in all, beside 8 epilogue warps (one group 62.7, two
+// 60.8).  The MFCC kernels with the DCT on the CUDA cores have one group of 4
+// (their epilogue warps and registers fill the block).  With
 // the fused MLP, 3: the warps go to the epilogue (64 x 30 s: 2 / 3 / 4 converter
 // warps 75.3 / 73.8 / 76.2 us; 8 or 16 epilogue warps 75 and more).
-__host__ __device__ constexpr int pair_cvt_warps(int prec, bool mfcc, int nch, bool dtc = false, bool mlp = false) {
-  return mlp ? kMlpCvtWarps : prec != MELT_FP8E4M3 ? 4 : !mfcc ? 16 : dtc ? 8 : 4;
+__host__ __device__ constexpr int pair_cvt_warps(int prec, bool mfcc, int nch, bool dtc = false, bool mlp = false,
+                                                 int groups = 1) {
+  return mlp ? kMlpCvtWarps : prec != MELT_FP8E4M3 ? 4 : !mfcc ? 8 * groups : dtc ? 8 : 4;
 }
-// Converter warps that share a staged chunk: half of FP8's, the halves taking
-// chunks in turn, so that two chunks' chains overlap.
-__host__ __device__ constexpr int pair_cvt_group(int prec, int cw) { return prec == MELT_FP8E4M3 && cw >= 8 ? cw / 2 : cw; }
+// Converter groups of an FP8 layout of `slots` staging slots and `chunks` chunks a
+// tile.  A group that skips a chunk does not see its copy land, copies land in any
+// order, and the parity that the group waits for tells only neighbouring turns of
+// the ring apart: so two groups only where a slot is always the same group's
+// (`slots` even), or where its chunk of the turn before is of an earlier tile
+// (`slots` at least `chunks`), whose chunks all warps have met behind.
+__host__ __device__ constexpr int pair_cvt_groups(int slots, int chunks) {
+  return slots % 2 == 0 || slots >= chunks ? 2 : 1;
+}
 __host__ __device__ constexpr int pair_threads(bool mlp, int prec = MELT_BF16, bool mfcc = false, int nch = 1,
-                                               bool dtc = false) {
-  return 32 * (pair_epi_warps(mlp, mfcc, nch, dtc) + (mlp ? 2 : 3) + pair_cvt_warps(prec, mfcc, nch, dtc, mlp));
+                                               bool dtc = false, int groups = 1) {
+  return 32 * (pair_epi_warps(mlp, mfcc, nch, dtc) + (mlp ? 2 : 3) + pair_cvt_warps(prec, mfcc, nch, dtc, mlp, groups));
 }
 constexpr int kPQuads = 8;  // float4s per converter thread per staged chunk (<= 16 KB)
 constexpr uint32_t kSfOne = 0x7F7F7F7Fu;    // four UE8M0 codes of 2^0
@@ -933,7 +941,7 @@ static __device__ __forceinline__ void fp8_convert_chunk_any(const TcParams& p, 
   }
 }
 
-template <int CW>
+template <int CW, int GROUPS>
 static __device__ void pair_convert_fp8(const TcParams& p, uint8_t* gbase, const PairCtx& c,
                                         const PairBars& B, int cvt0, uint32_t tmem_base) {
   constexpr int kThr = 32 * CW;
@@ -948,7 +956,7 @@ static __device__ void pair_convert_fp8(const TcParams& p, uint8_t* gbase, const
   for (uint32_t o = 16u * (uint32_t)(threadIdx.x - 32 * cvt0); o < p.abuf_bytes * p.ZB; o += 16u * kThr)
     sts128(c.sbase + p.off_a + o, make_uint4(0u, 0u, 0u, 0u));
   fence_proxy_async();
-  constexpr int GW = pair_cvt_group(MELT_FP8E4M3, CW);
+  constexpr int GW = CW / GROUPS;  // warps that share a chunk
   int slot = 0, turn = 0;  // whose chunk it is
   uint32_t sphase = 0;
   for (int k = 0;; ++k) {
@@ -975,7 +983,7 @@ static __device__ void pair_convert_fp8(const TcParams& p, uint8_t* gbase, const
                                   nsamp, cw % GW, g, l8);
         warp_arrive(pbar(p, c, B.s_empty + slot));
       }
-      if (++turn == CW / GW) turn = 0;
+      if (++turn == GROUPS) turn = 0;
       if (++slot == p.NS) {
         slot = 0;
         sphase ^= 1;
@@ -1473,12 +1481,12 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
 
 // The work of one CTA of a pair kernel: cluster `cluster` of `n_clusters`
 // clusters that share the tile list of `p`.
-template <int NCH, bool MFCC, bool MLP, int PREC, bool DTC, bool GRP = false>  // GRP: of a two-basis launch
+template <int NCH, bool MFCC, bool MLP, int PREC, bool DTC, int GROUPS, bool GRP = false>  // GRP: of a two-basis launch
 __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_clusters) {
   constexpr int EPW = pair_epi_warps(MLP, MFCC, NCH, DTC);
   // (fused MLP: the MMA warp is the basis producer first)
   constexpr int kPMmaWarp = EPW, kPBWarp = MLP ? EPW : EPW + 1, kPProdWarp = kPBWarp + 1, kPCvtWarp0 = kPProdWarp + 1;
-  constexpr int CW = pair_cvt_warps(PREC, MFCC, NCH, DTC, MLP);
+  constexpr int CW = pair_cvt_warps(PREC, MFCC, NCH, DTC, MLP, GROUPS);
   extern __shared__ __align__(128) uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t sbase = (raw + 127u) & ~127u;
@@ -1497,7 +1505,7 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
     auto bar = [&](int i) { return sbase + p.off_bar + 8 * i; };
     for (int i = 0; i < p.NS; ++i) {
       mbar_init(bar(B.s_full + i), 1);
-      mbar_init(bar(B.s_empty + i), pair_cvt_group(PREC, CW));
+      mbar_init(bar(B.s_empty + i), CW / GROUPS);
     }
     for (int i = 0; i < p.ZB; ++i) {
       mbar_init(bar(B.z_full + i), 2 * CW);  // converters of both CTAs (even CTA's copy is used)
@@ -1585,7 +1593,7 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
   } else if (warp >= kPCvtWarp0) {
     if (!p.early_inputs) pdl_wait();
     if constexpr (PREC == MELT_FP8E4M3)
-      pair_convert_fp8<CW>(p, gbase, c, B, kPCvtWarp0, tmem_base);
+      pair_convert_fp8<CW, GROUPS>(p, gbase, c, B, kPCvtWarp0, tmem_base);
     else
       pair_convert<PREC == MELT_BF16X3, 32 * CW>(p, c, B, kPCvtWarp0);
     __syncwarp();
@@ -1617,10 +1625,10 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
   }
 }
 
-template <int NCH, bool MFCC, bool MLP, int PREC = MELT_BF16, bool DTC = false>
-__global__ void __launch_bounds__(pair_threads(MLP, PREC, MFCC, NCH, DTC), 1)
+template <int NCH, bool MFCC, bool MLP, int PREC = MELT_BF16, bool DTC = false, int GROUPS = 1>
+__global__ void __launch_bounds__(pair_threads(MLP, PREC, MFCC, NCH, DTC, GROUPS), 1)
     melt_tc_pair_kernel(const __grid_constant__ TcParams p) {
-  pair_cta<NCH, MFCC, MLP, PREC, DTC>(p, (int)(blockIdx.x >> 1), (int)(gridDim.x >> 1));
+  pair_cta<NCH, MFCC, MLP, PREC, DTC, GROUPS>(p, (int)(blockIdx.x >> 1), (int)(gridDim.x >> 1));
 }
 
 // Two bases in one persistent launch (the grouped call): clusters
@@ -1638,8 +1646,8 @@ __global__ void __launch_bounds__(pair_threads(MLP, PREC, MFCC, NCH, DTC), 1)
     melt_tc_pair_group_kernel(const __grid_constant__ TcGroupParams q) {
   const int cl = (int)(blockIdx.x >> 1), nc = (int)(gridDim.x >> 1);
   const bool second = cl >= q.split;
-  pair_cta<NCH, MFCC, MLP, PREC, DTC, true>(second ? q.g[1] : q.g[0], second ? cl - q.split : cl,
-                                      second ? nc - q.split : q.split);
+  pair_cta<NCH, MFCC, MLP, PREC, DTC, 1, true>(second ? q.g[1] : q.g[0], second ? cl - q.split : cl,
+                                               second ? nc - q.split : q.split);
 }
 
 using GroupKernelFn = void (*)(TcGroupParams);
@@ -1668,13 +1676,18 @@ KernelFn pick_pair_kernel(int nch, bool dtc = false) {
   }
 }
 
-// FP8 e4m3 instantiations (log-Mel, and MFCC by chunk count).  The pickers are
+// FP8 e4m3 instantiations (log-Mel and MFCC with the DCT on the tensor cores, each
+// with one and two converter groups; other MFCC by chunk count).  The pickers are
 // templates so that only the translation unit that calls one instantiates
 // its kernels.
 template <int = 0>
-KernelFn pick_pair_fp8_kernel(bool mfcc, int nch, bool dtc = false) {
-  if (!mfcc) return melt_tc_pair_kernel<1, false, false, MELT_FP8E4M3>;
-  if (dtc) return melt_tc_pair_kernel<1, true, false, MELT_FP8E4M3, true>;
+KernelFn pick_pair_fp8_kernel(bool mfcc, int nch, bool dtc, int groups) {
+  if (!mfcc)
+    return groups == 2 ? melt_tc_pair_kernel<1, false, false, MELT_FP8E4M3, false, 2>
+                       : melt_tc_pair_kernel<1, false, false, MELT_FP8E4M3>;
+  if (dtc)
+    return groups == 2 ? melt_tc_pair_kernel<1, true, false, MELT_FP8E4M3, true, 2>
+                       : melt_tc_pair_kernel<1, true, false, MELT_FP8E4M3, true>;
   switch (nch) {
     case 1: return melt_tc_pair_kernel<1, true, false, MELT_FP8E4M3>;
     case 2: return melt_tc_pair_kernel<2, true, false, MELT_FP8E4M3>;

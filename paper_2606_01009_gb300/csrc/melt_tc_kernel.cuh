@@ -115,6 +115,7 @@ struct TcParams {
   uint32_t smem_total;   // dynamic shared memory bytes (incl. alignment slack)
   // CTA-pair kernel only: FP32 span staging ring and the half-basis layout
   int NS, CH, NCHUNK;    // staging slots, Z rows per chunk, chunks per tile
+  int cvt_groups;        // groups of converter warps that take the chunks in turn
   uint32_t st_bytes;     // bytes per staging slot
   uint32_t off_st;
   uint32_t b_lbo;        // B operand: bytes between the two K core columns of a K-step block
@@ -882,7 +883,7 @@ KernelFn kernel_for_pair(bool mfcc, int nch, bool dtc);
 // Defined in melt_tc2_mlp.cu: the CTA-pair kernel with the fused correction MLP.
 KernelFn kernel_for_pair_mlp(int nch);
 // Defined in melt_tc2_fp8.cu: the CTA-pair kernel with FP8 e4m3 operands.
-KernelFn kernel_for_pair_fp8(bool mfcc, int nch, bool dtc);
+KernelFn kernel_for_pair_fp8(bool mfcc, int nch, bool dtc, int groups);
 // Defined in melt_tc2_x3.cu: the CTA-pair kernel with split-BF16 operands.
 KernelFn kernel_for_pair_x3();
 
