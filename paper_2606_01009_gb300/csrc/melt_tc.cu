@@ -264,6 +264,14 @@ bool try_layout_pair(const TcBasis* tb, TcParams& p, const melt_plan& c, int n_m
     // (split BF16's two A parts, long frames)
     for (int c2 = ch / 2; c2 >= 4 && nch_c < 3; c2 /= 2) chs[nch_c++] = c2;
   }
+  // Two converter groups want four slots, two for each (with two or three slots they
+  // took 1.1 to 4.7 times one group's time; so a ring of five that would allow one
+  // group only gives up a slot: 400 / 200 / 128 60 -> 56 us).  In the log-Mel kernel
+  // their 16 warps also get in the way of the MMA and epilogue warps where these
+  // bind: with n_fft n_mels^2 / hop above 75,000 (200 geometries timed: below, two
+  // groups took 0.85 to 1.00 of one group's time, above 0.98 to 1.18; at 64 x 30 s
+  // 1000 / 96 / 128 92 us one group, 104 two).
+  const bool turns = fp8 && (n_mfcc > 0 ? p.dct_tc != 0 : (long long)p.N * p.M * p.M < 75000ll * p.H);
   p.codes_stride = fp8 ? align_up((uint32_t)p.zrows + 3, 16) : 0u;
   for (int ci = 0; ci < nch_c; ++ci) {
     const int ch = chs[ci];
@@ -271,6 +279,7 @@ bool try_layout_pair(const TcBasis* tb, TcParams& p, const melt_plan& c, int n_m
     p.NCHUNK = (p.zrows + ch - 1) / ch;
     p.st_bytes = row_bytes * ch;
     for (int ns = 8; ns >= 2; --ns) {
+      if (turns && ns > 4 && pair_cvt_groups(ns, p.NCHUNK) == 1) continue;
       const PairBars B(ns, p.ZB, p.KS, streamed ? p.NB : 0);
       uint32_t off = 0;
       p.off_a = off;
@@ -291,7 +300,7 @@ bool try_layout_pair(const TcBasis* tb, TcParams& p, const melt_plan& c, int n_m
       off += align_up(p.dct_tc ? 2 * p.dct_part : 4 * ((n_mfcc + 3) & ~3) * p.MP, 128);
       if (off + 128 > kSmemLimit) continue;
       p.NS = ns;
-      p.cvt_groups = fp8 && (n_mfcc == 0 || p.dct_tc) ? pair_cvt_groups(ns, p.NCHUNK) : 1;
+      p.cvt_groups = turns && ns >= 4 ? pair_cvt_groups(ns, p.NCHUNK) : 1;
       p.smem_total = off + 128;
       p.tmem_cols = fp8 || p.dct_tc ? 512 : p.NC <= 32 ? 64 : p.NC <= 64 ? 128 : p.NC <= 128 ? 256 : 512;
       p.acc_stride = p.tmem_cols / 2;

@@ -98,8 +98,8 @@ __host__ __device__ constexpr int pair_cvt_warps(int prec, bool mfcc, int nch, b
                                                  int groups = 1) {
   return mlp ? kMlpCvtWarps : prec != MELT_FP8E4M3 ? 4 : !mfcc ? 8 * groups : dtc ? 8 : 4;
 }
-// Converter groups of an FP8 layout of `slots` staging slots and `chunks` chunks a
-// tile.  A group that skips a chunk does not see its copy land, copies land in any
+// Converter groups that an FP8 layout of `slots` staging slots and `chunks` chunks a
+// tile can have.  A group that skips a chunk does not see its copy land, copies land in any
 // order, and the parity that the group waits for tells only neighbouring turns of
 // the ring apart: so two groups only where a slot is always the same group's
 // (`slots` even), or where its chunk of the turn before is of an earlier tile
