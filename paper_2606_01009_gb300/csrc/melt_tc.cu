@@ -601,7 +601,7 @@ cudaError_t tc_launch(const TcBasis* tb, const TcLaunch& L, cudaStream_t stream)
                 : pair ? (tb->precision == MELT_FP8E4M3
                               ? kernel_for_pair_fp8(L.n_mfcc > 0, p.MP / 16, p.dct_tc, p.cvt_groups)
                           : tb->precision == MELT_BF16X3 ? kernel_for_pair_x3()
-                                                         : kernel_for_pair(L.n_mfcc > 0, p.MP / 16, p.dct_tc))
+                                                         : kernel_for_pair(L.n_mfcc > 0, p.MP / 16, p.dct_tc, (p.H + 15) / 16))
                        : (L.n_mfcc ? kernel_for_mfcc(tb->precision, p.MP / 16)
                                    : kernel_for_plain(tb->precision, p.MP / 16, L.stft_bands > 0));
   if (!fn) return cudaErrorInvalidValue;

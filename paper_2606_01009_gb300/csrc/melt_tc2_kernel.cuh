@@ -479,33 +479,66 @@ static __device__ __forceinline__ void pair_dct_gemm(const TcParams& p, const Pa
 // reads A at a + j + kk a_step and the basis at w + (K-steps before it) w_step
 // (descriptor low words, 16-byte units).
 struct PairSteps {
-  uint32_t a, a_step, w, w_step, hi, d, idesc;
+  uint32_t a, a_step, w_step, hi, d, idesc;
   uint32_t a_lo, w_lo;  // split BF16: from a hi part to its lo part
-  uint32_t sfa, sfb;    // FP8: scale columns of A's rows and of the basis
 };
 
-// Issues n <= U K-steps of slice j from group k0 on.
+// Issues n <= U K-steps of slice j from group k0 on (BF16 forms).
 template <int PREC, int U>
 static __device__ __forceinline__ void pair_steps(const PairSteps& m, int j, int k0, int n, uint32_t w) {
   uint32_t a = m.a + (uint32_t)j + (uint32_t)k0 * m.a_step;
 #pragma unroll
   for (int k = 0; k < U; ++k) {
     if (k >= n) break;
-    const bool acc = k > 0 || j + k0 > 0;
-    if constexpr (PREC == MELT_FP8E4M3) {
-      // A row t of slice j is Z row t + j, whose scale is byte j % 4 of scale group j / 4
-      mma_f8_pair_bs(m.d, desc64(a, m.hi), desc64(w, m.hi), m.idesc | ((uint32_t)(j & 3) << 29),
-                     m.sfa + 4u * (uint32_t)(j >> 2), m.sfb, acc);
-    } else {
-      mma_f16_pair(m.d, desc64(a, m.hi), desc64(w, m.hi), m.idesc, acc);
-      if constexpr (PREC == MELT_BF16X3) {
-        // hi*lo and lo*hi, in the order of the single-CTA kernel (bit-identical sums)
-        mma_f16_pair(m.d, desc64(a, m.hi), desc64(w + m.w_lo, m.hi), m.idesc, true);
-        mma_f16_pair(m.d, desc64(a + m.a_lo, m.hi), desc64(w, m.hi), m.idesc, true);
-      }
+    mma_f16_pair(m.d, desc64(a, m.hi), desc64(w, m.hi), m.idesc, k > 0 || j + k0 > 0);
+    if constexpr (PREC == MELT_BF16X3) {
+      // hi*lo and lo*hi, in the order of the single-CTA kernel (bit-identical sums)
+      mma_f16_pair(m.d, desc64(a, m.hi), desc64(w + m.w_lo, m.hi), m.idesc, true);
+      mma_f16_pair(m.d, desc64(a + m.a_lo, m.hi), desc64(w, m.hi), m.idesc, true);
     }
     a += m.a_step;
     w += m.w_step;
+  }
+}
+
+// All K-steps of a tile in BF16 or FP8, as a function of its own: with the loops
+// inline a slice costs some 150 clocks beside its MMAs, and layouts whose slices
+// are one or two K-steps long took up to twice what a lookup of each K-step in
+// shared memory had (one clip of 1.25 M frames at 1024 / 16 / 40: table 235 us,
+// inline 464).
+constexpr int kStraight = 3;    // K-steps of a slice at most that are issued as straight-line code
+constexpr int kShortSlice = 6;  // K-steps of a slice up to which the BF16 log-Mel kernel, too, is the one that calls it
+template <int PREC>
+static __device__ __noinline__ void pair_walk(uint32_t a, uint32_t a_step, uint32_t w, uint32_t w_step, uint32_t hi,
+                                              uint32_t d, uint32_t idesc, uint32_t sfa, uint32_t sfb, int J, int nk,
+                                              int nk_last) {
+  uint32_t acc = 0;
+  const auto step = [&](uint32_t x, int j) {
+    if constexpr (PREC == MELT_FP8E4M3)
+      // A row t of slice j is Z row t + j, whose scale is byte j % 4 of scale group j / 4
+      mma_f8_pair_bs(d, desc64(x, hi), desc64(w, hi), idesc | ((uint32_t)(j & 3) << 29), sfa + 4u * (uint32_t)(j >> 2),
+                     sfb, acc != 0);
+    else
+      mma_f16_pair(d, desc64(x, hi), desc64(w, hi), idesc, acc != 0);
+    acc = 1;
+    w += w_step;
+  };
+  if (nk <= kStraight) {
+#pragma unroll 4
+    for (int j = 0; j < J; ++j) {
+      const int n = j + 1 < J ? nk : nk_last;
+#pragma unroll
+      for (int k = 0; k < kStraight; ++k)
+        if (k < n) step(a + (uint32_t)j + (uint32_t)k * a_step, j);
+    }
+    return;
+  }
+#pragma unroll 1
+  for (int j = 0; j < J; ++j) {
+    const int n = j + 1 < J ? nk : nk_last;
+    uint32_t x = a + (uint32_t)j;
+#pragma unroll 5
+    for (int k = 0; k < n; ++k, x += a_step) step(x, j);
   }
 }
 
@@ -517,11 +550,11 @@ static __device__ __forceinline__ void pair_steps(const PairSteps& m, int j, int
 // 4096 mixed clips 711 -> 692.)  The waits acquire at CTA scope, 100 clocks for
 // 250 at cluster scope: what the peer wrote is read by the MMAs only, through the
 // async proxy, after its writers' proxy fences.
-template <bool MLP, int PREC, bool DTC, bool GRP>
+// INLINE: the BF16 log-Mel kernel of longer slices, whose samples' bytes in flight
+// bind it, walks them inline (a call a tile took 0.3 to 0.5 % longer there).
+template <bool MLP, int PREC, bool DTC, bool GRP, bool INLINE>
 static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairBars& B, uint32_t tmem_base) {
-  // K-steps issued in a run.  Longer ones pay only where the DCT's MMAs wait behind
-  // them (MFCC 43.6 us with 5, 44.3 with 1; log-Mel 38.5 and 38.2).
-  constexpr int kU = DTC ? 5 : 1;
+  constexpr int kU = 1;  // K-steps issued in a run of the inline walk (64 x 30 s: runs of 5 38.5 us, of 1 38.2)
   constexpr int kstep = PREC == MELT_FP8E4M3 ? 32 : 16;
   const int nacc = MLP ? 1 : p.nacc;  // the fused MLP's TMEM leaves room for one accumulator
   const int J = p.J, nk = (p.H + kstep - 1) / kstep, nk_last = (p.N - (p.J - 1) * p.H + kstep - 1) / kstep;
@@ -535,7 +568,7 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
   m.idesc = p.idesc;
   m.a_lo = p.a_bytes >> 4;  // the lo part of an A buffer, or of a K-step's basis block, follows its hi part
   m.w_lo = (p.step_bytes / 2) >> 4;
-  m.sfb = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * p.ZB);  // FP8: basis scale 2^-8
+  const uint32_t sfb = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * p.ZB);  // FP8: basis scale 2^-8
   const auto wait = [&](int bar, int phase) {
     return __all_sync(0xffffffffu, mbar_wait(pbar(p, c, bar), (uint32_t)phase & 1u, c.abort, p.err, kErrTimeout)) != 0;
   };
@@ -569,15 +602,13 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
     tc_fence_after();
     m.d = tmem_base + acc * p.acc_stride;
     m.a = a0 + zb * (p.abuf_bytes >> 4);
-    m.sfa = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * zb);
-    m.w = b0;
+    const uint32_t sfa = tmem_base + p.sf_col + (uint32_t)(4 * p.sfg * zb);
     if (PREC != MELT_FP8E4M3 && !MLP && !DTC && !p.b_resident) {  // (planned for these only)
       // streamed half basis: slot by slot, each once both CTAs' halves are in.  One
-      // election for a slot where streaming is what the kernel is for (two bases' 4096
-      // clips in one launch 1074 us for 1146; split BF16 at N = 640, hop 64, 64 x 20 s
-      // 134 for 170); one a K-step in the BF16 log-Mel kernel, whose resident loop is
-      // 0.8 % slower beside any other form of this one (38.4 for 38.05 us)
-      constexpr bool kSlotRuns = GRP || PREC == MELT_BF16X3;
+      // election for a slot (two bases' 4096 clips in one launch 1074 us for 1146;
+      // split BF16 at N = 640, hop 64, 64 x 20 s 134 for 170), but one a K-step beside
+      // the inline walk, which is 0.8 % slower beside any other form of this loop (38.4
+      // for 38.05 us)
       int j = 0, k0 = 0;
       for (int s0 = 0; s0 < p.KS; s0 += p.kps, ++g) {
         const int slot = g % p.NB;
@@ -587,7 +618,7 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
         }
         tc_fence_after();
         uint32_t w = b0 + (uint32_t)slot * (p.bslot_bytes >> 4);
-        if constexpr (kSlotRuns) {
+        if constexpr (!INLINE) {
           for (int left = min(p.kps, p.KS - s0); left > 0;) {  // (a slot may run on into the next slice)
             const int nj = j + 1 < J ? nk : nk_last, n = min(left, nj - k0);
             if (elect_one()) {
@@ -622,14 +653,18 @@ static __device__ void pair_mma(const TcParams& p, const PairCtx& c, const PairB
       }
       if (!ok) break;
     } else if (elect_one()) {
-      uint32_t w = b0;
-      for (int j = 0; j < J; ++j) {
-        const int nj = j + 1 < J ? nk : nk_last;
-        for (int k0 = 0; k0 < nj; k0 += kU) {
-          const int n = min(kU, nj - k0);
-          pair_steps<PREC, kU>(m, j, k0, n, w);
-          w += (uint32_t)n * m.w_step;
+      if constexpr (INLINE) {
+        uint32_t w = b0;
+        for (int j = 0; j < J; ++j) {
+          const int nj = j + 1 < J ? nk : nk_last;
+          for (int k0 = 0; k0 < nj; k0 += kU) {
+            const int n = min(kU, nj - k0);
+            pair_steps<PREC, kU>(m, j, k0, n, w);
+            w += (uint32_t)n * m.w_step;
+          }
         }
+      } else {
+        pair_walk<PREC>(m.a, m.a_step, b0, m.w_step, m.hi, m.d, m.idesc, sfa, sfb, J, nk, nk_last);
       }
     }
     __syncwarp();
@@ -1489,7 +1524,8 @@ __device__ void pair_epilogue_mlp(const TcParams& p, uint8_t* gbase, const PairC
 
 // The work of one CTA of a pair kernel: cluster `cluster` of `n_clusters`
 // clusters that share the tile list of `p`.
-template <int NCH, bool MFCC, bool MLP, int PREC, bool DTC, int GROUPS, bool GRP = false>  // GRP: of a two-basis launch
+template <int NCH, bool MFCC, bool MLP, int PREC, bool DTC, int GROUPS, bool SHORT,
+          bool GRP = false>  // SHORT: slices of at most kShortSlice K-steps (BF16 log-Mel); GRP: of a two-basis launch
 __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_clusters) {
   constexpr int EPW = pair_epi_warps(MLP, MFCC, NCH, DTC);
   // (fused MLP: the MMA warp is the basis producer first)
@@ -1587,7 +1623,8 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
   if (warp == kPMmaWarp) {
     if (MLP && lane == 0) pair_basis_producer(p, c, B);
     __syncwarp();
-    if (c.rank == 0) pair_mma<MLP, PREC, DTC, GRP>(p, c, B, __shfl_sync(0xffffffffu, tmem_base, 0));
+    constexpr bool kInline = PREC == MELT_BF16 && !MFCC && !MLP && !SHORT && !GRP;
+    if (c.rank == 0) pair_mma<MLP, PREC, DTC, GRP, kInline>(p, c, B, __shfl_sync(0xffffffffu, tmem_base, 0));
     else if (lane == 0 && !p.b_resident) pair_basis_signal(p, c, B);  // the odd CTA's slots, to the even CTA
     if (lane == 0) drain_wait(pbar(p, c, B.drain), 0, p.err);
     __syncwarp();
@@ -1633,10 +1670,10 @@ __device__ __forceinline__ void pair_cta(const TcParams& p, int cluster, int n_c
   }
 }
 
-template <int NCH, bool MFCC, bool MLP, int PREC = MELT_BF16, bool DTC = false, int GROUPS = 1>
+template <int NCH, bool MFCC, bool MLP, int PREC = MELT_BF16, bool DTC = false, int GROUPS = 1, bool SHORT = false>
 __global__ void __launch_bounds__(pair_threads(MLP, PREC, MFCC, NCH, DTC, GROUPS), 1)
     melt_tc_pair_kernel(const __grid_constant__ TcParams p) {
-  pair_cta<NCH, MFCC, MLP, PREC, DTC, GROUPS>(p, (int)(blockIdx.x >> 1), (int)(gridDim.x >> 1));
+  pair_cta<NCH, MFCC, MLP, PREC, DTC, GROUPS, SHORT>(p, (int)(blockIdx.x >> 1), (int)(gridDim.x >> 1));
 }
 
 // Two bases in one persistent launch (the grouped call): clusters
@@ -1654,7 +1691,7 @@ __global__ void __launch_bounds__(pair_threads(MLP, PREC, MFCC, NCH, DTC), 1)
     melt_tc_pair_group_kernel(const __grid_constant__ TcGroupParams q) {
   const int cl = (int)(blockIdx.x >> 1), nc = (int)(gridDim.x >> 1);
   const bool second = cl >= q.split;
-  pair_cta<NCH, MFCC, MLP, PREC, DTC, 1, true>(second ? q.g[1] : q.g[0], second ? cl - q.split : cl,
+  pair_cta<NCH, MFCC, MLP, PREC, DTC, 1, false, true>(second ? q.g[1] : q.g[0], second ? cl - q.split : cl,
                                                second ? nc - q.split : q.split);
 }
 
@@ -1663,12 +1700,14 @@ using GroupKernelFn = void (*)(TcGroupParams);
 GroupKernelFn kernel_for_pair_group();
 
 template <bool MFCC>
-KernelFn pick_pair_kernel(int nch, bool dtc = false) {
+KernelFn pick_pair_kernel(int nch, bool dtc, int nk) {
   if constexpr (!MFCC) {
     (void)nch;
     (void)dtc;
-    return melt_tc_pair_kernel<1, false, false>;
+    return nk <= kShortSlice ? melt_tc_pair_kernel<1, false, false, MELT_BF16, false, 1, true>
+                             : melt_tc_pair_kernel<1, false, false>;
   } else {
+    (void)nk;
     if (dtc) return melt_tc_pair_kernel<1, true, false, MELT_BF16, true>;
     switch (nch) {
       case 1: return melt_tc_pair_kernel<1, true, false>;

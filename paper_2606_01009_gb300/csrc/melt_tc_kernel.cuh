@@ -878,8 +878,8 @@ KernelFn pick_kernel(int nch) {
 // Defined in melt_tc_plain.cu (log-Mel) and melt_tc_mfcc.cu (MFCC epilogue).
 KernelFn kernel_for_plain(int prec, int nch, bool stft = false);
 KernelFn kernel_for_mfcc(int prec, int nch);
-// Defined in melt_tc2.cu: the CTA-pair kernel (BF16).
-KernelFn kernel_for_pair(bool mfcc, int nch, bool dtc);
+// Defined in melt_tc2.cu: the CTA-pair kernel (BF16); nk: K-steps of a whole slice.
+KernelFn kernel_for_pair(bool mfcc, int nch, bool dtc, int nk);
 // Defined in melt_tc2_mlp.cu: the CTA-pair kernel with the fused correction MLP.
 KernelFn kernel_for_pair_mlp(int nch);
 // Defined in melt_tc2_fp8.cu: the CTA-pair kernel with FP8 e4m3 operands.

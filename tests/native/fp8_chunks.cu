@@ -20,7 +20,7 @@ cudaError_t slab_launch(SlabBasis*, const SlabLaunch&, cudaStream_t) { return cu
 namespace tc {
 KernelFn kernel_for_plain(int, int, bool) { return nullptr; }
 KernelFn kernel_for_mfcc(int, int) { return nullptr; }
-KernelFn kernel_for_pair(bool, int, bool) { return nullptr; }
+KernelFn kernel_for_pair(bool, int, bool, int) { return nullptr; }
 KernelFn kernel_for_pair_mlp(int) { return nullptr; }
 KernelFn kernel_for_pair_fp8(bool, int, bool, int) { return nullptr; }
 KernelFn kernel_for_pair_x3() { return nullptr; }
