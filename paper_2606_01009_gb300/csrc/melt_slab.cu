@@ -42,7 +42,9 @@ uint32_t mfcc_bytes(const SlabParams& p, int n_mfcc) {
 // Geometry and shared-memory plan.  P 3: false where two stages do not fit (three
 // or more do for every basis that can be created).  P 1, 2: false where a tile
 // has more rows than a converter copies at once, or its slabs and a few more do
-// not fit beside the basis ring.
+// not fit beside the basis ring; P 1 also where hops above 416 leave two teams,
+// which are slower than the single-CTA layouts (64 x 7.8 s, 41 geometries: 1.13
+// times their time; at 944 / 656 / 64 27.6 us for 21.2; three teams 0.92 times).
 bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
   const int P = sb->parts;
   p.N = sb->n_fft;
@@ -94,7 +96,7 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
         if (end || left(0, least_nb) < (int)(least_nb * basis)) continue;
         int na = std::min({(left(0, least_nb) - (int)(least_nb * basis)) / (int)p.stage, 2 * p.n_slab, kMaxA});
         if (left(na, least_nb) < (int)(least_nb * basis)) --na;  // (its own barriers)
-        if (teams > na || na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
+        if (teams > na || (P == 1 && teams == 2 && p.n_slab > 26) || na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
         p.NS = na;
         p.NB = std::max(least_nb, std::min(kMaxB, left(na, kMaxB) / (int)basis));
         p.ncv = teams;
