@@ -347,13 +347,25 @@ int candidate_list(const TcBasis* tb, const TcParams& p, melt_plan* out, int cap
     // (its converter is the polyphase one with a per-row scale).  The static
     // schedule is the default: the dynamic one measured no gain (42.6 against
     // 42.4 us).
+    // Two A buffers first, but where they leave room only for staging chunks of
+    // fewer than 12 rows, one: a chunk's copy and hand-over then cost more than the
+    // overlap gives (64 x 30 s, 90 such layouts: one buffer 0.3 to 1.0 of their time,
+    // four MMA-bound ones up to 1.2; 400 / 320 / 64, 64 x 7.8 s, 36 us for 24; FP8
+    // 1000 / 240 / 128 with 40 MFCCs 207 for 92).
+    melt_plan small;
+    bool have_small = false;
     for (int zb = 2; zb >= 1; --zb) {
       melt_plan pc{1, zb, 0, p.KS, 1, 1, kDefaultSchedule};
       TcParams q = p;
       if (n < cap && try_layout_pair(tb, q, pc, tb->n_mfcc) && q.NS >= 2) {
         const bool bf16_logmel = tb->precision == MELT_BF16 && tb->n_mfcc == 0;
         if ((q.NS < 4 || bf16_logmel) && !tb->mlp_hd) pc.prefetch_tiles = kDefaultSchedule ? 0 : 1;
-        out[n++] = pc;
+        if (zb == 2 && q.CH < 12) {
+          small = pc;
+          have_small = true;
+        } else {
+          out[n++] = pc;
+        }
         // the other pair schedule, for melt_autotune (after every default layout)
         melt_plan alt = pc;
         alt.schedule = 1 - kDefaultSchedule;
@@ -361,6 +373,7 @@ int candidate_list(const TcBasis* tb, const TcParams& p, melt_plan* out, int cap
         if (n_alt < 2) alts[n_alt++] = alt;
       }
     }
+    if (have_small && n < cap) out[n++] = small;
   }
   if (tb->precision == MELT_FP8E4M3) {  // no single-CTA FP8 layouts
     for (int i = 0; i < n_alt && n < cap; ++i) out[n++] = alts[i];
