@@ -194,11 +194,12 @@ melt_status melt_autotune(melt_basis* basis, const float* wave, const int64_t* o
  *   The file at `path` (text, one line per tuned configuration, created if
  *   missing) is read first.  A line for this GPU (by name), this basis
  *   configuration (n_fft, hop, frequency count, precision, n_mfcc, fused
- *   correction's hidden units, comparator bands) and this batch size class
- *   (log2 of the batch's tile count) that still fits the device sets its plan
- *   without timing (*hit = 1).  Otherwise melt_autotune runs (arguments as
- *   there) and its plan is appended as one line (*hit = 0).  The plan in
- *   effect is returned in *best.  `best` and `hit` may be NULL.
+ *   correction's hidden units, comparator bands; whether the slab kernel of
+ *   melt_plan's cta_pair serves it, so that lines tuned without that kernel do
+ *   not count) and this batch size class (log2 of the batch's tile count) that
+ *   still fits the device sets its plan without timing (*hit = 1).  Otherwise
+ *   melt_autotune runs (arguments as there) and its plan is appended as one
+ *   line (*hit = 0).  The plan in effect is returned in *best.  `best` and `hit` may be NULL.
  *   Errors: those of melt_autotune; MELT_ERR_ARG for a NULL path;
  *   MELT_ERR_CUDA if the device name cannot be read.  A file that cannot be
  *   written only skips the append.

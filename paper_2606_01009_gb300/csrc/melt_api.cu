@@ -488,9 +488,11 @@ bool device_token(int device, char* buf, size_t n) {
   return true;
 }
 
+// (The mark of bases that the slab kernel serves keeps lines that were written
+// before it existed, and hold single-CTA layouts, from being taken for theirs.)
 void basis_plan_key(const melt_basis* b, char* buf, size_t n) {
-  std::snprintf(buf, n, "%d %d %d %d %d %d %d", b->n_fft, b->hop, b->n_mels, b->precision, b->n_mfcc,
-                b->correction ? mlp_hidden(b->correction) : 0, b->stft_bands);
+  std::snprintf(buf, n, "%d %d %d %d %d %d %d%s", b->n_fft, b->hop, b->n_mels, b->precision, b->n_mfcc,
+                b->correction ? mlp_hidden(b->correction) : 0, b->stft_bands, b->tc.slab ? " slab" : "");
 }
 
 int tile_class(long long tiles) {
