@@ -505,7 +505,8 @@ static __device__ __forceinline__ void pair_steps(const PairSteps& m, int j, int
 // inline a slice costs some 150 clocks beside its MMAs, and layouts whose slices
 // are one or two K-steps long took up to twice what a lookup of each K-step in
 // shared memory had (one clip of 1.25 M frames at 1024 / 16 / 40: table 235 us,
-// inline 464).
+// inline 464; 400,000 frames: table 84, here 48, and 75 without the form for slices
+// of one K-step).
 constexpr int kStraight = 3;    // K-steps of a slice at most that are issued as straight-line code
 constexpr int kShortSlice = 6;  // K-steps of a slice up to which the BF16 log-Mel kernel, too, is the one that calls it
 template <int PREC>
@@ -523,6 +524,11 @@ static __device__ __noinline__ void pair_walk(uint32_t a, uint32_t a_step, uint3
     acc = 1;
     w += w_step;
   };
+  if (nk == 1) {
+#pragma unroll 8
+    for (int j = 0; j < J; ++j) step(a + (uint32_t)j, j);
+    return;
+  }
   if (nk <= kStraight) {
 #pragma unroll 4
     for (int j = 0; j < J; ++j) {
