@@ -11,7 +11,9 @@ the stream, so each launch stages samples while the previous one drains).
   e2e       frames/s through the public Python API with pinned HOST buffers:
             H2D of the step's waveforms, the forward, D2H of its features
   roofline  dominant kernel vs the measured HBM copy bandwidth
-            (bound "hbm" for the tensor-core forms, "alu" for FP32 SIMT)
+            (bound "hbm"; FP32, six BF16 products on the tensor cores, against
+            their peak in "forms" and as tensor_frac_of_bf16_peak, and against the
+            FFMA peak of CUDA cores, which it exceeds, as "alu")
   cpu_baseline  the FP64 oracle on the host cores on a bounded sample
 
 Inputs larger than L2: the step's inputs and outputs rotate over several
@@ -399,9 +401,13 @@ def time_form(args, W, precision, steps, warmup, world, want_e2e):
     return res
 
 
+FP32_PRODUCTS = 6  # BF16 products of the FP32 form's three-part split operands
+
+
 def roofline(cfg, W, r, peaks, peak_kind):
     prec, T, n_out = r["precision"], r["T"], r["n_out"]
     flops = 2 * cfg["n_fft"] * 2 * cfg["n_mels"] * T * (3 if prec == "bf16x3" else 1)
+    bf16_peak = peaks.get("bf16_tflops", 1900.0)
     alg_bytes = algorithmic_bytes(W.lens, cfg["n_fft"], cfg["hop"], n_out)
     sec = r["launch_ms"] / 1e3
     if prec == "fp32":
@@ -409,7 +415,9 @@ def roofline(cfg, W, r, peaks, peak_kind):
         ach = flops / sec / 1e12
         return {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
                 "traffic": None, "peak_note": "FP32 FFMA peak derived: 152 SMs x 128 lanes x 2 FLOP x "
-                f"{peaks.get('sm_max_mhz', 2070.0):.0f} MHz max SM clock",
+                f"{peaks.get('sm_max_mhz', 2070.0):.0f} MHz max SM clock; the form runs {FP32_PRODUCTS} BF16 products "
+                "on the tensor cores instead (tensor_tflops)",
+                "tensor_tflops": FP32_PRODUCTS * ach, "tensor_frac_of_bf16_peak": FP32_PRODUCTS * ach / bf16_peak,
                 "algorithmic_flops_per_launch": flops, "launch_ms": r["launch_ms"]}
     ach = alg_bytes / sec / 1e9
     peak = peaks["hbm_gbs"]
@@ -418,7 +426,7 @@ def roofline(cfg, W, r, peaks, peak_kind):
            "traffic": measured_traffic(key), "traffic_key": key, "peak_note": f"hbm_gbs of {peak_kind} peaks (copy bandwidth)",
            "algorithmic_bytes_per_launch": alg_bytes, "launch_ms": r["launch_ms"],
            "tensor_tflops": flops / sec / 1e12}
-    out["tensor_frac_of_bf16_peak"] = out["tensor_tflops"] / peaks.get("bf16_tflops", 1900.0)
+    out["tensor_frac_of_bf16_peak"] = out["tensor_tflops"] / bf16_peak
     return out
 
 
@@ -503,6 +511,8 @@ def run_melt(args, rank, world):
                 res["forms"][name] = r
                 continue
             rf = roofline(cfg, W, r, peaks, peak_kind)
+            if rf["bound"] == "alu":
+                rf.update(bound="tensor", frac=rf["tensor_frac_of_bf16_peak"], achieved=rf["tensor_tflops"])
             res["forms"][name] = {"value": r["value"], "ms_per_step": r["ms_per_step"], "steps": r["steps"],
                                   "trials": r["trials"],
                                   "roofline_frac": rf["frac"], "bound": rf["bound"],
@@ -865,9 +875,9 @@ def frontend_leg(melt, dev, clips, cfg, precision, n_mfcc=0, steps=10, peaks=Non
            "frames_per_s": T / (ms / 1e3), "hbm_gbs": alg / (ms / 1e3) / 1e9}
     if peaks:
         if precision == "fp32":
-            flops = 2 * cfg["n_fft"] * 2 * cfg["n_mels"] * T
-            peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6
-            res["roofline_frac"], res["bound"] = flops / (ms / 1e3) / peak, "alu"
+            flops = FP32_PRODUCTS * 2 * cfg["n_fft"] * 2 * cfg["n_mels"] * T
+            res["roofline_frac"] = flops / (ms / 1e3) / (peaks.get("bf16_tflops", 1900.0) * 1e12)
+            res["bound"] = "tensor"
         else:
             res["roofline_frac"], res["bound"] = res["hbm_gbs"] / peaks["hbm_gbs"], "hbm"
     if oracle_clips:
