@@ -227,10 +227,12 @@ int64_t frames_of(const melt_basis* b, int64_t len) {
   return (len - b->n_fft) / b->hop + 1;
 }
 
-// The CUDA-core kernel's CTAs take tiles in list order, round by round, and a
-// tile costs it in proportion to its frames (warps past the tile's end
-// idle); with the longest tiles first, the last, partly filled round holds
-// the short tiles that end clips.  Tiles are independent (each writes its
+// The slab kernel takes tiles two by two in list order; with the longest tiles
+// first, the short tiles that end clips share pairs, and the last, partly filled
+// round has the pairs with the fewest samples to convert and rows to store (FP32,
+// 64 x 30 s 95.6 -> 94.7 us, 2000 clips of 0.3 to 3 s 144.3 -> 143.1; the
+// CUDA-core kernel's CTAs take them one by one, and a tile costs it in proportion
+// to its frames).  Tiles are independent (each writes its
 // own rows), so the order changes no result.
 void order_longest_first(TileDesc* t, long long n) {
   std::stable_sort(t, t + n, [](const TileDesc& a, const TileDesc& b) { return a.n_frames > b.n_frames; });

@@ -29,7 +29,7 @@ static_assert(sizeof(TileDesc) == 32, "TileDesc is 32 bytes");
 // Error bits latched by kernels in the per-basis device error word.
 enum : int { kErrTimeout = 1, kErrBadTile = 2 };
 
-// Parameters of the FP32 SIMT kernel (raw R | I projections).
+// Parameters of the CUDA-core kernel (raw FP32 R | I projections, melt_forward_components).
 struct SimtParams {
   const float* wave;
   const TileDesc* tiles;
@@ -53,7 +53,7 @@ inline cudaError_t host_alloc_pinned(T** p, size_t bytes) {
   return host_alloc_pinned_bytes(reinterpret_cast<void**>(p), bytes);
 }
 
-// Launch the FP32 SIMT kernel for `p` (grid picked by the caller).
+// Launch the CUDA-core kernel for `p`.
 // Persistent launch: as many CTAs as fit on sm_count SMs (at most one per tile).
 cudaError_t launch_simt(const SimtParams& p, int mj, int sm_count, cudaStream_t stream);
 

@@ -85,8 +85,8 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
     p.stage = p.a_bytes;
     p.b_slot = basis;
     // As many converter teams and slabs beside the tile in use (up to another
-    // tile of them) as leave three basis slots; then more of those.  Measured,
-    // split BF16 256 x 10 s: 6 / 4 / 3 teams 76 / 77 / 81 us with 5 slabs, 2 / 8
+    // tile of them) as leave three basis slots; then more of those.  Measured in
+    // one process on a fixed input, split BF16 256 x 10 s: 6 / 4 / 3 teams 76 / 77 / 81 us with 5 slabs, 2 / 8
     // slabs (fewer teams) 82 / 78; BF16 at 22.05 kHz, 64 x 20 s: 10 / 7 / 4 slabs
     // 42.4 / 43.8 / 45.2.  (Never more teams than slots: see SlabParams::ncv.)
     for (int least_nb = 3; least_nb >= 2; --least_nb)
@@ -96,7 +96,8 @@ bool plan(const SlabBasis* sb, int n_mfcc, SlabParams& p) {
         if (end || left(0, least_nb) < (int)(least_nb * basis)) continue;
         int na = std::min({(left(0, least_nb) - (int)(least_nb * basis)) / (int)p.stage, 2 * p.n_slab, kMaxA});
         if (left(na, least_nb) < (int)(least_nb * basis)) --na;  // (its own barriers)
-        if (teams > na || (P == 1 && teams == 2 && p.n_slab > 26) || na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
+        if (teams > na || (P == 1 && teams == 2 && p.n_slab > 26)) continue;
+        if (na < p.n_slab + std::max(2, least_nb == 3 ? p.n_slab / 3 : 2)) continue;
         p.NS = na;
         p.NB = std::max(least_nb, std::min(kMaxB, left(na, kMaxB) / (int)basis));
         p.ncv = teams;

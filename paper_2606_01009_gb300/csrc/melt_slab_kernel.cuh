@@ -1,8 +1,10 @@
 // Device side of the slab kernel, included by melt_slab.cu.
 #pragma once
-// The FP32 form of the projection (Eq. 6) on the tensor cores.
+// The projection (Eq. 6) on the tensor cores with both operands streamed in K
+// slabs: the FP32 form (P 3), and log-Mel of split BF16 (P 2) and of BF16 bases
+// that do not stay resident (P 1).
 //
-// Every FP32 sample and every basis value is split exactly into three BF16
+// FP32.  Every FP32 sample and every basis value is split exactly into three BF16
 // parts (hi = rn(v), mid = rn(v - hi), lo = rn(v - hi - mid): 3 x 8 bits), and
 // the six products of parts whose weight is at least 2^-16 of the leading one
 // are formed: hi hi, hi mid, mid hi, mid mid, hi lo, lo hi.  What is dropped
@@ -19,7 +21,7 @@
 // larger: not kept.)
 //
 // Bound.  Six products make 6 x 128,000 flops a frame at (N, M) = (400, 80):
-// 147 TFLOP for the 64 x 30 s batch, tensor-bound (its 184 MB of samples and
+// 147 GFLOP for the 64 x 30 s batch, tensor-bound (its 184 MB of samples and
 // features take a third of that time).  So everything else has to stay out of
 // the MMAs' way: the basis (384 KB in three parts) does not fit shared memory
 // and neither do two converted tiles (125 KB each), but one K slab of both
@@ -273,7 +275,9 @@ static __device__ __forceinline__ int slab_steps(const SlabParams& p, int kk) {
 // ---- basis producer: each unit's K-steps of this CTA's half, stage by stage
 // (A bulk prefetch of the next tile's samples into L2 from here, a unit ahead of the
 // converters, cost more than it gave: 64 x 30 s FP32 91.6 us with, 90.2 without; 256
-// x 10 s split BF16 76.2, 73.5; BF16 at 22.05 kHz, 64 x 20 s 42.1, 40.8.)
+// x 10 s split BF16 76.2, 73.5; BF16 at 22.05 kHz, 64 x 20 s 42.1, 40.8, all in one
+// process on a fixed input; over changing inputs the calls take 95 to 98, 77 to 80 and
+// 43.)
 template <int P>
 static __device__ void basis_producer(const SlabParams& p, const Ctx& c, const SlabBars& B) {
   const uint64_t pol = policy_evict_last();
@@ -595,7 +599,7 @@ static __device__ __forceinline__ void copy_quad(uint32_t dst, const float* src,
 static __device__ __forceinline__ void stage_rows(const SlabParams& p, const float* src, int nsamp, int rows, bool live,
                                                   int s0, uint32_t to, int u0, int tw) {
   int s = s0 + u0 * p.H;
-  if (s0 + rows * p.H <= nsamp && p.H % 16 == 0) {  // (the same for all lanes) no sample past the clip's end
+  if (s0 + rows * p.H <= nsamp && p.H % 16 == 0) {  // no sample of this lane's past the clip's end
     const float* from = src + s;
 #pragma unroll 4
     for (int u = u0; u < rows; u += 8 * tw, from += 8 * tw * p.H, to += 512 * tw) copy_quad(to, from, 16);

@@ -386,7 +386,10 @@ int candidate_list(const TcBasis* tb, const TcParams& p, melt_plan* out, int cap
   // N = 1200, 128 bins, 16 x 30 s 29 against 33 us).  The pair kernel's own
   // streamed layout measured no faster than the single-CTA ones (64 x 30 s split
   // BF16: 86.6 against 83.4 us), so elsewhere they come after those, for
-  // melt_autotune.
+  // melt_autotune.  (Split BF16 above 80 bins runs as two blocks, each converting the
+  // samples: over 215 geometries 160,000 samples take 0.4 to 0.9 of the single-CTA
+  // layouts' time, 0.61 in the mean, 32 million 0.7 to 1.55, 1.03 in the mean;
+  // melt_autotune tells.)
   auto streamed_pairs = [&] {
     if ((tb->precision != MELT_BF16 && tb->precision != MELT_BF16X3) || !tb->d_b2 || tb->n_mfcc != 0 || tb->mlp_hd)
       return;

@@ -1,5 +1,5 @@
-// Device side of the CTA-pair tensor-core MelT kernel (BF16), included by
-// melt_tc2.cu.
+// Device side of the CTA-pair tensor-core MelT kernel (BF16, split BF16, FP8),
+// included by its instantiation units melt_tc2*.cu and by melt_tc.cu.
 #pragma once
 // The pair kernel (BF16 and FP8 e4m3) runs as clusters of two CTAs on
 // neighbouring SMs.  The even
