@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <utility>
 #include <vector>
 
@@ -132,6 +133,8 @@ melt_status slab_build(SlabBasis* sb, int n_fft, int hop, int n_mels, int n_mfcc
   SlabParams p;
   std::memset(&p, 0, sizeof(p));
   if (!plan(sb, n_mfcc, p)) return MELT_ERR_UNSUPPORTED;
+  sb->layout = new (std::nothrow) SlabParams(p);
+  if (!sb->layout) return MELT_ERR_OOM;
   const size_t half = (size_t)sb->ksteps * p.step_bytes;
   std::vector<uint16_t> img(half);  // two halves of half / 2 values each
   // K-steps slab by slab over the slices (P 3), or slice by slice over the slabs
@@ -166,12 +169,13 @@ melt_status slab_build(SlabBasis* sb, int n_fft, int hop, int n_mels, int n_mfcc
 void slab_free(SlabBasis* sb) {
   cudaFree(sb->d_img);
   sb->d_img = nullptr;
+  delete sb->layout;
+  sb->layout = nullptr;
 }
 
 cudaError_t slab_launch(SlabBasis* sb, const SlabLaunch& L, cudaStream_t stream) {
-  SlabParams p;
-  std::memset(&p, 0, sizeof(p));
-  if (!sb->d_img || !plan(sb, L.n_mfcc, p)) return cudaErrorInvalidConfiguration;
+  if (!sb->d_img || !sb->layout) return cudaErrorInvalidConfiguration;
+  SlabParams p = *sb->layout;
   p.wave = L.wave;
   p.tiles = L.tiles;
   p.img = static_cast<const uint8_t*>(sb->d_img);

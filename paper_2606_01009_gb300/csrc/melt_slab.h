@@ -6,6 +6,10 @@
 
 namespace melt {
 
+namespace slab {
+struct SlabParams;
+}
+
 // Device-resident operands of one basis for the slab kernel.
 struct SlabBasis {
   int parts = 0;                       // BF16 parts per operand: 3 for the FP32 form, 2 for split BF16, 1 for BF16
@@ -13,6 +17,7 @@ struct SlabBasis {
   int J = 0, n_slab = 0, ksteps = 0;   // polyphase slices, 16-sample slabs, MMA K-steps
   int groups = 0;                      // groups of 8 Mel bins
   void* d_img = nullptr;               // two halves (W_r rows, W_i rows) of K-step blocks
+  slab::SlabParams* layout = nullptr;  // geometry and shared-memory plan (the launch's other fields are zero)
   int clusters = -1, clusters_smem = 0;  // co-resident clusters of the kernel at that shared-memory size
 };
 
