@@ -126,7 +126,8 @@ struct SlabParams {
   int nacc;            // TMEM accumulators, acc_cols columns apart
   uint32_t acc_cols;
   int ncv, tw;         // converter teams at work (at most NS: a team that took slab g waits for the place of slab
-                       // g + ncv by a parity, which tells only neighbouring phases apart), warps of a team
+                       // g + ncv by a parity, which tells only neighbouring phases apart; P 3's stages are
+                       // freed in order, by commits a stage's MMAs apart, P 1, 2: freed_bar), warps of a team
   uint32_t lbo_a, a_part, a_bytes, stage, step_bytes;  // a stage: A (a_bytes: P parts of two core columns), then B;
                                                        // P 1, 2: an A slot
   uint32_t off_b, b_slot;  // P 1, 2: the basis ring

@@ -1,6 +1,8 @@
 // Host check of the slab kernel's shared-memory plans and ring waits, from the
 // planner's and the kernel's own code (no GPU), over every frame length, hop and
-// bin count that the forms of one and two parts accept.  Converter teams take
+// bin count that the forms of one and two parts accept.  (Of the three-part form,
+// whose stages are freed in order, only the rule that there are no more teams than
+// stages is checked, over every hop and every 20th length.)  Converter teams take
 // slabs in turn, so a team sees only some of the completions of a slot's
 // barriers, and a parity wait cannot tell a phase from the one two before it.
 // The check replays every wait of a team against every count of completions that
@@ -83,6 +85,25 @@ int main() {
             std::printf("parts %d, %d / %d / %d: %u bytes of shared memory\n", parts, n_fft, hop, mels, smem_bytes(p, 0));
           if (s >= 0 && bad++ < 20)
             std::printf("parts %d, %d / %d / %d: %d teams, %d slots, slab %d\n", parts, n_fft, hop, mels, p.ncv, p.NS, s);
+        }
+  for (int n_fft = 16; n_fft <= 4096; n_fft += n_fft < 256 ? 4 : 20)
+    for (int hop = 4; hop <= n_fft; hop += 4)
+      for (int mels : {1, 17, 80, 81, 128})
+        for (int mfcc : {0, 13}) {
+          if (mfcc > mels) continue;
+          SlabBasis sb;
+          sb.parts = 3;
+          sb.n_fft = n_fft;
+          sb.hop = hop;
+          sb.n_mels = mels;
+          sb.J = (n_fft + hop - 1) / hop;
+          sb.n_slab = (hop + 15) / 16;
+          sb.groups = (mels + 15) / 16 * 2;
+          SlabParams p;
+          std::memset(&p, 0, sizeof(p));
+          const bool ok = plan(&sb, mfcc, p);
+          ++plans;
+          if (!ok || p.ncv < 1 || p.ncv > p.NS || smem_bytes(p, mfcc) > 227u * 1024u) ++bad;
         }
   std::printf("plans %ld bad %ld\n", plans, bad);
   return plans > 0 && bad == 0 ? 0 : 1;
